@@ -204,6 +204,31 @@ static jdft_status build_twiddles(jdft_basis_s* b) {
             t32.push_back(make_float2((float)w.x, (float)w.y));
         }
     }
+    // fixed-point tables of the same lengths: w = hi 2^-30 + lo 2^-62 per component
+    for (int d = 0; d < 3; ++d) {
+        const int n = b->S[d];
+        int found = -1;
+        for (int e = 0; e < d; ++e)
+            if (b->S[e] == n) found = e;
+        if (found >= 0) { b->plan[d].fx_offset = b->plan[found].fx_offset; continue; }
+        b->plan[d].fx_offset = (int)t64.size();
+        for (int e = 0; e < n; ++e) {
+            const long double a = 2.0L * 3.14159265358979323846264338327950288L * (long double)e / (long double)n;
+            const long double z[2] = {std::cos(a), std::sin(a)};
+            int32_t w[4];
+            for (int c = 0; c < 2; ++c) {
+                const long long q = std::llround(std::ldexp(z[c], 62));
+                const long long h = (q + (1ll << 31)) >> 32;
+                const long long l = q - h * (1ll << 32);
+                w[2 * c] = (int32_t)h;
+                w[2 * c + 1] = (int32_t)std::max(l, -(1ll << 31) + 1);  // the kernels negate it
+            }
+            double2 bits;
+            static_assert(sizeof(bits) == sizeof(w), "one 16-byte entry");
+            std::memcpy(&bits, w, sizeof(w));
+            t64.push_back(bits);
+        }
+    }
     jdft_status st;
     if ((st = upload(&b->tw64, t64)) != JDFT_OK) return st;
     if ((st = upload(&b->tw32, t32)) != JDFT_OK) return st;

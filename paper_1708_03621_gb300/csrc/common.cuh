@@ -81,6 +81,7 @@ struct FftPlan {
     int npass;
     int radix[kMaxPasses];
     int tw_offset;  // offset of this length's table in the basis twiddle arrays
+    int fx_offset;  // offset of its fixed-point table (16-byte entries, fft_fix.cuh) in the FP64 twiddle array
 };
 
 // Per k-point sphere maps on the device.
@@ -143,7 +144,7 @@ struct jdft_basis_s {
     std::vector<jdft::KSphere> ks;
     // transforms
     jdft::FftPlan plan[3];
-    double2* tw64 = nullptr;  // twiddle tables, all lengths back to back
+    double2* tw64 = nullptr;  // twiddle tables, all lengths back to back, then their fixed-point tables
     float2* tw32 = nullptr;
     // local potential, permuted for the plane pass: Vp[(j2 * S1 + j1) * S0 + j0]
     double* V = nullptr;

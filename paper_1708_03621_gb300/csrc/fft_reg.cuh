@@ -11,7 +11,10 @@
 // barrier is involved.  Unnormalised: y_m = sum_t x_t exp(SIGN 2 pi i t m / N).
 #pragma once
 
+#include <type_traits>
+
 #include "fft.cuh"
+#include "fft_fix.cuh"
 
 namespace jdft {
 
@@ -68,7 +71,8 @@ __device__ __forceinline__ void dft16(c_t<T>* v) {
 
 template <typename T, int SIGN, int R>
 __device__ __forceinline__ void dft_r(c_t<T>* v) {
-    if constexpr (R == 2) dft2<T, SIGN>(v);
+    if constexpr (std::is_same<T, fix64>::value) dft_fix<SIGN, R>(v);
+    else if constexpr (R == 2) dft2<T, SIGN>(v);
     else if constexpr (R == 3) dft3<T, SIGN>(v);
     else if constexpr (R == 4) dft4<T, SIGN>(v);
     else if constexpr (R == 5) dft5<T, SIGN>(v);
@@ -101,27 +105,29 @@ struct LineShape {
 // Twiddles w[r] = W[r b], r = 1 .. R-1 (r b < N): the table is read at the
 // powers of two r = 1, 2, 4, 8 and the other w[r] are products
 // w[r] = w[r - lowbit(r)] w[lowbit(r)] (at most three roundings), which moves
-// work from the shared-memory pipe to the FMA pipe.
+// work from the shared-memory pipe to the FMA pipe.  Fixed-point twiddles are
+// all read: a product of two costs twelve wide multiplies.
 template <typename T, int R>
-__device__ __forceinline__ void stage_twiddles(c_t<T>* w, int b, const c_t<T>* __restrict__ W) {
+__device__ __forceinline__ void stage_twiddles(tw_t<T>* w, int b, const tw_t<T>* __restrict__ W) {
 #pragma unroll
     for (int r = 1; r < R; ++r) {
         const int low = r & (-r);
-        if (low == r) w[r] = W[r * b];
+        if constexpr (std::is_same<T, fix64>::value) w[r] = W[r * b];
+        else if (low == r) w[r] = W[r * b];
         else w[r] = cmul(w[r - low], w[low]);
     }
 }
 
 // One stage: v holds the inputs of this lane's butterflies, v[u*R + r].
 template <typename T, int N, int TL, int E, int SIGN, int NS, int R>
-__device__ __forceinline__ void stage_compute(c_t<T>* v, int t, const c_t<T>* __restrict__ W) {
+__device__ __forceinline__ void stage_compute(c_t<T>* v, int t, const tw_t<T>* __restrict__ W) {
     constexpr int NB = E / R;
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
         const int j = t + TL * u;
         const int k = j % NS;
         if (NS > 1 && k != 0) {
-            c_t<T> w[R];
+            tw_t<T> w[R];
             stage_twiddles<T, R>(w, k * (N / (NS * R)), W);
 #pragma unroll
             for (int r = 1; r < R; ++r) v[u * R + r] = SIGN > 0 ? cmul(v[u * R + r], w[r]) : cmulc(v[u * R + r], w[r]);
@@ -135,7 +141,7 @@ __device__ __forceinline__ void stage_compute(c_t<T>* v, int t, const c_t<T>* __
 // conjugate twiddles.  On return v[u*R + r] holds the stage's input position
 // j + r N/R (j = t + TL u).
 template <typename T, int N, int TL, int E, int SIGN2, int NS, int R>
-__device__ __forceinline__ void stage_adjoint(c_t<T>* v, int t, const c_t<T>* __restrict__ W) {
+__device__ __forceinline__ void stage_adjoint(c_t<T>* v, int t, const tw_t<T>* __restrict__ W) {
     constexpr int NB = E / R;
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
@@ -143,7 +149,7 @@ __device__ __forceinline__ void stage_adjoint(c_t<T>* v, int t, const c_t<T>* __
         const int j = t + TL * u;
         const int k = j % NS;
         if (NS > 1 && k != 0) {
-            c_t<T> w[R];
+            tw_t<T> w[R];
             stage_twiddles<T, R>(w, k * (N / (NS * R)), W);
 #pragma unroll
             for (int r = 1; r < R; ++r)
@@ -163,7 +169,7 @@ __device__ __forceinline__ int stage_out_index(int t, int u, int r) {
 template <typename T, int N, int TL, int E, int SIGN, int NS, int R, int... Rest>
 struct StageRunner {
     // Runs this stage and the rest; on return v holds the last stage's outputs.
-    static __device__ __forceinline__ void run(c_t<T>* v, int t, c_t<T>* scr, const c_t<T>* __restrict__ W) {
+    static __device__ __forceinline__ void run(c_t<T>* v, int t, c_t<T>* scr, const tw_t<T>* __restrict__ W) {
         stage_compute<T, N, TL, E, SIGN, NS, R>(v, t, W);
         if constexpr (sizeof...(Rest) > 0) {
             constexpr int R2 = RadInfo<Rest...>::prod;  // unused, keeps the pack named
@@ -198,7 +204,7 @@ struct FirstRadix {
 // stage's adjoint.
 template <typename T, int N, int TL, int E, int SIGN2, int NS, int R, int... Rest>
 struct AdjRunner {
-    static __device__ __forceinline__ void run(c_t<T>* v, int t, c_t<T>* scr, const c_t<T>* __restrict__ W) {
+    static __device__ __forceinline__ void run(c_t<T>* v, int t, c_t<T>* scr, const tw_t<T>* __restrict__ W) {
         if constexpr (sizeof...(Rest) > 0) {
             AdjRunner<T, N, TL, E, SIGN2, NS * R, Rest...>::run(v, t, scr, W);
             constexpr int Rn = FirstRadix<Rest...>::value;
@@ -241,13 +247,32 @@ struct LineFFT<T, N, E, SIGN, Rad<R0, R...>> {
     static_assert(RadInfo<R0, R...>::prod == N, "radices must multiply to N");
     static_assert(E % RadInfo<R0, R...>::lcm == 0, "E must be a multiple of every radix");
     // v[u*R0 + r] must hold input first_in(t, u, r); on return v[e] holds output out(t, e).
-    static __device__ __forceinline__ void run(c_t<T>* v, int t, c_t<T>* scr, const c_t<T>* __restrict__ W) {
-        StageRunner<T, N, TL, E, SIGN, 1, R0, R...>::run(v, t, scr, W);
+    // FP64 lines are transformed in fixed point (fft_fix.cuh): W then holds the
+    // fixed-point table (16 bytes an entry, as the FP64 one) and every lane of
+    // the warp must take part.
+    static __device__ __forceinline__ void run(c_t<T>* v, int t, c_t<T>* scr, const tw_t<T>* __restrict__ W) {
+        if constexpr (std::is_same<T, double>::value) {
+            longlong2 x[E];
+            const FixScale sc = fix_line_in<E, TL>(v, x);
+            StageRunner<fix64, N, TL, E, SIGN, 1, R0, R...>::run(x, t, reinterpret_cast<longlong2*>(scr),
+                                                                 reinterpret_cast<const int4*>(W));
+            fix_line_out<E>(x, v, sc);
+        } else {
+            StageRunner<T, N, TL, E, SIGN, 1, R0, R...>::run(v, t, scr, W);
+        }
     }
     // The transform of sign -SIGN from the layout run() leaves: v[e] must hold
     // input out(t, e); on return v[e] holds output in(t, e).
-    static __device__ __forceinline__ void run_adjoint(c_t<T>* v, int t, c_t<T>* scr, const c_t<T>* __restrict__ W) {
-        AdjRunner<T, N, TL, E, -SIGN, 1, R0, R...>::run(v, t, scr, W);
+    static __device__ __forceinline__ void run_adjoint(c_t<T>* v, int t, c_t<T>* scr, const tw_t<T>* __restrict__ W) {
+        if constexpr (std::is_same<T, double>::value) {
+            longlong2 x[E];
+            const FixScale sc = fix_line_in<E, TL>(v, x);
+            AdjRunner<fix64, N, TL, E, -SIGN, 1, R0, R...>::run(x, t, reinterpret_cast<longlong2*>(scr),
+                                                                reinterpret_cast<const int4*>(W));
+            fix_line_out<E>(x, v, sc);
+        } else {
+            AdjRunner<T, N, TL, E, -SIGN, 1, R0, R...>::run(v, t, scr, W);
+        }
     }
     static __device__ __forceinline__ int in_index(int t, int e) {
         return first_in_index<N, TL, R0>(t, e / R0, e % R0);

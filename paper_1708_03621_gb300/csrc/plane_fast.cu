@@ -18,6 +18,7 @@
 // temporaries; here the real-space box never leaves on-chip memory.)
 #include <algorithm>
 #include <cstdlib>
+#include <type_traits>
 
 #include "chain.cuh"
 #include "fft_reg.cuh"
@@ -627,6 +628,12 @@ template <> struct FastCfg<256> { static constexpr int E = 16; using R = Rad<16,
 
 constexpr size_t kFastMaxSmem = 220 * 1024;
 
+// The table the register line FFTs of type T read: the fixed-point one for FP64.
+template <typename T>
+static const c_t<T>* reg_table(const c_t<T>* tw_base, const FftPlan& p) {
+    return tw_base + (std::is_same<T, double>::value ? p.fx_offset : p.tw_offset);
+}
+
 template <int N0, int N1>
 static size_t fast_smem(const ChainGeom& g, size_t elem, int nw = kFastWarps) {
     constexpr int E0 = FastCfg<N0>::E, E1 = FastCfg<N1>::E;
@@ -661,8 +668,8 @@ static jdft_status apply_fast_impl(const ChainGeom& g, c_t<T>* colbuf, const T* 
     if (e != cudaSuccess) return set_error(JDFT_ERR_CUDA, std::string("plane_apply_fast: ") + cudaGetErrorString(e));
     {
         Trace tr_("plane_apply_fast", st);
-        kern<<<dim3(g.S2, nb), kFastThreads, smem, st>>>(g, colbuf, Vp, tw_base + g.p0.tw_offset,
-                                                         tw_base + g.p1.tw_offset);
+        kern<<<dim3(g.S2, nb), kFastThreads, smem, st>>>(g, colbuf, Vp, reg_table<T>(tw_base, g.p0),
+                                                         reg_table<T>(tw_base, g.p1));
     }
     return check_launch("plane_apply_fast");
 }
@@ -713,7 +720,8 @@ static jdft_status zinv_fast_impl(const ChainGeom& g, const c_t<T>* C, int ldc, 
     if (e != cudaSuccess) return set_error(JDFT_ERR_CUDA, std::string("zpass_inverse_fast: ") + cudaGetErrorString(e));
     {
         Trace tr_("zpass_inverse", st);
-        kern<<<dim3(zpass_fast_blocks<N2>(g), nb), kZThreads, smem, st>>>(g, C, ldc, colbuf, tw2);
+        kern<<<dim3(zpass_fast_blocks<N2>(g), nb), kZThreads, smem, st>>>(g, C, ldc, colbuf,
+                                                                          reg_table<T>(tw2 - g.p2.tw_offset, g.p2));
     }
     return check_launch("zpass_inverse_fast");
 }
@@ -730,7 +738,8 @@ static jdft_status zfwd_fast_impl(const ChainGeom& g, const c_t<T>* colbuf, cons
     {
         Trace tr_("zpass_forward", st);
         kern<<<dim3(zpass_fast_blocks<N2>(g), nb), kZThreads, smem, st>>>(g, colbuf, C, ldc, out, ldo, kin, omega,
-                                                                            scale, tw2);
+                                                                            scale,
+                                                                            reg_table<T>(tw2 - g.p2.tw_offset, g.p2));
     }
     return check_launch("zpass_forward_fast");
 }
