@@ -697,8 +697,8 @@ jdft_status jdft_profile_read(char* buf, int buflen);
  * clear the record.  JDFT_OK otherwise. */
 jdft_status jdft_device_status(void* stream);
 
-/* Limit, in seconds, of each device-side wait of the tensor-core products on
- * the current device (default 2 s; kernels launched after the call use it).
+/* Limit, in seconds, of each device-side wait of the tensor-core products
+ * (large FP64 products run on the tensor cores too) on the current device (default 2 s; kernels launched after the call use it).
  * A wait that runs out records JDFT_ERR_TIMEOUT for jdft_device_status, stops
  * issuing products, waits (under a fixed 2 s limit of its own) for the products
  * it already committed, and frees its tensor memory; the product's output is

@@ -58,6 +58,30 @@ jdft_status ensure_ws(Workspace& w, size_t bytes) {
     return JDFT_OK;
 }
 
+void* ProductScratch::get(size_t need) {
+    if (bytes >= need) return ptr;
+    // half again, so that the blocks outgrown stay few; the plain size where that much is not left
+    for (const size_t want : {std::max(need, bytes + bytes / 2), need}) {
+        void* p = nullptr;
+        if (cudaMalloc(&p, want) == cudaSuccess) {
+            if (ptr) retired.push_back(ptr);
+            ptr = p;
+            bytes = want;
+            return ptr;
+        }
+        cudaGetLastError();
+    }
+    return nullptr;
+}
+
+void ProductScratch::release() {
+    cudaFree(ptr);
+    for (void* p : retired) cudaFree(p);
+    retired.clear();
+    ptr = nullptr;
+    bytes = 0;
+}
+
 jdft_status ensure_workspace(jdft_basis_s* b, size_t bytes) { return ensure_ws(b->work, bytes); }
 
 // Radices for a length n = 2^a 3^b 5^c: eights first, then a four or two,
@@ -374,6 +398,7 @@ jdft_status jdft_basis_destroy(jdft_basis_t b) {
     cudaSetDevice(b->device);
     for (auto& s : b->ks) free_sphere(s);
     cudaFree(b->tw64); cudaFree(b->tw32); cudaFree(b->V); cudaFree(b->V32); cudaFree(b->work.ptr);
+    b->prodwork.release();
     if (b->side) {
         cudaStreamSynchronize(b->side);
         cudaStreamDestroy(b->side);

@@ -612,7 +612,7 @@ static jdft_status run_apply_H(jdft_basis_s* b, int ik, const void* C, int ldc, 
     }
     if (sp.nproj > 0)
         return nonlocal_accumulate<T>(sp, C, ldc, HC, ldhc, nb, prec, (char*)b->work.ptr + colbytes, st, true, nullptr,
-                                      true);
+                                      true, &b->prodwork);
     return JDFT_OK;
 }
 
@@ -669,7 +669,7 @@ static jdft_status run_apply_H_density(jdft_basis_s* b, int ik, const void* C, i
     }
     if (sp.nproj > 0)
         return nonlocal_accumulate<T>(sp, C, ldc, HC, ldhc, nb, prec, (char*)b->work.ptr + colbytes, st, !Csplit,
-                                      Csplit, true);
+                                      Csplit, true, &b->prodwork);
     return JDFT_OK;
 }
 

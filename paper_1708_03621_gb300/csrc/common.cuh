@@ -129,6 +129,18 @@ struct Workspace {
     size_t bytes = 0;
 };
 
+// Scratch of the sliced FP64 products.  It grows by at least half again and keeps the
+// blocks it has outgrown until the basis goes (their sizes add up to less than
+// twice the last one), so that a captured graph that holds a pointer to one
+// stays valid.  get() returns nullptr when the device has no room.
+struct ProductScratch {
+    void* ptr = nullptr;
+    size_t bytes = 0;
+    std::vector<void*> retired;
+    void* get(size_t need);
+    void release();
+};
+
 }  // namespace jdft
 
 struct jdft_basis_s {
@@ -162,6 +174,7 @@ struct jdft_basis_s {
     // full-box field transforms (Hartree, Kohn-Sham potential): a complex FP64
     // box and per-block partial sums (grown on first use)
     jdft::Workspace fieldwork;
+    jdft::ProductScratch prodwork;
     // spinor calls: real-space boxes and sphere blocks of a band chunk
     jdft::Workspace spinwork;
     cudaStream_t side = nullptr;

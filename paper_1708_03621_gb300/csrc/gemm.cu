@@ -202,7 +202,7 @@ template <> const float2* proj_ptr<float>(const KSphere& sp) { return (const flo
 template <typename T>
 jdft_status nonlocal_accumulate(const KSphere& sp, const void* C, int ldc, void* HC, int ldhc, int nb,
                                 jdft_prec prec, void* work, cudaStream_t st, bool split_c, const void* Csplit,
-                                bool partials) {
+                                bool partials, ProductScratch* scratch) {
     if (sp.nproj == 0 || nb == 0) return JDFT_OK;
     double2* Bc = (double2*)work;
     const size_t abytes = ((size_t)sp.nproj * nb * sizeof(double2) + 255) / 256 * 256;
@@ -226,7 +226,8 @@ jdft_status nonlocal_accumulate(const KSphere& sp, const void* C, int ldc, void*
         s = tcx_cn(sp.nproj, nb, sp.npw, sp.Psplit, Cs, Bc, nb, 1.0, st, part,
                    partials ? tcx_cn_partial_bytes(sp.nproj, nb, sp.npw) : 0);
     } else {
-        s = gemm_cn<T>(prec, sp.nproj, nb, sp.npw, proj_ptr<T>(sp), sp.npw, (const c_t<T>*)C, ldc, Bc, nb, 1.0, st);
+        s = gemm_cn<T>(prec, sp.nproj, nb, sp.npw, proj_ptr<T>(sp), sp.npw, (const c_t<T>*)C, ldc, Bc, nb, 1.0, st,
+                       scratch);
     }
     if (s != JDFT_OK) return s;
     {
@@ -241,29 +242,37 @@ jdft_status nonlocal_accumulate(const KSphere& sp, const void* C, int ldc, void*
         if ((s = tcx_split_t((const float2*)Bd, nb, nb, sp.nproj, Bt, st))) return s;
         return tcx_nn(sp.npw, nb, sp.nproj, sp.Psplit_t, Bt, (float2*)HC, ldhc, true, st);
     }
-    return gemm_nn_acc<T>(prec, sp.npw, nb, sp.nproj, proj_ptr<T>(sp), sp.npw, Bd, nb, (c_t<T>*)HC, ldhc, st);
+    return gemm_nn_acc<T>(prec, sp.npw, nb, sp.nproj, proj_ptr<T>(sp), sp.npw, Bd, nb, (c_t<T>*)HC, ldhc, st, true, scratch);
 }
 
 template <>
 jdft_status gemm_cn<double>(jdft_prec, int M, int N, int K, const double2* A, int lda, const double2* B, int ldb,
-                            double2* out, int ldo, double alpha, cudaStream_t st) {
+                            double2* out, int ldo, double alpha, cudaStream_t st, ProductScratch* scratch) {
+    if (scratch && sl_eligible(M, N, K)) {
+        const jdft_status s = sl_zgemm_cn(M, N, K, A, lda, B, ldb, out, ldo, alpha, *scratch, st);
+        if (s != JDFT_ERR_UNSUPPORTED) return s;
+    }
     return zgemm_cn<double>(M, N, K, A, lda, B, ldb, out, ldo, alpha, st);
 }
 template <>
 jdft_status gemm_cn<float>(jdft_prec prec, int M, int N, int K, const float2* A, int lda, const float2* B, int ldb,
-                           double2* out, int ldo, double alpha, cudaStream_t st) {
+                           double2* out, int ldo, double alpha, cudaStream_t st, ProductScratch*) {
     if (prec == JDFT_TF32X3 || prec == JDFT_BF16X3)
         return tc_zgemm_cn(M, N, K, A, lda, B, ldb, out, ldo, alpha, prec == JDFT_BF16X3, st);
     return zgemm_cn<float>(M, N, K, A, lda, B, ldb, out, ldo, alpha, st);
 }
 template <>
 jdft_status gemm_nn_acc<double>(jdft_prec, int M, int N, int K, const double2* A, int lda, const double2* Bm, int ldb,
-                                double2* out, int ldo, cudaStream_t st, bool accumulate) {
+                                double2* out, int ldo, cudaStream_t st, bool accumulate, ProductScratch* scratch) {
+    if (scratch && sl_eligible(M, N, K)) {
+        const jdft_status s = sl_zgemm_nn(M, N, K, A, lda, Bm, ldb, out, ldo, accumulate, *scratch, st);
+        if (s != JDFT_ERR_UNSUPPORTED) return s;
+    }
     return zgemm_nn_acc<double>(M, N, K, A, lda, Bm, ldb, out, ldo, st, accumulate);
 }
 template <>
 jdft_status gemm_nn_acc<float>(jdft_prec prec, int M, int N, int K, const float2* A, int lda, const float2* Bm, int ldb,
-                               float2* out, int ldo, cudaStream_t st, bool accumulate) {
+                               float2* out, int ldo, cudaStream_t st, bool accumulate, ProductScratch*) {
     if (prec == JDFT_TF32X3 || prec == JDFT_BF16X3)
         return tc_zgemm_nn_acc(M, N, K, A, lda, Bm, ldb, out, ldo, prec == JDFT_BF16X3, st, accumulate);
     return zgemm_nn_acc<float>(M, N, K, A, lda, Bm, ldb, out, ldo, st, accumulate);
@@ -278,9 +287,9 @@ template jdft_status zgemm_nn_acc<double>(int, int, int, const double2*, int, co
 template jdft_status zgemm_nn_acc<float>(int, int, int, const float2*, int, const float2*, int, float2*, int,
                                          cudaStream_t, bool);
 template jdft_status nonlocal_accumulate<double>(const KSphere&, const void*, int, void*, int, int, jdft_prec, void*,
-                                                 cudaStream_t, bool, const void*, bool);
+                                                 cudaStream_t, bool, const void*, bool, ProductScratch*);
 template jdft_status nonlocal_accumulate<float>(const KSphere&, const void*, int, void*, int, int, jdft_prec, void*,
-                                                cudaStream_t, bool, const void*, bool);
+                                                cudaStream_t, bool, const void*, bool, ProductScratch*);
 
 }  // namespace jdft
 
@@ -325,8 +334,8 @@ extern "C" jdft_status jdft_subspace(jdft_basis_t b, int ik, const void* C, int 
     if (CHC) {
         JDFT_CUDA_TRY(cudaMemsetAsync(CHC, 0, (size_t)nb * nb * sizeof(double2), st));
         s = (prec == JDFT_FP64)
-                ? zgemm_cn<double>(nb, nb, npw, (const double2*)C, ldc, (const double2*)HC, ldhc, (double2*)CHC, nb,
-                                   1.0, st)
+                ? gemm_cn<double>(prec, nb, nb, npw, (const double2*)C, ldc, (const double2*)HC, ldhc, (double2*)CHC,
+                                  nb, 1.0, st, &b->prodwork)
                 : gemm_cn<float>(prec, nb, nb, npw, (const float2*)C, ldc, (const float2*)HC, ldhc, (double2*)CHC, nb, 1.0,
                                   st);
         if (s != JDFT_OK) return s;
@@ -334,8 +343,8 @@ extern "C" jdft_status jdft_subspace(jdft_basis_t b, int ik, const void* C, int 
     if (COC) {
         JDFT_CUDA_TRY(cudaMemsetAsync(COC, 0, (size_t)nb * nb * sizeof(double2), st));
         s = (prec == JDFT_FP64)
-                ? zgemm_cn<double>(nb, nb, npw, (const double2*)C, ldc, (const double2*)C, ldc, (double2*)COC, nb,
-                                   b->omega, st)
+                ? gemm_cn<double>(prec, nb, nb, npw, (const double2*)C, ldc, (const double2*)C, ldc, (double2*)COC, nb,
+                                  b->omega, st, &b->prodwork)
                 : gemm_cn<float>(prec, nb, nb, npw, (const float2*)C, ldc, (const float2*)C, ldc, (double2*)COC, nb,
                                   b->omega, st);
     }

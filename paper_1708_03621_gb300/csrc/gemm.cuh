@@ -57,14 +57,25 @@ size_t tcx_cn_partial_bytes(int M, int N, int K);
 jdft_status tcx_cn(int M, int N, int K, const void* Aplanes, const void* Bplanes, double2* out, int ldo, double alpha,
                    cudaStream_t st, void* partials = nullptr, size_t partial_bytes = 0, bool hermitian = false);
 
+// FP64 products from 7-bit slices on the tensor cores (tc_slices.cuh), with their
+// scratch; JDFT_ERR_UNSUPPORTED, with nothing launched, when the device has no
+// room for it.  sl_eligible: whether they are faster than the CUDA-core products.
+bool sl_eligible(int M, int N, int K);
+jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* out,
+                        int ldo, double scale, ProductScratch& scratch, cudaStream_t st);
+jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const double2* Bm, int ldb, double2* out,
+                        int ldo, bool accumulate, ProductScratch& scratch, cudaStream_t st);
+
 // Precision dispatch: JDFT_TF32X3 and JDFT_BF16X3 run the tensor-core
-// versions (T = float only), the other precisions the CUDA-core ones.
+// versions (T = float only), the other precisions the CUDA-core ones; FP64
+// products large enough run from slices when the caller has scratch for them.
 template <typename T>
 jdft_status gemm_cn(jdft_prec prec, int M, int N, int K, const c_t<T>* A, int lda, const c_t<T>* B, int ldb,
-                    double2* out, int ldo, double alpha, cudaStream_t st);
+                    double2* out, int ldo, double alpha, cudaStream_t st, ProductScratch* scratch = nullptr);
 template <typename T>
 jdft_status gemm_nn_acc(jdft_prec prec, int M, int N, int K, const c_t<T>* A, int lda, const c_t<T>* Bm, int ldb,
-                        c_t<T>* out, int ldo, cudaStream_t st, bool accumulate = true);
+                        c_t<T>* out, int ldo, cudaStream_t st, bool accumulate = true,
+                        ProductScratch* scratch = nullptr);
 
 // Whether gemm_nn_acc(prec, M, N, K, A, ...) may write its output over A
 // (out == A, same leading dimension, K == N): true when one block computes
@@ -87,9 +98,11 @@ size_t nonlocal_workspace_bytes(int nproj, int nb, size_t elem, int npw = 0, jdf
 // of its own when the projection is eligible.
 // partials: the workspace holds nonlocal_workspace_bytes(..., split_c, true)
 // and the projection's split-K partial tiles go there (no atomics).
+// scratch: for the sliced FP64 products.
 template <typename T>
 jdft_status nonlocal_accumulate(const KSphere& sp, const void* C, int ldc, void* HC, int ldhc, int nb,
                                 jdft_prec prec, void* work, cudaStream_t st, bool split_c = false,
-                                const void* Csplit = nullptr, bool partials = false);
+                                const void* Csplit = nullptr, bool partials = false,
+                                ProductScratch* scratch = nullptr);
 
 }  // namespace jdft

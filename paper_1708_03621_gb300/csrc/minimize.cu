@@ -494,7 +494,7 @@ struct MinState {
             if (s != JDFT_OK) return s;
             return tcx_cn(nb, nb, npw, sp1, Yb != X ? sp2 : sp1, out, nb, alpha, st, spp, spp_bytes, Yb == X);
         }
-        return gemm_cn<T>(prec, nb, nb, npw, X, ld, Yb, ld, out, nb, alpha, st);
+        return gemm_cn<T>(prec, nb, nb, npw, X, ld, Yb, ld, out, nb, alpha, st, &b->prodwork);
     }
     // Z (+)= X . S for a small block-type S, from split operands
     jdft_status tcx_times(const c_t<T>* X, const c_t<T>* S, c_t<T>* Z, bool accumulate) {
@@ -512,12 +512,12 @@ struct MinState {
         jdft_status s = check_launch("small_scale");
         if (s != JDFT_OK) return s;
         if (tcx) return tcx_times(X, Bm, Z, true);
-        return gemm_nn_acc<T>(prec, npw, nb, nb, X, ld, Bm, nb, Z, ld, st);
+        return gemm_nn_acc<T>(prec, npw, nb, nb, X, ld, Bm, nb, Z, ld, st, true, &b->prodwork);
     }
     // Z = X . W  (W already in block type)
     jdft_status rotate(const c_t<T>* X, c_t<T>* Z) {
         if (tcx) return tcx_times(X, W, Z, false);
-        return gemm_nn_acc<T>(prec, npw, nb, nb, X, ld, W, nb, Z, ld, st, false);
+        return gemm_nn_acc<T>(prec, npw, nb, nb, X, ld, W, nb, Z, ld, st, false, &b->prodwork);
     }
     jdft_status hermitize(double2* A, double* tr) {
         {
@@ -773,18 +773,20 @@ static jdft_status orthonormalize_impl(jdft_basis_s* b, int ik, void* C, int ldc
             if ((s = tcx_cn(nb, nb, npw, planes, planes, U, nb, b->omega, st, (char*)planes + spl, pb, true)))
                 return s;
         } else if ((s = gemm_cn<T>(prec, nb, nb, npw, (const c_t<T>*)C, ldc, (const c_t<T>*)C, ldc, U, nb, b->omega,
-                                   st))) {
+                                   st, &b->prodwork))) {
             return s;
         }
     }
     if ((s = small_cholesky_winv(nb, U, work, W, std::is_same<T, double>::value, status, st))) return s;
     if (gemm_nn_inplace_ok(prec, nb)) {
         // C <- C W in place: each block reads its rows of C for every band before writing them
-        if ((s = gemm_nn_acc<T>(prec, npw, nb, nb, (const c_t<T>*)C, ldc, W, nb, (c_t<T>*)C, ldc, st, false)))
+        if ((s = gemm_nn_acc<T>(prec, npw, nb, nb, (const c_t<T>*)C, ldc, W, nb, (c_t<T>*)C, ldc, st, false, &b->prodwork)))
             return s;
     } else {
         JDFT_CUDA_TRY(cudaMemcpyAsync(tmp, C, (size_t)nb * ldc * sizeof(c_t<T>), cudaMemcpyDeviceToDevice, st));
-        if ((s = gemm_nn_acc<T>(prec, npw, nb, nb, tmp, ldc, W, nb, (c_t<T>*)C, ldc, st, false))) return s;
+        if ((s = gemm_nn_acc<T>(prec, npw, nb, nb, tmp, ldc, W, nb, (c_t<T>*)C, ldc, st, false,
+                                &b->prodwork)))
+            return s;
     }
     if (sticky) {
         {
@@ -871,7 +873,7 @@ static jdft_status hamiltonian_step_impl(jdft_basis_s* b, int ik, void* C, int l
     if (split) {
         if ((s = tcx_split((const float2*)C, ldc, nb, npw, Cs, st))) return s;
         if ((s = tcx_cn(nb, nb, npw, Cs, Cs, COC, nb, b->omega, st, part, pb, true))) return s;
-    } else if ((s = gemm_cn<T>(prec, nb, nb, npw, Cc, ldc, Cc, ldc, COC, nb, b->omega, st))) {
+    } else if ((s = gemm_cn<T>(prec, nb, nb, npw, Cc, ldc, Cc, ldc, COC, nb, b->omega, st, &b->prodwork))) {
         return s;
     }
     c_t<T>* W = nullptr;
@@ -891,7 +893,8 @@ static jdft_status hamiltonian_step_impl(jdft_basis_s* b, int ik, void* C, int l
         if ((s = tcx_split((const float2*)HC, ldhc, nb, npw, HCs, st))) return s;
         // H C is this step's own H C, so C^dag H C is Hermitian up to rounding
         if ((s = tcx_cn(nb, nb, npw, Cs, HCs, CHC, nb, 1.0, st, part, pb, true))) return s;
-    } else if ((s = gemm_cn<T>(prec, nb, nb, npw, Cc, ldc, (const c_t<T>*)HC, ldhc, CHC, nb, 1.0, st))) {
+    } else if ((s = gemm_cn<T>(prec, nb, nb, npw, Cc, ldc, (const c_t<T>*)HC, ldhc, CHC, nb, 1.0, st,
+                               &b->prodwork))) {
         return s;
     }
     if (!ortho) return JDFT_OK;
@@ -905,10 +908,11 @@ static jdft_status hamiltonian_step_impl(jdft_basis_s* b, int ik, void* C, int l
         if ((s = tcx_split_t((const float2*)W, nb, nb, nb, Wt, st))) return s;
         return tcx_nn(npw, nb, nb, Ct, Wt, (float2*)C, ldc, false, st);
     }
-    if (inplace) return gemm_nn_acc<T>(prec, npw, nb, nb, Cc, ldc, W, nb, (c_t<T>*)C, ldc, st, false);
+    if (inplace)
+        return gemm_nn_acc<T>(prec, npw, nb, nb, Cc, ldc, W, nb, (c_t<T>*)C, ldc, st, false, &b->prodwork);
     c_t<T>* tmp = (c_t<T>*)ws;
     JDFT_CUDA_TRY(cudaMemcpyAsync(tmp, C, (size_t)nb * ldc * sizeof(c_t<T>), cudaMemcpyDeviceToDevice, st));
-    return gemm_nn_acc<T>(prec, npw, nb, nb, tmp, ldc, W, nb, (c_t<T>*)C, ldc, st, false);
+    return gemm_nn_acc<T>(prec, npw, nb, nb, tmp, ldc, W, nb, (c_t<T>*)C, ldc, st, false, &b->prodwork);
 }
 }  // namespace jdft
 

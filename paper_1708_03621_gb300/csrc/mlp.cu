@@ -657,7 +657,7 @@ jdft_status jdft_mlp_rows(jdft_basis_t b, int ik, const void* C, const void* Cst
     if ((s = jdft_apply_H(b, ik, Cd, npw, HC, npw, nb, JDFT_FP64, stream))) return done(s);
     if (cudaMemsetAsync(Hs, 0, (size_t)nb * nb * sizeof(double2), st) != cudaSuccess)
         return done(set_error(JDFT_ERR_CUDA, "memset"));
-    if ((s = zgemm_cn<double>(nb, nb, npw, Cd, npw, HC, npw, Hs, nb, 1.0, st))) return done(s);
+    if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, Cd, npw, HC, npw, Hs, nb, 1.0, st, &b->prodwork))) return done(s);
     if (cudaMemcpyAsync(G, HC, blk, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         return done(set_error(JDFT_ERR_CUDA, "copy"));
     {
@@ -665,14 +665,14 @@ jdft_status jdft_mlp_rows(jdft_basis_t b, int ik, const void* C, const void* Cst
         rows_scale_kernel<<<grid_rows((int64_t)nb * nb, 256), 256, 0, st>>>(nb * nb, Hs, -b->omega, Bm);
     }
     if ((s = check_launch("rows_scale"))) return done(s);
-    if ((s = zgemm_nn_acc<double>(npw, nb, nb, Cd, npw, Bm, nb, G, npw, st))) return done(s);
+    if ((s = gemm_nn_acc<double>(JDFT_FP64, npw, nb, nb, Cd, npw, Bm, nb, G, npw, st, true, &b->prodwork))) return done(s);
     // target t = C - C* (Omega C*^dag C)
     if (cudaMemsetAsync(M, 0, (size_t)nb * nb * sizeof(double2), st) != cudaSuccess)
         return done(set_error(JDFT_ERR_CUDA, "memset"));
-    if ((s = zgemm_cn<double>(nb, nb, npw, Cs, npw, Cd, npw, M, nb, -b->omega, st))) return done(s);
+    if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, Cs, npw, Cd, npw, M, nb, -b->omega, st, &b->prodwork))) return done(s);
     if (cudaMemcpyAsync(Tt, Cd, blk, cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         return done(set_error(JDFT_ERR_CUDA, "copy"));
-    if ((s = zgemm_nn_acc<double>(npw, nb, nb, Cs, npw, M, nb, Tt, npw, st))) return done(s);
+    if ((s = gemm_nn_acc<double>(JDFT_FP64, npw, nb, nb, Cs, npw, M, nb, Tt, npw, st, true, &b->prodwork))) return done(s);
     // features
     {
         Trace tr_("mlp_rows_band_kinetic", st);

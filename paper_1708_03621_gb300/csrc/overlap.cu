@@ -59,7 +59,8 @@ jdft_status run_op_S(jdft_basis_s* b, int ik, const void* C, int ldc, void* SC, 
     aug.Dval = sp.Qval;
     if ((s = ensure_workspace(b, nonlocal_workspace_bytes(sp.nproj, nb, sizeof(c_t<T>), sp.npw, prec, false, false))))
         return s;
-    s = nonlocal_accumulate<T>(aug, C, ldc, SC, ldsc, nb, prec, b->work.ptr, st);
+    s = nonlocal_accumulate<T>(aug, C, ldc, SC, ldsc, nb, prec, b->work.ptr, st, false, nullptr, false,
+                               &b->prodwork);
     aug.iG.clear();
     return s;
 }
@@ -215,10 +216,10 @@ struct GenMin {
 
     jdft_status cn(const double2* A, const double2* Bm, double2* out) {   // out = A^dag B (nb x nb)
         JDFT_CUDA_TRY(cudaMemsetAsync(out, 0, (size_t)nb * nb * sizeof(double2), st));
-        return gemm_cn<double>(JDFT_FP64, nb, nb, npw, A, npw, Bm, npw, out, nb, 1.0, st);
+        return gemm_cn<double>(JDFT_FP64, nb, nb, npw, A, npw, Bm, npw, out, nb, 1.0, st, &b->prodwork);
     }
     jdft_status nn_acc(const double2* A, const double2* Mm, double2* out) {   // out += A Mm
-        return gemm_nn_acc<double>(JDFT_FP64, npw, nb, nb, A, npw, Mm, nb, out, npw, st, true);
+        return gemm_nn_acc<double>(JDFT_FP64, npw, nb, nb, A, npw, Mm, nb, out, npw, st, true, &b->prodwork);
     }
     jdft_status neg(const double2* A, double2* out) {
         {
@@ -371,9 +372,10 @@ jdft_status jdft_subspace_generalized(jdft_basis_t b, int ik, const void* C, int
         cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess)
         return done(set_error(JDFT_ERR_CUDA, "jdft_subspace_generalized: memset"));
     if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, (const double2*)C, ldc, (const double2*)HC, ldhc,
-                             (double2*)CHC, nb, 1.0, st)))
+                             (double2*)CHC, nb, 1.0, st, &b->prodwork)))
         return done(s);
-    if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, (const double2*)C, ldc, SCb, npw, (double2*)CSC, nb, 1.0, st)))
+    if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, (const double2*)C, ldc, SCb, npw, (double2*)CSC, nb, 1.0, st,
+                             &b->prodwork)))
         return done(s);
     if (eigs) {
         // C' = C L^{-dag}, (HC)' = HC L^{-dag} with C^dag S C = L L^dag; eigenvalues of C'^dag (HC)'
@@ -384,7 +386,8 @@ jdft_status jdft_subspace_generalized(jdft_basis_t b, int ik, const void* C, int
             return done(set_error(JDFT_ERR_CUDA, "jdft_subspace_generalized: copies"));
         if ((s = jdft_orthonormalize_async(b, ik, Cc, npw, nb, CSC, JDFT_FP64, status, stream))) return done(s);
         if ((s = jdft_orthonormalize_async(b, ik, Hc, npw, nb, CSC, JDFT_FP64, status, stream))) return done(s);
-        if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, Cc, npw, Hc, npw, A, nb, 1.0, st))) return done(s);
+        if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, Cc, npw, Hc, npw, A, nb, 1.0, st, &b->prodwork)))
+            return done(s);
         int hs = 0;
         if (cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             cudaStreamSynchronize(st) != cudaSuccess)
@@ -416,7 +419,7 @@ jdft_status jdft_orthonormalize_generalized(jdft_basis_t b, int ik, void* C, int
     if (cudaMemsetAsync(U, 0, (size_t)nb * nb * sizeof(double2), st) != cudaSuccess ||
         cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess)
         return done(set_error(JDFT_ERR_CUDA, "jdft_orthonormalize_generalized: memset"));
-    if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, (const double2*)C, ldc, SCb, npw, U, nb, 1.0, st)))
+    if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, (const double2*)C, ldc, SCb, npw, U, nb, 1.0, st, &b->prodwork)))
         return done(s);
     if ((s = jdft_orthonormalize_async(b, ik, C, ldc, nb, U, JDFT_FP64, status, stream))) return done(s);
     int hs = 0;

@@ -38,6 +38,7 @@
 #include "minimize.cuh"
 #include "profile.cuh"
 #include "tc_ptx.cuh"
+#include "fft_fix.cuh"
 
 namespace jdft {
 
@@ -1594,3 +1595,5 @@ extern "C" jdft_status jdft_autotune_gemm(int M, int N, int K, const void* A, in
     if (splits) *splits = best_c;
     return JDFT_OK;
 }
+
+#include "tc_slices.cuh"
