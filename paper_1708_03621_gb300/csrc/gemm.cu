@@ -13,43 +13,65 @@
 namespace jdft {
 
 // ---------------------------------------------------------------------------
-// C^dag-style product with split K.  Tile 32 x 32 outputs, 16-deep K slices,
-// 256 threads, 2 x 2 outputs per thread.  Each split adds its partial sum to
-// the FP64 output with atomics.
+// C^dag-style product with split K, for the shapes whose FP64 products are too
+// small for the sliced ones and for FP32 blocks.  FP64: bound by the FP64 pipe (2
+// multiply-adds per clock and SM), so what counts is that every SM has work and
+// no lane multiplies padding.  A block of four warps holds a TM x TN tile (16 or
+// 32 each way, whichever pads less) and a range of K in chunks of 32; each warp
+// takes a quarter of a chunk's K with the whole tile in its registers (lanes
+// 8 x 4, TM/8 x TN/4 outputs each), so one shared-memory read feeds 5 to 11
+// multiply-adds.  The warps' sums meet in shared memory, the blocks' in FP64 atomics.
+// Against a 32 x 32 tile of 256 threads with 2 x 2 outputs each and at least 64
+// K to a block, 16 x 16 over 4 259 plane waves took 142 us and takes 27 (event times).
 // ---------------------------------------------------------------------------
-constexpr int CN_BM = 32, CN_BN = 32, CN_BK = 16;
+constexpr int CN_BK = 32, CN_WARPS = 4;
 
-template <typename T>
-__global__ void __launch_bounds__(256) zgemm_cn_kernel(int M, int N, int K, int kchunk, const c_t<T>* __restrict__ A,
-                                                       int lda, const c_t<T>* __restrict__ B, int ldb,
-                                                       double2* __restrict__ out, int ldo, double scale) {
-    __shared__ c_t<T> As[CN_BK][CN_BM + 1];
-    __shared__ c_t<T> Bs[CN_BK][CN_BN + 1];
-    const int m0 = blockIdx.x * CN_BM, n0 = blockIdx.y * CN_BN;
+template <typename T, int TM, int TN>
+__global__ void __launch_bounds__(32 * CN_WARPS)
+    zgemm_cn_kernel(int M, int N, int K, int kchunk, const c_t<T>* __restrict__ A, int lda,
+                    const c_t<T>* __restrict__ B, int ldb, double2* __restrict__ out, int ldo, double scale) {
+    constexpr int PM = TM / 8, PN = TN / 4, THREADS = 32 * CN_WARPS;
+    constexpr int STAGE = CN_BK * (TM + 1 + TN + 1);
+    constexpr int ELEMS = STAGE > CN_WARPS * TM * TN ? STAGE : CN_WARPS * TM * TN;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    c_t<T>* As = reinterpret_cast<c_t<T>*>(smem_raw);  // [CN_BK][TM + 1]
+    c_t<T>* Bs = As + CN_BK * (TM + 1);                // [CN_BK][TN + 1]
+    static_assert(ELEMS * sizeof(c_t<T>) <= 64 * 1024, "shared memory of a block");
+    const int m0 = blockIdx.x * TM, n0 = blockIdx.y * TN;
     const int kA = blockIdx.z * kchunk, kB = min(K, kA + kchunk);
-    const int tm = threadIdx.x / 16, tn = threadIdx.x % 16;
-    c_t<T> acc[2][2];
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int lm = lane >> 2, ln = lane & 3;
+    c_t<T> acc[PM][PN];
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < PM; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) acc[i][j] = mk<T>(T(0), T(0));
+        for (int j = 0; j < PN; ++j) acc[i][j] = mk<T>(T(0), T(0));
     for (int k0 = kA; k0 < kB; k0 += CN_BK) {
-        for (int e = threadIdx.x; e < CN_BM * CN_BK; e += 256) {
-            const int r = e / CN_BK, kk = e % CN_BK;
-            const int m = m0 + r, k = k0 + kk;
-            As[kk][r] = (m < M && k < kB) ? A[(size_t)m * lda + k] : mk<T>(T(0), T(0));
-            const int n = n0 + r;
-            Bs[kk][r] = (n < N && k < kB) ? B[(size_t)n * ldb + k] : mk<T>(T(0), T(0));
+        // a warp reads 32 consecutive K values of one row
+        for (int e = threadIdx.x; e < (TM + TN) * CN_BK; e += THREADS) {
+            const int r = e / CN_BK, kk = e % CN_BK, k = k0 + kk;
+            c_t<T> v = mk<T>(T(0), T(0));
+            if (r < TM) {
+                if (m0 + r < M && k < kB) v = A[(size_t)(m0 + r) * lda + k];
+                As[kk * (TM + 1) + r] = v;
+            } else {
+                if (n0 + r - TM < N && k < kB) v = B[(size_t)(n0 + r - TM) * ldb + k];
+                Bs[kk * (TN + 1) + r - TM] = v;
+            }
         }
         __syncthreads();
+        const int kn = min(CN_BK, kB - k0);
+#pragma unroll 2
+        for (int kk = warp; kk < kn; kk += CN_WARPS) {
+            c_t<T> a[PM], b[PN];
 #pragma unroll
-        for (int kk = 0; kk < CN_BK; ++kk) {
-            c_t<T> a[2] = {As[kk][tm], As[kk][tm + 16]};
-            c_t<T> b[2] = {Bs[kk][tn], Bs[kk][tn + 16]};
+            for (int i = 0; i < PM; ++i) a[i] = As[kk * (TM + 1) + lm + 8 * i];
 #pragma unroll
-            for (int i = 0; i < 2; ++i)
+            for (int j = 0; j < PN; ++j) b[j] = Bs[kk * (TN + 1) + ln + 4 * j];
 #pragma unroll
-                for (int j = 0; j < 2; ++j) {
+            for (int i = 0; i < PM; ++i)
+#pragma unroll
+                for (int j = 0; j < PN; ++j) {
                     // conj(a) * b
                     acc[i][j].x += a[i].x * b[j].x + a[i].y * b[j].y;
                     acc[i][j].y += a[i].x * b[j].y - a[i].y * b[j].x;
@@ -57,83 +79,106 @@ __global__ void __launch_bounds__(256) zgemm_cn_kernel(int M, int N, int K, int 
         }
         __syncthreads();
     }
+    c_t<T>* red = As;  // [warp][m][n]
 #pragma unroll
-    for (int i = 0; i < 2; ++i)
+    for (int i = 0; i < PM; ++i)
 #pragma unroll
-        for (int j = 0; j < 2; ++j) {
-            const int m = m0 + tm + 16 * i, n = n0 + tn + 16 * j;
-            if (m < M && n < N) {
-                atomicAdd(&out[(size_t)m * ldo + n].x, scale * (double)acc[i][j].x);
-                atomicAdd(&out[(size_t)m * ldo + n].y, scale * (double)acc[i][j].y);
-            }
+        for (int j = 0; j < PN; ++j) red[(warp * TM + lm + 8 * i) * TN + ln + 4 * j] = acc[i][j];
+    __syncthreads();
+    for (int e = threadIdx.x; e < TM * TN; e += THREADS) {
+        const int m = m0 + e / TN, n = n0 + e % TN;
+        if (m >= M || n >= N) continue;
+        double x = 0.0, y = 0.0;
+#pragma unroll
+        for (int w = 0; w < CN_WARPS; ++w) {
+            const c_t<T> v = red[w * TM * TN + e];
+            x += (double)v.x;
+            y += (double)v.y;
         }
+        atomicAdd(&out[(size_t)m * ldo + n].x, scale * x);
+        atomicAdd(&out[(size_t)m * ldo + n].y, scale * y);
+    }
+}
+
+template <typename T, int TM, int TN>
+static jdft_status launch_zgemm_cn(int M, int N, int K, const c_t<T>* A, int lda, const c_t<T>* B, int ldb,
+                                   double2* out, int ldo, double scale, cudaStream_t st) {
+    const int tiles = ((M + TM - 1) / TM) * ((N + TN - 1) / TN);
+    // enough K splits for two blocks per SM (one for a single tile: fewer atomics), each at least 16 deep
+    int splits = tiles == 1 ? 152 : (304 + tiles - 1) / tiles;
+    splits = std::min(splits, std::max(1, K / 16));
+    int kchunk = (K + splits - 1) / splits;
+    kchunk = (kchunk + CN_WARPS - 1) / CN_WARPS * CN_WARPS;
+    splits = (K + kchunk - 1) / kchunk;
+    dim3 grid((M + TM - 1) / TM, (N + TN - 1) / TN, splits);
+    const size_t smem = std::max<size_t>(CN_BK * (TM + 1 + TN + 1), CN_WARPS * TM * TN) * sizeof(c_t<T>);
+    cudaError_t e = set_smem_attr((const void*)zgemm_cn_kernel<T, TM, TN>, smem);
+    if (e != cudaSuccess) return set_error(JDFT_ERR_CUDA, std::string("zgemm_cn: ") + cudaGetErrorString(e));
+    {
+        Trace tr_("zgemm_cn", st);
+        zgemm_cn_kernel<T, TM, TN><<<grid, 32 * CN_WARPS, smem, st>>>(M, N, K, kchunk, A, lda, B, ldb, out, ldo, scale);
+    }
+    return check_launch("zgemm_cn");
 }
 
 template <typename T>
 jdft_status zgemm_cn(int M, int N, int K, const c_t<T>* A, int lda, const c_t<T>* B, int ldb, double2* out, int ldo,
                      double scale, cudaStream_t st) {
     if (M == 0 || N == 0 || K == 0) return JDFT_OK;
-    const int tiles = ((M + CN_BM - 1) / CN_BM) * ((N + CN_BN - 1) / CN_BN);
-    // enough K splits for ~4 blocks per SM, each at least 64 deep
-    int splits = std::max(1, (152 * 4 + tiles - 1) / tiles);
-    splits = std::min(splits, std::max(1, K / 64));
-    int kchunk = (K + splits - 1) / splits;
-    kchunk = (kchunk + CN_BK - 1) / CN_BK * CN_BK;
-    splits = (K + kchunk - 1) / kchunk;
-    dim3 grid((M + CN_BM - 1) / CN_BM, (N + CN_BN - 1) / CN_BN, splits);
-    {
-        Trace tr_("zgemm_cn", st);
-        zgemm_cn_kernel<T><<<grid, 256, 0, st>>>(M, N, K, kchunk, A, lda, B, ldb, out, ldo, scale);
-    }
-    return check_launch("zgemm_cn");
+    // 16-wide tiles where a 32-wide one would be at most half full at the edge
+    const bool m16 = (M - 1) % 32 < 16, n16 = (N - 1) % 32 < 16;
+    if (m16 && n16) return launch_zgemm_cn<T, 16, 16>(M, N, K, A, lda, B, ldb, out, ldo, scale, st);
+    if (m16) return launch_zgemm_cn<T, 16, 32>(M, N, K, A, lda, B, ldb, out, ldo, scale, st);
+    if (n16) return launch_zgemm_cn<T, 32, 16>(M, N, K, A, lda, B, ldb, out, ldo, scale, st);
+    return launch_zgemm_cn<T, 32, 32>(M, N, K, A, lda, B, ldb, out, ldo, scale, st);
 }
 
 // ---------------------------------------------------------------------------
-// out[n][m] += sum_i A[i][m] Bm[i][n]: tile 64 (m) x 16 (n), 16-deep i slices,
-// each thread one m and 4 n.
+// out[n][m] += sum_i A[i][m] Bm[i][n].  A block holds 32 m x 16 n, warp w the
+// columns 4 w .. 4 w + 3: a lane owns one m, reads A straight from global memory
+// (32 consecutive values a warp, sixteen rows in flight) and Bm, staged 64 rows deep, by broadcast.
+// Small blocks, because N is small where this kernel is used and M/32 of them
+// just fill the SMs: 16 x 16 over 4 259 rows 40 -> 23 us in FP64 against 64 m to a
+// block, which used 67 SMs.
 // ---------------------------------------------------------------------------
-constexpr int NN_BM = 64, NN_BN = 16, NN_BK = 16;
+constexpr int NN_BM = 32, NN_PN = 4, NN_WARPS = 4, NN_BN = NN_PN * NN_WARPS, NN_BK = 64;
 
 template <typename T>
-__global__ void __launch_bounds__(256) zgemm_nn_kernel(int M, int N, int K, const c_t<T>* __restrict__ A, int lda,
-                                                       const c_t<T>* __restrict__ Bm, int ldb, c_t<T>* __restrict__ out,
-                                                       int ldo, bool accumulate) {
-    __shared__ c_t<T> As[NN_BK][NN_BM];
-    __shared__ c_t<T> Bs[NN_BK][NN_BN];
-    const int m0 = blockIdx.x * NN_BM, n0 = blockIdx.y * NN_BN;
-    const int tm = threadIdx.x % NN_BM, tq = threadIdx.x / NN_BM;  // tq in 0..3
-    c_t<T> acc[4];
+__global__ void __launch_bounds__(32 * NN_WARPS)
+    zgemm_nn_kernel(int M, int N, int K, const c_t<T>* __restrict__ A, int lda, const c_t<T>* __restrict__ Bm, int ldb,
+                    c_t<T>* __restrict__ out, int ldo, bool accumulate) {
+    __shared__ __align__(16) c_t<T> Bs[NN_BK][NN_BN];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int m = blockIdx.x * NN_BM + lane, n0 = blockIdx.y * NN_BN;
+    c_t<T> acc[NN_PN];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[j] = mk<T>(T(0), T(0));
+    for (int j = 0; j < NN_PN; ++j) acc[j] = mk<T>(T(0), T(0));
     for (int k0 = 0; k0 < K; k0 += NN_BK) {
-        for (int e = threadIdx.x; e < NN_BK * NN_BM; e += 256) {
-            const int kk = e / NN_BM, r = e % NN_BM;
-            const int m = m0 + r, k = k0 + kk;
-            As[kk][r] = (m < M && k < K) ? A[(size_t)k * lda + m] : mk<T>(T(0), T(0));
-        }
-        for (int e = threadIdx.x; e < NN_BK * NN_BN; e += 256) {
+        for (int e = threadIdx.x; e < NN_BK * NN_BN; e += 32 * NN_WARPS) {
             const int kk = e / NN_BN, c = e % NN_BN;
-            const int n = n0 + c, k = k0 + kk;
-            Bs[kk][c] = (n < N && k < K) ? Bm[(size_t)k * ldb + n] : mk<T>(T(0), T(0));
+            Bs[kk][c] = (n0 + c < N && k0 + kk < K) ? Bm[(size_t)(k0 + kk) * ldb + n0 + c] : mk<T>(T(0), T(0));
         }
         __syncthreads();
+        const int kn = min(NN_BK, K - k0);
+        if (m < M) {
+            const c_t<T>* Ak = A + (size_t)k0 * lda + m;
+#pragma unroll 16
+            for (int kk = 0; kk < kn; ++kk) {
+                const c_t<T> a = Ak[(size_t)kk * lda];
 #pragma unroll
-        for (int kk = 0; kk < NN_BK; ++kk) {
-            const c_t<T> a = As[kk][tm];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const c_t<T> b = Bs[kk][tq * 4 + j];
-                acc[j].x += a.x * b.x - a.y * b.y;
-                acc[j].y += a.x * b.y + a.y * b.x;
+                for (int j = 0; j < NN_PN; ++j) {
+                    const c_t<T> b = Bs[kk][warp * NN_PN + j];
+                    acc[j].x += a.x * b.x - a.y * b.y;
+                    acc[j].y += a.x * b.y + a.y * b.x;
+                }
             }
         }
         __syncthreads();
     }
-    const int m = m0 + tm;
     if (m < M) {
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const int n = n0 + tq * 4 + j;
+        for (int j = 0; j < NN_PN; ++j) {
+            const int n = n0 + warp * NN_PN + j;
             if (n < N) out[(size_t)n * ldo + m] = accumulate ? cadd(out[(size_t)n * ldo + m], acc[j]) : acc[j];
         }
     }
@@ -152,7 +197,7 @@ jdft_status zgemm_nn_acc(int M, int N, int K, const c_t<T>* A, int lda, const c_
     dim3 grid((M + NN_BM - 1) / NN_BM, (N + NN_BN - 1) / NN_BN);
     {
         Trace tr_("zgemm_nn", st);
-        zgemm_nn_kernel<T><<<grid, 256, 0, st>>>(M, N, K, A, lda, Bm, ldb, out, ldo, accumulate);
+        zgemm_nn_kernel<T><<<grid, 32 * NN_WARPS, 0, st>>>(M, N, K, A, lda, Bm, ldb, out, ldo, accumulate);
     }
     return check_launch("zgemm_nn");
 }
