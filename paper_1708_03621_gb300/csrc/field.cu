@@ -41,10 +41,13 @@
 // summing i G_d (J ...)_d into the result (and the CG product d.Hd).
 #include <chrono>
 #include <cmath>
+#include <cstdlib>
 #include <vector>
 
 #include "common.cuh"
 #include "fft.cuh"
+#include "field_fast.cuh"
+#include "field_lda.cuh"
 #include "profile.cuh"
 
 namespace jdft {
@@ -97,39 +100,6 @@ AxisGeom axis_geom(const jdft_basis_s* b, int axis) {
 }
 
 __device__ __forceinline__ int fold(int m, int S) { return m < (S + 1) / 2 ? m : m - S; }
-
-// Slater exchange + Perdew-Zunger correlation: energy per electron e and
-// potential v at density n (both zero for n <= 0).
-__device__ __forceinline__ void lda_pz(double n, double& e, double& v) {
-    if (!(n > 0.0)) { e = 0.0; v = 0.0; return; }
-    // one cube root and one reciprocal per point (FP64 transcendentals and
-    // divisions are the cost of this epilogue on this GPU's FP64 rate)
-    const double cx = -0.73855876638202240588423003065;   // -(3/4)(3/pi)^{1/3}
-    const double kr = 0.62035049089940001666800681204778;  // (3/(4 pi))^{1/3}
-    const double third = 1.0 / 3.0;
-    const double c = cbrt(n);
-    const double ex = cx * c;
-    const double rs = kr / c;
-    double ec, vc;
-    if (rs >= 1.0) {
-        const double g = -0.1423, b1 = 1.0529, b2 = 0.3334;
-        const double sq = sqrt(rs);
-        const double iden = 1.0 / (1.0 + b1 * sq + b2 * rs);
-        ec = g * iden;
-        // r_s de_c/dr_s = -g (b1 sqrt(r_s) / 2 + b2 r_s) / den^2
-        const double rdec = -g * (0.5 * b1 * sq + b2 * rs) * iden * iden;
-        vc = ec - third * rdec;
-    } else {
-        const double A = 0.0311, B = -0.048, C = 0.0020, D = -0.0116;
-        const double lr = log(rs);
-        ec = A * lr + B + C * rs * lr + D * rs;
-        // r_s de_c/dr_s = A + r_s (C (ln r_s + 1) + D)
-        const double rdec = A + rs * (C * (lr + 1.0) + D);
-        vc = ec - third * rdec;
-    }
-    e = ex + ec;
-    v = (4.0 * third) * ex + vc;
-}
 
 // Sum over the block; thread 0 returns the total (others: partial values).
 __device__ __forceinline__ double block_sum(double x) {
@@ -366,6 +336,50 @@ jdft_status field_work(jdft_basis_s* b, FieldWork* w, int nbox = 1) {
     return JDFT_OK;
 }
 
+// Call of a member of FieldFast<T, n> or HartreeFast<n> for the compiled length n
+// (JDFT_ERR_UNSUPPORTED otherwise): the call's template argument is N.
+#define JDFT_FIELD_LENGTH(n, ...)                                       \
+    [&]() -> jdft_status {                                              \
+        switch (n) {                                                    \
+            case 12: { constexpr int N = 12; return __VA_ARGS__; }      \
+            case 16: { constexpr int N = 16; return __VA_ARGS__; }      \
+            case 40: { constexpr int N = 40; return __VA_ARGS__; }      \
+            case 48: { constexpr int N = 48; return __VA_ARGS__; }      \
+            case 64: { constexpr int N = 64; return __VA_ARGS__; }      \
+            case 80: { constexpr int N = 80; return __VA_ARGS__; }      \
+            case 128: { constexpr int N = 128; return __VA_ARGS__; }    \
+            case 256: { constexpr int N = 256; return __VA_ARGS__; }    \
+        }                                                               \
+        return JDFT_ERR_UNSUPPORTED;                                    \
+    }()
+
+// JDFT_FAST_PLANE=0 turns every register-FFT path off (tests compare the two).
+bool field_fast(int n) {
+    const char* e = getenv("JDFT_FAST_PLANE");
+    return field_fast_length(n) && !(e && e[0] == '0');
+}
+
+FieldCell field_cell(const jdft_basis_s* b) {
+    FieldCell q;
+    for (int i = 0; i < 9; ++i) q.B[i] = b->B[i];
+    for (int d = 0; d < 3; ++d) q.S[d] = b->S[d];
+    return q;
+}
+
+// Lines of an axis of a box whose last edge is s2 (the full box or the half one).
+LineGeom line_geom(const jdft_basis_s* b, int axis, int s2) {
+    const int S0 = b->S[0], S1 = b->S[1];
+    LineGeom g;
+    if (axis == 2) {
+        g.nlines = S0 * S1; g.inner = g.nlines; g.istride = s2; g.ostride = 0; g.es = 1;
+    } else if (axis == 1) {
+        g.nlines = S0 * s2; g.inner = s2; g.istride = 1; g.ostride = (int64_t)S1 * s2; g.es = s2;
+    } else {
+        g.nlines = S1 * s2; g.inner = g.nlines; g.istride = 1; g.ostride = 0; g.es = (int64_t)S1 * s2;
+    }
+    return g;
+}
+
 size_t axis_smem(const AxisGeom& g) {
     // two padded buffers, the line bases and (for the Coulomb-kernel pass) 3 doubles a line
     return (size_t)2 * padded_len(g.W * g.n) * sizeof(double2) + (size_t)g.W * sizeof(int64_t) +
@@ -375,6 +389,13 @@ size_t axis_smem(const AxisGeom& g) {
 template <int SIGN, bool IN_REAL, bool KERNEL, int OUT>
 jdft_status launch_axis(const char* name, jdft_basis_s* b, int axis, const void* in, void* out, const FieldArgs& a,
                         cudaStream_t st, int* nblocks = nullptr, int batch = 1) {
+    if constexpr (!IN_REAL && !KERNEL && OUT == OUT_COMPLEX) {
+        if (field_fast(b->S[axis]))
+            return JDFT_FIELD_LENGTH(b->S[axis],
+                                     FieldFast<double, N>::axis(name, SIGN, (const double2*)in, (double2*)out,
+                                                                line_geom(b, axis, b->S[2]), a.scale, batch, a.bstride,
+                                                                b->tw64, b->plan[axis], st));
+    }
     const AxisGeom g = axis_geom(b, axis);
     const int64_t grid = (g.nlines + g.W - 1) / g.W;
     if ((KERNEL || OUT == OUT_KS) && grid > kPartialMax)
@@ -426,6 +447,33 @@ jdft_status hartree_chain(jdft_basis_s* b, const double* n, const double* vion, 
     const int64_t half = kPartialMax / 2;
     FieldArgs a = field_args(b, w.partial);
     int nb_h = 0, nb_x = 0;
+    if (field_fast(b->S[0]) && field_fast(b->S[1]) && field_fast(b->S[2])) {
+        // real fields on the half box; every pass has fewer than `half` blocks (256^2 lines at most, 8 and more a block)
+        const FieldCell q = field_cell(b);
+        const int H = b->S[2] / 2 + 1, lines = b->S[0] * b->S[1];
+        const LineGeom g1 = line_geom(b, 1, H);
+        double2* x = w.box;
+        if ((s = JDFT_FIELD_LENGTH(b->S[2], HartreeFast<N>::forward2(n, x, lines, b->tw64, b->plan[2], st)))) return s;
+        if ((s = JDFT_FIELD_LENGTH(b->S[1], FieldFast<double, N>::axis("field_fft_axis1", -1, x, x, g1, 1.0, 1, 0,
+                                                                       b->tw64, b->plan[1], st))))
+            return s;
+        if ((s = JDFT_FIELD_LENGTH(b->S[0], HartreeFast<N>::kernel0(x, q, w.partial, &nb_h, b->tw64, b->plan[0], st))))
+            return s;
+        if ((s = JDFT_FIELD_LENGTH(b->S[1], FieldFast<double, N>::axis("field_fft_axis1", +1, x, x, g1, 1.0, 1, 0,
+                                                                       b->tw64, b->plan[1], st))))
+            return s;
+        if ((s = JDFT_FIELD_LENGTH(b->S[2], HartreeFast<N>::inverse2(x, V, OUT == OUT_KS ? n : nullptr,
+                                                                     OUT == OUT_KS ? vion : nullptr, w.partial + half,
+                                                                     &nb_x, lines, b->tw64, b->plan[2], st))))
+            return s;
+        if (energies) {
+            if ((s = launch_reduce(w.partial, nb_h, 1, 1, 0.5 * b->omega, energies, false, st))) return s;
+            if (OUT == OUT_KS)
+                if ((s = launch_reduce(w.partial + half, nb_x, 1, 1, b->omega / (double)b->N, energies + 1, false, st)))
+                    return s;
+        }
+        return JDFT_OK;
+    }
     for (int axis = 0; axis < 3; axis += 2) {
         const AxisGeom g = axis_geom(b, axis);
         if ((g.nlines + g.W - 1) / g.W > half) return set_error(JDFT_ERR_ARG, "box too large for the partial sums");
@@ -962,6 +1010,27 @@ template <typename T>
 jdft_status pcm_hessian(jdft_basis_s* b, const T* eps, const c_t<T>* X, c_t<T>* out, c_t<T>* Yg,
                         const c_t<T>* din, double* partial, int* nblocks, cudaStream_t st) {
     const GArgs q = g_args(b);
+    if (field_fast(b->S[0]) && field_fast(b->S[1]) && field_fast(b->S[2])) {
+        const FieldCell c = field_cell(b);
+        const c_t<T>* tw = twiddles_of<T>(b);
+        const LineGeom g1 = line_geom(b, 1, b->S[2]);
+        const int64_t NB = b->N;
+        int blocks = 0;
+        jdft_status s;
+        if ((s = JDFT_FIELD_LENGTH(b->S[0], FieldFast<T, N>::grad(X, Yg, c, NB, tw, b->plan[0], st)))) return s;
+        if ((s = JDFT_FIELD_LENGTH(b->S[1], FieldFast<T, N>::axis("field_fft_axis1_batch", +1, Yg, Yg, g1, T(1), 3, NB,
+                                                                  tw, b->plan[1], st))))
+            return s;
+        if ((s = JDFT_FIELD_LENGTH(b->S[2], FieldFast<T, N>::eps(Yg, eps, b->S[0] * b->S[1], NB, tw, b->plan[2], st))))
+            return s;
+        if ((s = JDFT_FIELD_LENGTH(b->S[1], FieldFast<T, N>::axis("field_fft_axis1_batch", -1, Yg, Yg, g1, T(1), 3, NB,
+                                                                  tw, b->plan[1], st))))
+            return s;
+        s = JDFT_FIELD_LENGTH(b->S[0], FieldFast<T, N>::div(Yg, din, out, c, NB, -1.0 / (kFourPi * (double)NB),
+                                                            partial, &blocks, tw, b->plan[0], st));
+        if (nblocks) *nblocks = blocks;
+        return s;
+    }
     const AxisGeom g0 = axis_geom(b, 0), g1 = axis_geom(b, 1), g2 = axis_geom(b, 2);
     const int64_t grid0 = (g0.nlines + g0.W - 1) / g0.W;
     const int64_t grid1 = (g1.nlines + g1.W - 1) / g1.W;

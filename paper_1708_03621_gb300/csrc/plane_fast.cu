@@ -21,7 +21,7 @@
 #include <type_traits>
 
 #include "chain.cuh"
-#include "fft_reg.cuh"
+#include "fft_lanes.cuh"
 #include "profile.cuh"
 #include "tc_ptx.cuh"
 
@@ -33,48 +33,9 @@ constexpr int kFastWarps = kFastThreads / 32;
 constexpr int kZWarps = 8;
 constexpr int kZThreads = 32 * kZWarps;
 
-// i mod N in [0, N) for either sign of i: one bit mask when N is a power of
-// two (two's complement), else a remainder and a correction.
-template <int N>
-__device__ __forceinline__ int wrapn(int i) {
-    if constexpr ((N & (N - 1)) == 0) {
-        return i & (N - 1);
-    } else {
-        const int r = i % N;
-        return r < 0 ? r + N : r;
-    }
-}
-
-// Shared-memory layout of the register-FFT kernels.  A warp's 8-byte shared
-// access is served in two halves of 16 lanes and a 16-byte access in four
-// quarters of 8 lanes; lanes of one group that hit different addresses in the
-// same bank slot (16 eight-byte or 8 sixteen-byte slots per 128 bytes) cost
-// one wavefront each.  The constants below are the ones with the fewest such
-// conflicts over every shared access of these kernels, counted access by
-// access (plane_layout.py beside this package prints them); the 128^3 FP32
-// plane pass has none.
-//
-// Lanes: a line of N values is split over TL = N / E lanes and a warp serves
-// LPW = 32 / TL lines; lane l takes position l / LPW of line l % LPW, so a
-// half-warp covers several lines at once and several consecutive rows or
-// columns of the plane array.
-template <int N, int E>
-struct Lanes {
-    static constexpr int TL = N / E, LPW = 32 / TL;
-    static __device__ __forceinline__ int line(int lane) { return lane % LPW; }
-    static __device__ __forceinline__ int pos(int lane) { return lane / LPW; }
-};
-
-// Elements between the LPW scratch lines of one warp (each line needs
-// padded_line(N)).
-template <typename T, int N>
-struct ScratchSpacing;
-#define JDFT_SCRATCH_SPACING(T, N, SP)                                                      \
-    template <>                                                                             \
-    struct ScratchSpacing<T, N> {                                                           \
-        static constexpr int value = SP;                                                    \
-        static_assert(SP >= padded_line(N), "scratch lines of one warp must not overlap"); \
-    };
+// The scratch-line spacings of fft_lanes.cuh, listed with the plane strides below
+// (plane_layout.py prints both tables).
+#define JDFT_SCRATCH_SPACING(T, N, SP) static_assert(ScratchSpacing<T, N>::value == SP, "spacing table");
 JDFT_SCRATCH_SPACING(float, 12, 13)
 JDFT_SCRATCH_SPACING(float, 16, 17)
 JDFT_SCRATCH_SPACING(float, 40, 43)
@@ -202,8 +163,8 @@ __device__ __forceinline__ void column_inverse_fast(const ChainGeom& g, const c_
 }
 
 // The plane pass of H: rows inverse, columns inverse x V forward, rows forward.
-template <typename T, int N0, int E0, class R0, int N1, int E1, class R1>
-__global__ void __launch_bounds__(kFastThreads) plane_apply_fast_kernel(ChainGeom g, c_t<T>* __restrict__ colbuf,
+template <typename T, int N0, int E0, class R0, int N1, int E1, class R1, int NW, int MB>
+__global__ void __launch_bounds__(32 * NW, MB) plane_apply_fast_kernel(ChainGeom g, c_t<T>* __restrict__ colbuf,
                                                                         const T* __restrict__ Vp,
                                                                         const c_t<T>* __restrict__ tw0,
                                                                         const c_t<T>* __restrict__ tw1) {
@@ -213,7 +174,7 @@ __global__ void __launch_bounds__(kFastThreads) plane_apply_fast_kernel(ChainGeo
     c_t<T>* W0 = reinterpret_cast<c_t<T>*>(smem_raw);
     c_t<T>* W1 = W0 + N0;
     c_t<T>* scr_all = W1 + N1;
-    c_t<T>* A = scr_all + kFastWarps * SCR;
+    c_t<T>* A = scr_all + NW * SCR;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     c_t<T>* wscr = scr_all + warp * SCR;
     for (int i = threadIdx.x; i < N0; i += blockDim.x) W0[i] = tw0[i];
@@ -222,7 +183,7 @@ __global__ void __launch_bounds__(kFastThreads) plane_apply_fast_kernel(ChainGeo
     const int j2 = blockIdx.x, b = blockIdx.y;
     c_t<T>* plane = colbuf + colbuf_index(g, b, j2, 0);
 
-    rows_inverse_fast<T, N1, E1, R1>(g, plane, A, lsA, wscr, W1, warp, lane);
+    rows_inverse_fast<T, N1, E1, R1, NW>(g, plane, A, lsA, wscr, W1, warp, lane);
     __syncthreads();
 
     {
@@ -232,8 +193,8 @@ __global__ void __launch_bounds__(kFastThreads) plane_apply_fast_kernel(ChainGeo
         const int liw = LN::line(lane), t = LN::pos(lane);
         c_t<T>* scr = wscr + liw * ScratchSpacing<T, N0>::value;
         // every lane has a column when the rounds tile the plane exactly
-        constexpr bool kAllCols = N1 % (kFastWarps * LPW) == 0;
-        for (int base = warp * LPW; base < N1; base += kFastWarps * LPW) {
+        constexpr bool kAllCols = N1 % (NW * LPW) == 0;
+        for (int base = warp * LPW; base < N1; base += NW * LPW) {
             const int j1 = base + liw;
             const bool act = kAllCols || j1 < N1;
             c_t<T> v[E0];
@@ -255,7 +216,7 @@ __global__ void __launch_bounds__(kFastThreads) plane_apply_fast_kernel(ChainGeo
     }
     __syncthreads();
 
-    rows_forward_fast<T, N1, E1, R1>(g, plane, A, lsA, wscr, W1, warp, lane);
+    rows_forward_fast<T, N1, E1, R1, NW>(g, plane, A, lsA, wscr, W1, warp, lane);
 }
 
 // Density, FP32 blocks: block (j2, band group) accumulates f_b |psi_b|^2 in
@@ -615,33 +576,30 @@ __global__ void __launch_bounds__(kZThreads) zpass_forward_batch_kernel(const KJ
     }
 }
 
-// Line shapes per compiled length: E values per lane and the radix list.
-template <int N> struct FastCfg;
-template <> struct FastCfg<12> { static constexpr int E = 12; using R = Rad<4, 3>; };
-template <> struct FastCfg<16> { static constexpr int E = 16; using R = Rad<16>; };
-template <> struct FastCfg<40> { static constexpr int E = 20; using R = Rad<2, 4, 5>; };
-template <> struct FastCfg<48> { static constexpr int E = 12; using R = Rad<4, 4, 3>; };
-template <> struct FastCfg<64> { static constexpr int E = 8; using R = Rad<8, 8>; };
-template <> struct FastCfg<80> { static constexpr int E = 20; using R = Rad<4, 4, 5>; };
-template <> struct FastCfg<128> { static constexpr int E = 16; using R = Rad<16, 8>; };
-template <> struct FastCfg<256> { static constexpr int E = 16; using R = Rad<16, 16>; };
-
 constexpr size_t kFastMaxSmem = 220 * 1024;
 
-// The table the register line FFTs of type T read: the fixed-point one for FP64.
-template <typename T>
-static const c_t<T>* reg_table(const c_t<T>* tw_base, const FftPlan& p) {
-    return tw_base + (std::is_same<T, double>::value ? p.fx_offset : p.tw_offset);
+template <typename T, int N0, int N1>
+static size_t fast_smem(const ChainGeom& g, int nw = kFastWarps) {
+    constexpr int scr = warp_scratch<T, N0, RegCfg<T, N0>::E, N1, RegCfg<T, N1>::E>();
+    return ((size_t)N0 + N1 + (size_t)nw * scr + (size_t)g.nrows * PlaneStride<T, N0, N1>::value) * sizeof(c_t<T>);
 }
 
-template <int N0, int N1>
-static size_t fast_smem(const ChainGeom& g, size_t elem, int nw = kFastWarps) {
-    constexpr int E0 = FastCfg<N0>::E, E1 = FastCfg<N1>::E;
-    const bool dbl = elem == sizeof(double2);
-    const int lsA = dbl ? PlaneStride<double, N0, N1>::value : PlaneStride<float, N0, N1>::value;
-    const int scr = dbl ? warp_scratch<double, N0, E0, N1, E1>() : warp_scratch<float, N0, E0, N1, E1>();
-    return ((size_t)N0 + N1 + (size_t)nw * scr + (size_t)g.nrows * lsA) * elem;
-}
+// Warps of a block of the H plane pass, and the blocks an SM must hold (the
+// register limit).  FP64 lines are long integer chains, so what counts is warps in
+// flight, and on small planes that few of a block's warps idle: 48 columns are 6
+// warps' worth of lines, 21 sphere rows 3, so blocks of 3 warps, 6 to an SM, against
+// one block of 8 warps: 48^3, 16 bands 205 -> 81 us (the limit of 96 registers costs
+// some 50 spilled words); 128^3, 64 bands, 16 warps of 8-value lanes against 8 of
+// 16-value ones 5.34 -> 4.05 ms.
+template <typename T, int N0, int N1>
+struct PlaneBlock {
+    static constexpr int warps = kFastWarps, per_sm = 1;
+};
+template <> struct PlaneBlock<double, 40, 40> { static constexpr int warps = 3, per_sm = 3; };
+template <> struct PlaneBlock<double, 48, 48> { static constexpr int warps = 3, per_sm = 6; };
+template <> struct PlaneBlock<double, 64, 64> { static constexpr int warps = 8, per_sm = 2; };
+template <> struct PlaneBlock<double, 80, 80> { static constexpr int warps = 5, per_sm = 2; };
+template <> struct PlaneBlock<double, 128, 128> { static constexpr int warps = 16, per_sm = 1; };
 
 // Warps of a density block: enough that the per-lane accumulators of the
 // plane (N0 N1 / (32 warps) values) stay at 32 or fewer where the shared
@@ -659,16 +617,17 @@ static bool fast_disabled() {
 template <typename T, int N0, int N1>
 static jdft_status apply_fast_impl(const ChainGeom& g, c_t<T>* colbuf, const T* Vp, int nb, const c_t<T>* tw_base,
                                    cudaStream_t st) {
-    using C0 = FastCfg<N0>;
-    using C1 = FastCfg<N1>;
-    const size_t smem = fast_smem<N0, N1>(g, sizeof(c_t<T>));
+    using C0 = RegCfg<T, N0>;
+    using C1 = RegCfg<T, N1>;
+    using PB = PlaneBlock<T, N0, N1>;
+    const size_t smem = fast_smem<T, N0, N1>(g, PB::warps);
     if (smem > kFastMaxSmem) return JDFT_ERR_UNSUPPORTED;
-    auto kern = plane_apply_fast_kernel<T, N0, C0::E, typename C0::R, N1, C1::E, typename C1::R>;
+    auto kern = plane_apply_fast_kernel<T, N0, C0::E, typename C0::R, N1, C1::E, typename C1::R, PB::warps, PB::per_sm>;
     cudaError_t e = set_smem_attr((const void*)kern, smem);
     if (e != cudaSuccess) return set_error(JDFT_ERR_CUDA, std::string("plane_apply_fast: ") + cudaGetErrorString(e));
     {
         Trace tr_("plane_apply_fast", st);
-        kern<<<dim3(g.S2, nb), kFastThreads, smem, st>>>(g, colbuf, Vp, reg_table<T>(tw_base, g.p0),
+        kern<<<dim3(g.S2, nb), 32 * PB::warps, smem, st>>>(g, colbuf, Vp, reg_table<T>(tw_base, g.p0),
                                                          reg_table<T>(tw_base, g.p1));
     }
     return check_launch("plane_apply_fast");
@@ -680,7 +639,7 @@ static jdft_status density_fast_impl(const ChainGeom& g, const float2* colbuf, c
     using C0 = FastCfg<N0>;
     using C1 = FastCfg<N1>;
     constexpr int NW = DensityWarps<N0, N1>::value;
-    const size_t smem = fast_smem<N0, N1>(g, sizeof(float2), NW);
+    const size_t smem = fast_smem<float, N0, N1>(g, NW);
     if (smem > kFastMaxSmem) return JDFT_ERR_UNSUPPORTED;
     auto kern = plane_density_fast_kernel<N0, C0::E, typename C0::R, N1, C1::E, typename C1::R, NW>;
     cudaError_t e = set_smem_attr((const void*)kern, smem);
@@ -700,27 +659,27 @@ static jdft_status density_fast_impl(const ChainGeom& g, const float2* colbuf, c
 
 template <typename T, int N2>
 static size_t zpass_fast_smem() {
-    constexpr int LPW = Lanes<N2, FastCfg<N2>::E>::LPW;
+    constexpr int LPW = Lanes<N2, RegCfg<T, N2>::E>::LPW;
     return ((size_t)N2 + (size_t)kZWarps * LPW * ScratchSpacing<T, N2>::value) * sizeof(c_t<T>);
 }
 
-template <int N2>
+template <typename T, int N2>
 static int zpass_fast_blocks(const ChainGeom& g) {
-    constexpr int TL = N2 / FastCfg<N2>::E, LPW = 32 / TL;
+    constexpr int TL = N2 / RegCfg<T, N2>::E, LPW = 32 / TL;
     return (g.ncols + kZWarps * LPW - 1) / (kZWarps * LPW);
 }
 
 template <typename T, int N2>
 static jdft_status zinv_fast_impl(const ChainGeom& g, const c_t<T>* C, int ldc, c_t<T>* colbuf, int nb,
                                   const c_t<T>* tw2, cudaStream_t st) {
-    using C2 = FastCfg<N2>;
+    using C2 = RegCfg<T, N2>;
     auto kern = zpass_inverse_fast_kernel<T, N2, C2::E, typename C2::R>;
     const size_t smem = zpass_fast_smem<T, N2>();
     cudaError_t e = set_smem_attr((const void*)kern, smem);
     if (e != cudaSuccess) return set_error(JDFT_ERR_CUDA, std::string("zpass_inverse_fast: ") + cudaGetErrorString(e));
     {
         Trace tr_("zpass_inverse", st);
-        kern<<<dim3(zpass_fast_blocks<N2>(g), nb), kZThreads, smem, st>>>(g, C, ldc, colbuf,
+        kern<<<dim3(zpass_fast_blocks<T, N2>(g), nb), kZThreads, smem, st>>>(g, C, ldc, colbuf,
                                                                           reg_table<T>(tw2 - g.p2.tw_offset, g.p2));
     }
     return check_launch("zpass_inverse_fast");
@@ -730,14 +689,14 @@ template <typename T, int MODE, int N2>
 static jdft_status zfwd_fast_impl(const ChainGeom& g, const c_t<T>* colbuf, const c_t<T>* C, int ldc, c_t<T>* out,
                                   int ldo, int nb, const T* kin, T omega, T scale, const c_t<T>* tw2,
                                   cudaStream_t st) {
-    using C2 = FastCfg<N2>;
+    using C2 = RegCfg<T, N2>;
     auto kern = zpass_forward_fast_kernel<T, N2, C2::E, typename C2::R, MODE>;
     const size_t smem = zpass_fast_smem<T, N2>();
     cudaError_t e = set_smem_attr((const void*)kern, smem);
     if (e != cudaSuccess) return set_error(JDFT_ERR_CUDA, std::string("zpass_forward_fast: ") + cudaGetErrorString(e));
     {
         Trace tr_("zpass_forward", st);
-        kern<<<dim3(zpass_fast_blocks<N2>(g), nb), kZThreads, smem, st>>>(g, colbuf, C, ldc, out, ldo, kin, omega,
+        kern<<<dim3(zpass_fast_blocks<T, N2>(g), nb), kZThreads, smem, st>>>(g, colbuf, C, ldc, out, ldo, kin, omega,
                                                                             scale,
                                                                             reg_table<T>(tw2 - g.p2.tw_offset, g.p2));
     }
@@ -753,7 +712,7 @@ static jdft_status apply_density_fast_impl(const ChainGeom& g, float2* colbuf, c
                                            cudaStream_t st) {
     using C0 = FastCfg<N0>;
     using C1 = FastCfg<N1>;
-    const size_t smem = std::max<size_t>(fast_smem<N0, N1>(g, sizeof(float2)), 58 * 1024);
+    const size_t smem = std::max<size_t>(fast_smem<float, N0, N1>(g), 58 * 1024);
     if (smem > kFastMaxSmem) return JDFT_ERR_UNSUPPORTED;
     auto kern = plane_apply_density_fast_kernel<N0, C0::E, typename C0::R, N1, C1::E, typename C1::R>;
     cudaError_t e = set_smem_attr((const void*)kern, smem);
@@ -784,8 +743,6 @@ jdft_status launch_plane_apply_density_fast(const ChainGeom& g, float2* colbuf, 
     if (g.S0 == 16 && g.S1 == 12) return apply_density_fast_impl<16, 12>(g, colbuf, Vp, nb, f, w, n_r, tw_base, st);
     return JDFT_ERR_UNSUPPORTED;
 }
-
-#define JDFT_FAST_LENGTHS(X) X(12) X(16) X(40) X(48) X(64) X(80) X(128) X(256)
 
 template <typename T>
 jdft_status launch_zpass_inverse_fast(const ChainGeom& g, const c_t<T>* C, int ldc, c_t<T>* colbuf, int nb,
