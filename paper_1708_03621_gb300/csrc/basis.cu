@@ -9,6 +9,7 @@
 #include <map>
 #include <mutex>
 
+#include "chain.cuh"
 #include "common.cuh"
 #include "gemm.cuh"
 #include "profile.cuh"
@@ -263,8 +264,9 @@ static jdft_status build_twiddles(jdft_basis_s* b) {
 // Potential store: permute V (j2 fastest) into the plane-pass order
 // Vp[(j2 * S1 + j1) * S0 + j0], in FP64 and FP32.
 // ------------------------------------------------------------------------
+// Vn, Vn32: copies in natural order, or null.
 __global__ void permute_potential(const double* __restrict__ V, double* __restrict__ Vp, float* __restrict__ V32,
-                                  int S0, int S1, int S2) {
+                                  double* __restrict__ Vn, float* __restrict__ Vn32, int S0, int S1, int S2) {
     int64_t N = (int64_t)S0 * S1 * S2;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N; i += (int64_t)gridDim.x * blockDim.x) {
         int64_t j0 = i % S0;
@@ -274,6 +276,11 @@ __global__ void permute_potential(const double* __restrict__ V, double* __restri
         double v = V[(j0 * S1 + j1) * S2 + j2];
         Vp[i] = v;
         V32[i] = (float)v;
+        if (Vn) {
+            const double u = V[i];
+            Vn[i] = u;
+            Vn32[i] = (float)u;
+        }
     }
 }
 
@@ -397,7 +404,7 @@ jdft_status jdft_basis_destroy(jdft_basis_t b) {
     cudaGetDevice(&prev);
     cudaSetDevice(b->device);
     for (auto& s : b->ks) free_sphere(s);
-    cudaFree(b->tw64); cudaFree(b->tw32); cudaFree(b->V); cudaFree(b->V32); cudaFree(b->work.ptr);
+    cudaFree(b->tw64); cudaFree(b->tw32); cudaFree(b->V); cudaFree(b->V32); cudaFree(b->Vn); cudaFree(b->Vn32); cudaFree(b->work.ptr);
     b->prodwork.release();
     if (b->side) {
         cudaStreamSynchronize(b->side);
@@ -446,10 +453,14 @@ jdft_status jdft_set_potential(jdft_basis_t b, const double* V, void* stream) {
         JDFT_CUDA_TRY(cudaMalloc(&b->V, b->N * sizeof(double)));
         JDFT_CUDA_TRY(cudaMalloc(&b->V32, b->N * sizeof(float)));
     }
+    if (!b->Vn && lines_serve(b)) {
+        JDFT_CUDA_TRY(cudaMalloc(&b->Vn, b->N * sizeof(double)));
+        JDFT_CUDA_TRY(cudaMalloc(&b->Vn32, b->N * sizeof(float)));
+    }
     {
         Trace tr_("permute_potential", (cudaStream_t)stream);
-        permute_potential<<<grid_for(b->N, 256), 256, 0, (cudaStream_t)stream>>>(V, b->V, b->V32, b->S[0], b->S[1],
-                                                                                 b->S[2]);
+        permute_potential<<<grid_for(b->N, 256), 256, 0, (cudaStream_t)stream>>>(V, b->V, b->V32, b->Vn, b->Vn32, b->S[0],
+                                                                                 b->S[1], b->S[2]);
     }
     b->have_V = true;
     return check_launch("permute_potential");

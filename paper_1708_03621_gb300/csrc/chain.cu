@@ -21,6 +21,7 @@
 #include <type_traits>
 
 #include "chain.cuh"
+#include "line_path.cuh"
 #include "profile.cuh"
 #include "gemm.cuh"
 
@@ -512,13 +513,6 @@ static jdft_status check_block(const void* p, int ld, int npw, int nb, jdft_prec
     return JDFT_OK;
 }
 
-// Bands per chunk so one chunk's column buffer stays near `budget` bytes.
-static int chunk_bands(const ChainGeom& g, size_t elem, int nb, size_t budget) {
-    const size_t per = (size_t)g.S2 * g.ncols * elem;
-    int c = (int)std::max<size_t>(1, budget / per);
-    return std::max(1, std::min(nb, c));
-}
-
 // Column-buffer bytes per chunk of bands.  The environment variable
 // JDFT_CHUNK_MB overrides it (read on every call), then a value the
 // autotuner stored in the basis, then 256 MB: measured on the 128^3,
@@ -547,22 +541,129 @@ static const T* kinetic(const KSphere& s);
 template <> const double* kinetic<double>(const KSphere& s) { return s.kin; }
 template <> const float* kinetic<float>(const KSphere& s) { return s.kin32; }
 
+// ---------------------------------------------------------------------------
+// The chain of one chunk of bands: the z pass, plane pass and z pass of the fused
+// and generic plane kernels, or the line-transform chain (line_path.cuh).
+// ---------------------------------------------------------------------------
+bool lines_serve(const jdft_basis_s* b) {
+    return line_length(b->S[0]) && line_length(b->S[1]) && line_length(b->S[2]);
+}
+
+// What a chunk of bands is taken through.
+enum class ChainUse { kH, kDensity, kHDensity, kBox };
+
+// Whether the line-transform chain takes it (on boxes it serves).  I, J and the FP64
+// density have no fused plane kernel.  H C of FP32 blocks keeps the fused kernels
+// where they are compiled: 32 bands 92 us fused against 112 on 64^3, 518 against 835
+// on 128^3, 247 against 255 on 80 x 80 x 75, whose z passes are generic.  With FP64
+// blocks a fused block's shared plane and wide lines leave few warps an SM: 16 bands
+// 201 us fused against 109 on 40^3, 170 against 133 on 48^3, 755 against 546 on 80^3; on 64^3
+// (225, 229) and 128^3 (1983, 2213) the fused kernel is kept, with z lengths that have
+// a register z pass.
+// JDFT_LINE_PATH=1 takes every use, 0 none; JDFT_FAST_PLANE=0 leaves the generic
+// kernels only.
+template <typename T>
+static bool use_lines(const jdft_basis_s* b, const ChainGeom& g, ChainUse use) {
+    const char* e = getenv("JDFT_FAST_PLANE");
+    const char* l = getenv("JDFT_LINE_PATH");
+    if (!lines_serve(b) || (e && e[0] == '0') || (l && l[0] == '0')) return false;
+    if ((use == ChainUse::kH || use == ChainUse::kHDensity) && !b->Vn) return false;
+    if (l && l[0] == '1') return true;
+    constexpr bool dbl = std::is_same<T, double>::value;
+    if (use == ChainUse::kBox) return true;
+    if (dbl && use != ChainUse::kH) return true;
+    if (dbl && !(g.S0 == g.S1 && (g.S0 == 64 || g.S0 == 128) && zpass_fused(g.S2))) return true;
+    return !plane_apply_fused<T>(g);
+}
+
+template <typename T>
+static const T* potential_natural(const jdft_basis_s* b);
+template <> const double* potential_natural<double>(const jdft_basis_s* b) { return b->Vn; }
+template <> const float* potential_natural<float>(const jdft_basis_s* b) { return b->Vn32; }
+
+template <typename T>
+struct BandChain {
+    jdft_basis_s* b;
+    int ik, nc;
+    ChainGeom g;
+    bool lines;
+    size_t bytes;  // of the intermediates of nc bands
+    c_t<T>*col = nullptr, *row = nullptr;
+
+    BandChain(const jdft_basis_s* b_, int ik_, int nb, ChainUse use)
+        : b(const_cast<jdft_basis_s*>(b_)), ik(ik_), g(make_geom(b_, ik_)) {
+        lines = use_lines<T>(b, g, use);
+        // line chain: larger launches beat chunks that stay in L2 (128 bands on 90^3, FP32: 1142 us in
+        // chunks of 64 MB, 1043 of 256 MB), as for the fused kernels
+        const size_t per = ((size_t)g.ncols + (lines ? (size_t)g.nrows * g.S1 : 0)) * g.S2 * sizeof(c_t<T>);
+        nc = std::max(1, std::min(nb, (int)std::max<size_t>(1, chunk_budget(b) / per)));
+        bytes = (nc * per + 255) / 256 * 256;
+    }
+    void bind(void* work) {
+        col = (c_t<T>*)work;
+        row = col + (size_t)nc * g.S2 * g.ncols;
+    }
+    LineArgs args(int n) const {
+        return LineArgs{g.S0,    g.S1, g.S2,        g.ncols,         g.nrows,    g.i0min,
+                        g.i1min, n,    g.col_start, g.row_col_start, g.row_i1lo, g.pw_z};
+    }
+    // sphere -> after the z transforms (fused, generic) or the z and axis-1 ones (lines)
+    jdft_status inverse(const c_t<T>* C, int ldc, int n, cudaStream_t st) {
+        const c_t<T>* tw = twiddles<T>(b);
+        if (!lines) return launch_zpass_inverse<T>(g, C, ldc, col, n, tw, st);
+        const LineArgs a = args(n);
+        jdft_status s = JDFT_LINE_DISPATCH(g.S2, LinePath<T, N>::zinv(a, C, ldc, col, tw, g.p2, st));
+        if (s != JDFT_OK) return s;
+        return JDFT_LINE_DISPATCH(g.S1, LinePath<T, N>::rows(a, +1, col, row, tw, g.p1, st));
+    }
+    jdft_status apply(int n, cudaStream_t st) {
+        const c_t<T>* tw = twiddles<T>(b);
+        if (!lines) return launch_plane_apply<T>(g, col, potential<T>(b), n, tw, st);
+        return JDFT_LINE_DISPATCH(g.S0, LinePath<T, N>::apply(args(n), row, potential_natural<T>(b), tw, g.p0, st));
+    }
+    jdft_status density(const double* f, double* n_r, int n, cudaStream_t st) {
+        const c_t<T>* tw = twiddles<T>(b);
+        if (!lines) return launch_plane_density<T>(g, col, f, b->kweight[ik], n_r, n, tw, st);
+        return JDFT_LINE_DISPATCH(g.S0,
+                                  LinePath<T, N>::density(args(n), row, f, b->kweight[ik], n_r, tw, g.p0, st));
+    }
+    jdft_status box_inverse(c_t<T>* psi, T scale, int n, cudaStream_t st) {
+        const c_t<T>* tw = twiddles<T>(b);
+        if (!lines) return launch_plane_inverse_full<T>(g, col, psi, scale, n, tw, st);
+        return JDFT_LINE_DISPATCH(g.S0, LinePath<T, N>::full(args(n), +1, row, psi, scale, tw, g.p0, st));
+    }
+    jdft_status box_forward(const c_t<T>* psi, int n, cudaStream_t st) {
+        const c_t<T>* tw = twiddles<T>(b);
+        if (!lines) return launch_plane_forward_full<T>(g, psi, col, n, tw, st);
+        return JDFT_LINE_DISPATCH(g.S0,
+                                  LinePath<T, N>::full(args(n), -1, row, const_cast<c_t<T>*>(psi), T(1), tw, g.p0, st));
+    }
+    // back to the sphere: out = omega (kin C + scale y), or scale y without kin
+    jdft_status forward(const c_t<T>* C, int ldc, c_t<T>* out, int ldo, const T* kin, T omega, T scale, int n,
+                        cudaStream_t st) {
+        const c_t<T>* tw = twiddles<T>(b);
+        if (!lines)
+            return kin ? launch_zpass_forward<T, 0>(g, col, C, ldc, out, ldo, n, kin, omega, scale, tw, st)
+                       : launch_zpass_forward<T, 1>(g, col, C, ldc, out, ldo, n, kin, omega, scale, tw, st);
+        const LineArgs a = args(n);
+        jdft_status s = JDFT_LINE_DISPATCH(g.S1, LinePath<T, N>::rows(a, -1, col, row, tw, g.p1, st));
+        if (s != JDFT_OK) return s;
+        return JDFT_LINE_DISPATCH(g.S2, LinePath<T, N>::zfwd(a, col, C, ldc, out, ldo, kin, omega, scale, tw, g.p2, st));
+    }
+};
+
 // psi = scale * I C
 template <typename T>
 static jdft_status run_inverse_full(jdft_basis_s* b, int ik, const void* C, int ldc, void* psi, int nb, T scale,
                                     cudaStream_t st) {
-    const ChainGeom g = make_geom(b, ik);
-    const int nc = chunk_bands(g, sizeof(c_t<T>), nb, chunk_budget(b));
-    jdft_status s = ensure_workspace(b, (size_t)nc * g.S2 * g.ncols * sizeof(c_t<T>));
+    BandChain<T> ch(b, ik, nb, ChainUse::kBox);
+    jdft_status s = ensure_workspace(b, ch.bytes);
     if (s != JDFT_OK) return s;
-    c_t<T>* colbuf = (c_t<T>*)b->work.ptr;
-    for (int b0 = 0; b0 < nb; b0 += nc) {
-        const int n = std::min(nc, nb - b0);
-        if ((s = launch_zpass_inverse<T>(g, (const c_t<T>*)C + (size_t)b0 * ldc, ldc, colbuf, n, twiddles<T>(b), st)))
-            return s;
-        if ((s = launch_plane_inverse_full<T>(g, colbuf, (c_t<T>*)psi + (size_t)b0 * b->N, scale, n, twiddles<T>(b),
-                                              st)))
-            return s;
+    ch.bind(b->work.ptr);
+    for (int b0 = 0; b0 < nb; b0 += ch.nc) {
+        const int n = std::min(ch.nc, nb - b0);
+        if ((s = ch.inverse((const c_t<T>*)C + (size_t)b0 * ldc, ldc, n, st))) return s;
+        if ((s = ch.box_inverse((c_t<T>*)psi + (size_t)b0 * b->N, scale, n, st))) return s;
     }
     return JDFT_OK;
 }
@@ -571,19 +672,14 @@ static jdft_status run_inverse_full(jdft_basis_s* b, int ik, const void* C, int 
 template <typename T>
 static jdft_status run_forward_full(jdft_basis_s* b, int ik, const void* psi, void* C, int ldc, int nb, T scale,
                                     cudaStream_t st) {
-    const ChainGeom g = make_geom(b, ik);
-    const int nc = chunk_bands(g, sizeof(c_t<T>), nb, chunk_budget(b));
-    jdft_status s = ensure_workspace(b, (size_t)nc * g.S2 * g.ncols * sizeof(c_t<T>));
+    BandChain<T> ch(b, ik, nb, ChainUse::kBox);
+    jdft_status s = ensure_workspace(b, ch.bytes);
     if (s != JDFT_OK) return s;
-    c_t<T>* colbuf = (c_t<T>*)b->work.ptr;
-    for (int b0 = 0; b0 < nb; b0 += nc) {
-        const int n = std::min(nc, nb - b0);
-        if ((s = launch_plane_forward_full<T>(g, (const c_t<T>*)psi + (size_t)b0 * b->N, colbuf, n, twiddles<T>(b),
-                                              st)))
-            return s;
-        if ((s = launch_zpass_forward<T, 1>(g, colbuf, nullptr, 0, (c_t<T>*)C + (size_t)b0 * ldc, ldc, n, nullptr,
-                                            T(0), scale, twiddles<T>(b), st)))
-            return s;
+    ch.bind(b->work.ptr);
+    for (int b0 = 0; b0 < nb; b0 += ch.nc) {
+        const int n = std::min(ch.nc, nb - b0);
+        if ((s = ch.box_forward((const c_t<T>*)psi + (size_t)b0 * b->N, n, st))) return s;
+        if ((s = ch.forward(nullptr, 0, (c_t<T>*)C + (size_t)b0 * ldc, ldc, nullptr, T(0), scale, n, st))) return s;
     }
     return JDFT_OK;
 }
@@ -591,41 +687,35 @@ static jdft_status run_forward_full(jdft_basis_s* b, int ik, const void* psi, vo
 template <typename T>
 static jdft_status run_apply_H(jdft_basis_s* b, int ik, const void* C, int ldc, void* HC, int ldhc, int nb,
                                jdft_prec prec, cudaStream_t st) {
-    const ChainGeom g = make_geom(b, ik);
+    BandChain<T> ch(b, ik, nb, ChainUse::kH);
     const KSphere& sp = b->ks[ik];
-    const int nc = chunk_bands(g, sizeof(c_t<T>), nb, chunk_budget(b));
-    const size_t colbytes = ((size_t)nc * g.S2 * g.ncols * sizeof(c_t<T>) + 255) / 256 * 256;
     const size_t nlbytes = nonlocal_workspace_bytes(sp.nproj, nb, sizeof(c_t<T>), sp.npw, prec, true, true);
-    jdft_status s = ensure_workspace(b, colbytes + nlbytes);
+    jdft_status s = ensure_workspace(b, ch.bytes + nlbytes);
     if (s != JDFT_OK) return s;
-    c_t<T>* colbuf = (c_t<T>*)b->work.ptr;
+    ch.bind(b->work.ptr);
     const T omega = (T)b->omega, invN = (T)(1.0 / (double)b->N);
-    for (int b0 = 0; b0 < nb; b0 += nc) {
-        const int n = std::min(nc, nb - b0);
+    for (int b0 = 0; b0 < nb; b0 += ch.nc) {
+        const int n = std::min(ch.nc, nb - b0);
         const c_t<T>* Cc = (const c_t<T>*)C + (size_t)b0 * ldc;
         c_t<T>* Hc = (c_t<T>*)HC + (size_t)b0 * ldhc;
-        if ((s = launch_zpass_inverse<T>(g, Cc, ldc, colbuf, n, twiddles<T>(b), st))) return s;
-        if ((s = launch_plane_apply<T>(g, colbuf, potential<T>(b), n, twiddles<T>(b), st))) return s;
-        if ((s = launch_zpass_forward<T, 0>(g, colbuf, Cc, ldc, Hc, ldhc, n, kinetic<T>(sp), omega, invN,
-                                            twiddles<T>(b), st)))
-            return s;
+        if ((s = ch.inverse(Cc, ldc, n, st))) return s;
+        if ((s = ch.apply(n, st))) return s;
+        if ((s = ch.forward(Cc, ldc, Hc, ldhc, kinetic<T>(sp), omega, invN, n, st))) return s;
     }
     if (sp.nproj > 0)
-        return nonlocal_accumulate<T>(sp, C, ldc, HC, ldhc, nb, prec, (char*)b->work.ptr + colbytes, st, true, nullptr,
+        return nonlocal_accumulate<T>(sp, C, ldc, HC, ldhc, nb, prec, (char*)b->work.ptr + ch.bytes, st, true, nullptr,
                                       true, &b->prodwork);
     return JDFT_OK;
 }
 
-// H C and the density of the same block: per chunk one z pass in, then the
-// fused plane kernel where it exists (else density, then the H plane pass, on
-// the same column buffer), one z pass out; the nonlocal term after.
+// H C and the density of the same block: per chunk one pass in, then the fused
+// plane kernel where it exists (else density, then the H pass, on the same
+// intermediates), one pass out; the nonlocal term after.
 template <typename T>
 static size_t apply_H_density_bytes(const jdft_basis_s* b, int ik, int nb, jdft_prec prec, bool split_c) {
-    const ChainGeom g = make_geom(b, ik);
     const KSphere& sp = b->ks[ik];
-    const int nc = chunk_bands(g, sizeof(c_t<T>), nb, chunk_budget(b));
-    const size_t colbytes = ((size_t)nc * g.S2 * g.ncols * sizeof(c_t<T>) + 255) / 256 * 256;
-    return colbytes + nonlocal_workspace_bytes(sp.nproj, nb, sizeof(c_t<T>), sp.npw, prec, split_c, true);
+    return BandChain<T>(b, ik, nb, ChainUse::kHDensity).bytes +
+           nonlocal_workspace_bytes(sp.nproj, nb, sizeof(c_t<T>), sp.npw, prec, split_c, true);
 }
 
 // Csplit: the BF16 planes of C (tcx_split) when the caller has them, so the
@@ -634,41 +724,39 @@ template <typename T>
 static jdft_status run_apply_H_density(jdft_basis_s* b, int ik, const void* C, int ldc, void* HC, int ldhc, int nb,
                                        const double* f, double* n_r, jdft_prec prec, cudaStream_t st,
                                        const void* Csplit = nullptr) {
-    const ChainGeom g = make_geom(b, ik);
+    BandChain<T> ch(b, ik, nb, ChainUse::kHDensity);
     const KSphere& sp = b->ks[ik];
-    const int nc = chunk_bands(g, sizeof(c_t<T>), nb, chunk_budget(b));
-    const size_t colbytes = ((size_t)nc * g.S2 * g.ncols * sizeof(c_t<T>) + 255) / 256 * 256;
     const size_t nlbytes = nonlocal_workspace_bytes(sp.nproj, nb, sizeof(c_t<T>), sp.npw, prec, !Csplit, true);
-    jdft_status s = ensure_workspace(b, colbytes + nlbytes);
+    jdft_status s = ensure_workspace(b, ch.bytes + nlbytes);
     if (s != JDFT_OK) return s;
-    c_t<T>* colbuf = (c_t<T>*)b->work.ptr;
+    ch.bind(b->work.ptr);
     const T omega = (T)b->omega, invN = (T)(1.0 / (double)b->N);
-    const double wk = b->kweight[ik];
-    for (int b0 = 0; b0 < nb; b0 += nc) {
-        const int n = std::min(nc, nb - b0);
+    for (int b0 = 0; b0 < nb; b0 += ch.nc) {
+        const int n = std::min(ch.nc, nb - b0);
         const c_t<T>* Cc = (const c_t<T>*)C + (size_t)b0 * ldc;
         c_t<T>* Hc = (c_t<T>*)HC + (size_t)b0 * ldhc;
-        if ((s = launch_zpass_inverse<T>(g, Cc, ldc, colbuf, n, twiddles<T>(b), st))) return s;
+        if ((s = ch.inverse(Cc, ldc, n, st))) return s;
         jdft_status fs = JDFT_ERR_UNSUPPORTED;
         if constexpr (std::is_same<T, float>::value) {
-            fs = launch_plane_apply_density_pair(g, colbuf, potential<float>(b), n, f + b0, wk, n_r, twiddles<float>(b),
-                                                 st);
-            if (fs == JDFT_ERR_UNSUPPORTED)
-                fs = launch_plane_apply_density_fast(g, colbuf, potential<float>(b), n, f + b0, wk, n_r,
+            if (!ch.lines) {
+                const double wk = b->kweight[ik];
+                fs = launch_plane_apply_density_pair(ch.g, ch.col, potential<float>(b), n, f + b0, wk, n_r,
                                                      twiddles<float>(b), st);
+                if (fs == JDFT_ERR_UNSUPPORTED)
+                    fs = launch_plane_apply_density_fast(ch.g, ch.col, potential<float>(b), n, f + b0, wk, n_r,
+                                                         twiddles<float>(b), st);
+            }
         }
         if (fs == JDFT_ERR_UNSUPPORTED) {
-            if ((s = launch_plane_density<T>(g, colbuf, f + b0, wk, n_r, n, twiddles<T>(b), st))) return s;
-            if ((s = launch_plane_apply<T>(g, colbuf, potential<T>(b), n, twiddles<T>(b), st))) return s;
+            if ((s = ch.density(f + b0, n_r, n, st))) return s;
+            if ((s = ch.apply(n, st))) return s;
         } else if (fs != JDFT_OK) {
             return fs;
         }
-        if ((s = launch_zpass_forward<T, 0>(g, colbuf, Cc, ldc, Hc, ldhc, n, kinetic<T>(sp), omega, invN,
-                                            twiddles<T>(b), st)))
-            return s;
+        if ((s = ch.forward(Cc, ldc, Hc, ldhc, kinetic<T>(sp), omega, invN, n, st))) return s;
     }
     if (sp.nproj > 0)
-        return nonlocal_accumulate<T>(sp, C, ldc, HC, ldhc, nb, prec, (char*)b->work.ptr + colbytes, st, !Csplit,
+        return nonlocal_accumulate<T>(sp, C, ldc, HC, ldhc, nb, prec, (char*)b->work.ptr + ch.bytes, st, !Csplit,
                                       Csplit, true, &b->prodwork);
     return JDFT_OK;
 }
@@ -688,16 +776,14 @@ jdft_status apply_H_density_with_split(jdft_basis_s* b, int ik, const void* C, i
 template <typename T>
 static jdft_status run_density(jdft_basis_s* b, int ik, const void* C, int ldc, const double* f, int nb,
                                double* n_r, cudaStream_t st) {
-    const ChainGeom g = make_geom(b, ik);
-    const int nc = chunk_bands(g, sizeof(c_t<T>), nb, chunk_budget(b));
-    jdft_status s = ensure_workspace(b, (size_t)nc * g.S2 * g.ncols * sizeof(c_t<T>));
+    BandChain<T> ch(b, ik, nb, ChainUse::kDensity);
+    jdft_status s = ensure_workspace(b, ch.bytes);
     if (s != JDFT_OK) return s;
-    c_t<T>* colbuf = (c_t<T>*)b->work.ptr;
-    for (int b0 = 0; b0 < nb; b0 += nc) {
-        const int n = std::min(nc, nb - b0);
-        if ((s = launch_zpass_inverse<T>(g, (const c_t<T>*)C + (size_t)b0 * ldc, ldc, colbuf, n, twiddles<T>(b), st)))
-            return s;
-        if ((s = launch_plane_density<T>(g, colbuf, f + b0, b->kweight[ik], n_r, n, twiddles<T>(b), st))) return s;
+    ch.bind(b->work.ptr);
+    for (int b0 = 0; b0 < nb; b0 += ch.nc) {
+        const int n = std::min(ch.nc, nb - b0);
+        if ((s = ch.inverse((const c_t<T>*)C + (size_t)b0 * ldc, ldc, n, st))) return s;
+        if ((s = ch.density(f + b0, n_r, n, st))) return s;
     }
     return JDFT_OK;
 }

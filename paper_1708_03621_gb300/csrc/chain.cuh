@@ -136,6 +136,15 @@ jdft_status launch_zpass_forward_fast(const ChainGeom& g, const c_t<T>* colbuf, 
                                       int ldo, int nb, const T* kin, T omega, T scale, const c_t<T>* tw2,
                                       cudaStream_t st);
 
+// Whether a register-FFT plane kernel of type T serves the box's planes at this
+// sphere, and whether the z length has a register z pass.
+template <typename T>
+bool plane_apply_fused(const ChainGeom& g);
+bool zpass_fused(int S2);
+// Whether the line-transform chain (line_path.cuh) serves this box: all three edges
+// are compiled line lengths.
+bool lines_serve(const jdft_basis_s* b);
+
 template <typename T>
 jdft_status launch_plane_density(const ChainGeom& g, const c_t<T>* colbuf, const double* f, double w, double* n_r,
                                  int nb, const c_t<T>* tw_base, cudaStream_t st);

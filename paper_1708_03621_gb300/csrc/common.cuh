@@ -161,6 +161,9 @@ struct jdft_basis_s {
     // local potential, permuted for the plane pass: Vp[(j2 * S1 + j1) * S0 + j0]
     double* V = nullptr;
     float* V32 = nullptr;
+    // the same in natural order (j2 fastest), for boxes the line-transform chain serves
+    double* Vn = nullptr;
+    float* Vn32 = nullptr;
     bool have_V = false;
     int device = 0;
     int chunk_mb = 0;         // band-chunk budget chosen by jdft_autotune_chunk (0 = default)

@@ -58,6 +58,10 @@ constexpr i64 kFixC51 = 1425089352415399811ll;   // cos(2 pi/5)
 constexpr i64 kFixC52 = -3730932361629093763ll;  // cos(4 pi/5)
 constexpr i64 kFixS51 = 4385974038932618941ll;   // sin(2 pi/5)
 constexpr i64 kFixS52 = 2710681029835013083ll;   // sin(4 pi/5)
+// cos and sin of 2 pi k/9, k = 1, 2, 4
+constexpr i64 kFixC91 = 3532756447825785444ll, kFixS91 = 2964334632409774423ll;
+constexpr i64 kFixC92 = 800810873071977681ll, kFixS92 = 4541624145405292212ll;
+constexpr i64 kFixC94 = -4333567320897763126ll, kFixS94 = 1577289512995517789ll;
 
 // x = h 2^32 + l with both words signed.
 __device__ __forceinline__ void fix_words(i64 x, int& h, int& l) {
@@ -134,6 +138,17 @@ template <int SIGN>
 __device__ __forceinline__ longlong2 rot135_fix(longlong2 a) {
     constexpr FixW h = fix_split(kFixH);
     return make_longlong2(fix_mul(-a.x - SIGN * a.y, h), fix_mul(SIGN * a.x - a.y, h));
+}
+
+// W9^k, k = 1, 2, 4
+template <int SIGN>
+__device__ __forceinline__ longlong2 rot9_fix(longlong2 a, int k) {
+    constexpr FixW c1 = fix_split(kFixC91), s1 = fix_split(SIGN * kFixS91), c2 = fix_split(kFixC92),
+                   s2 = fix_split(SIGN * kFixS92), c4 = fix_split(kFixC94), s4 = fix_split(SIGN * kFixS94);
+    if (k == 0) return a;
+    if (k == 1) return cmul(a, make_int4(c1.h, c1.l, s1.h, s1.l));
+    if (k == 2) return cmul(a, make_int4(c2.h, c2.l, s2.h, s2.l));
+    return cmul(a, make_int4(c4.h, c4.l, s4.h, s4.l));
 }
 
 template <int SIGN>
@@ -237,14 +252,50 @@ __device__ __forceinline__ double fix_decode(i64 x, int q) {
     return __hiloint2double(hi | (s & 0x80000000), (int)r);
 }
 
-// E values per lane of lines of TL lanes (lane l belongs to line l mod (32 / TL)): v becomes integers.
+// Maximum and sum over the TL lanes of a line (lane l belongs to line l mod LPW,
+// LPW = 32 / TL; lanes past TL LPW belong to none).
+template <int TL>
+__device__ __forceinline__ int line_max(int x) {
+    constexpr int LPW = 32 / TL;
+    if constexpr ((TL & (TL - 1)) == 0) {
+#pragma unroll
+        for (int m = LPW; m < 32; m <<= 1) x = max(x, __shfl_xor_sync(0xffffffffu, x, m));
+        return x;
+    } else {
+        const int lane = threadIdx.x & 31;
+        int r = x;
+#pragma unroll
+        for (int i = 1; i < TL; ++i) {
+            const int s = lane + i * LPW;
+            r = max(r, __shfl_sync(0xffffffffu, x, s < TL * LPW ? s : s - TL * LPW));
+        }
+        return r;
+    }
+}
+template <int TL>
+__device__ __forceinline__ float line_sum(float x) {
+    constexpr int LPW = 32 / TL;
+    if constexpr ((TL & (TL - 1)) == 0) {
+#pragma unroll
+        for (int m = LPW; m < 32; m <<= 1) x += __shfl_xor_sync(0xffffffffu, x, m);
+        return x;
+    } else {
+        // every lane adds in the same order (from the line's first lane), so all lanes get the same scale
+        const int line = (threadIdx.x & 31) % LPW;
+        float r = 0.f;
+#pragma unroll
+        for (int i = 0; i < TL; ++i) r += __shfl_sync(0xffffffffu, x, line + i * LPW);
+        return r;
+    }
+}
+
+// E values per lane of lines of TL lanes: v becomes integers.
 template <int E, int TL>
 __device__ __forceinline__ FixScale fix_line_in(const double2* v, longlong2* x) {
     int amax = 0;
 #pragma unroll
     for (int e = 0; e < E; ++e) amax = max(amax, max(fix_abs_hi(v[e].x), fix_abs_hi(v[e].y)));
-#pragma unroll
-    for (int m = 32 / TL; m < 32; m <<= 1) amax = max(amax, __shfl_xor_sync(0xffffffffu, amax, m));
+    amax = line_max<TL>(amax);
     int emax = amax >> 20;
     const bool bad = emax == 0x7ff;
     int up = 0;
@@ -262,8 +313,7 @@ __device__ __forceinline__ FixScale fix_line_in(const double2* v, longlong2* x) 
             w[e].y *= f;
             amax = max(amax, max(fix_abs_hi(w[e].x), fix_abs_hi(w[e].y)));
         }
-#pragma unroll
-        for (int m = 32 / TL; m < 32; m <<= 1) amax = max(amax, __shfl_xor_sync(0xffffffffu, amax, m));
+        amax = line_max<TL>(amax);
         emax = amax >> 20;
     }
     emax = max(emax, 64);  // all-zero lines
@@ -271,8 +321,7 @@ __device__ __forceinline__ FixScale fix_line_in(const double2* v, longlong2* x) 
     float s = 1e-30f;
 #pragma unroll
     for (int e = 0; e < E; ++e) s += fix_relative(w[e].x, bias) + fix_relative(w[e].y, bias);
-#pragma unroll
-    for (int m = 32 / TL; m < 32; m <<= 1) s += __shfl_xor_sync(0xffffffffu, s, m);
+    s = line_sum<TL>(s);
     // L1 < 2^(es + 1) 2^(emax - 1023), with a margin for the truncated terms and the float sum
     const int es = max((__float_as_int(s * 1.0001f) >> 23) - 127, 0);
     // x = 1.f 2^(ex - 1023) becomes 1.f 2^(59 - es - (emax - ex)): L1 < 2^60 units

@@ -793,6 +793,25 @@ jdft_status launch_plane_apply_fast(const ChainGeom& g, c_t<T>* colbuf, const T*
     return JDFT_ERR_UNSUPPORTED;
 }
 
+template <typename T>
+bool plane_apply_fused(const ChainGeom& g) {
+#define JDFT_CASE(a, b) \
+    if (g.S0 == a && g.S1 == b) return fast_smem<T, a, b>(g, PlaneBlock<T, a, b>::warps) <= kFastMaxSmem;
+    JDFT_FAST_SHAPES(JDFT_CASE)
+#undef JDFT_CASE
+    return false;
+}
+template bool plane_apply_fused<double>(const ChainGeom&);
+template bool plane_apply_fused<float>(const ChainGeom&);
+
+bool zpass_fused(int S2) {
+#define JDFT_CASE(a) \
+    if (S2 == a) return true;
+    JDFT_FAST_LENGTHS(JDFT_CASE)
+#undef JDFT_CASE
+    return false;
+}
+
 jdft_status launch_plane_density_fast(const ChainGeom& g, const float2* colbuf, const double* f, double w,
                                       double* n_r, int nb, const float2* tw_base, cudaStream_t st) {
     if (fast_disabled()) return JDFT_ERR_UNSUPPORTED;
