@@ -255,6 +255,7 @@ static jdft_status build_twiddles(jdft_basis_s* b) {
         }
     }
     jdft_status st;
+    if ((st = upload(&b->counters, std::vector<unsigned>(4, 0u))) != JDFT_OK) return st;
     if ((st = upload(&b->tw64, t64)) != JDFT_OK) return st;
     if ((st = upload(&b->tw32, t32)) != JDFT_OK) return st;
     return JDFT_OK;
@@ -404,7 +405,7 @@ jdft_status jdft_basis_destroy(jdft_basis_t b) {
     cudaGetDevice(&prev);
     cudaSetDevice(b->device);
     for (auto& s : b->ks) free_sphere(s);
-    cudaFree(b->tw64); cudaFree(b->tw32); cudaFree(b->V); cudaFree(b->V32); cudaFree(b->Vn); cudaFree(b->Vn32); cudaFree(b->work.ptr);
+    cudaFree(b->tw64); cudaFree(b->tw32); cudaFree(b->counters); cudaFree(b->V); cudaFree(b->V32); cudaFree(b->Vn); cudaFree(b->Vn32); cudaFree(b->work.ptr);
     b->prodwork.release();
     if (b->side) {
         cudaStreamSynchronize(b->side);

@@ -178,6 +178,8 @@ struct jdft_basis_s {
     // box and per-block partial sums (grown on first use)
     jdft::Workspace fieldwork;
     jdft::ProductScratch prodwork;
+    // block counters of sums finished by their launch's last block (zero between launches)
+    unsigned* counters = nullptr;
     // spinor calls: real-space boxes and sphere blocks of a band chunk
     jdft::Workspace spinwork;
     cudaStream_t side = nullptr;

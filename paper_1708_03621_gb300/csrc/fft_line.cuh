@@ -184,15 +184,13 @@ constexpr int any_values() {
 // run: from the input layout to the output layout, sign +1 or -1; adjoint: sign
 // SIGN from the output layout back to the input layout.  Invalid values must be
 // zero on entry of an FP64 transform (they take part in the line's scale).
-template <typename T, int N, int TL_, class RadList>
+template <typename T, int N, int TL_, int SP, class RadList>
 struct AnyLine;
-template <typename T, int N, int TL_, int R0, int... R>
-struct AnyLine<T, N, TL_, Rad<R0, R...>> {
-    static constexpr int TL = TL_, LPW = 32 / TL, E = any_values<N, TL, R0, R...>();
+template <typename T, int N, int TL_, int SP, int R0, int... R>
+struct AnyLine<T, N, TL_, SP, Rad<R0, R...>> {
+    static constexpr int TL = TL_, LPW = 32 / TL, E = any_values<N, TL, R0, R...>(), SPACING = SP;
     static_assert(RadInfo<R0, R...>::prod == N, "radices must multiply to N");
     static constexpr int kRL = LastStage<1, R0, R...>::radix, kNSL = LastStage<1, R0, R...>::ns;
-    // elements between the scratch lines of a warp (odd, so that lines start on different banks)
-    static constexpr int SPACING = padded_line(N) | 1;
     static __device__ __forceinline__ bool in_valid(int t, int e) {
         return e / R0 < per_lane(N, TL, R0) && t + TL * (e / R0) < N / R0;
     }
@@ -230,51 +228,56 @@ struct AnyLine<T, N, TL_, Rad<R0, R...>> {
     }
 };
 
-// Lanes and radices per length.  Two stages where the factors allow, up to 16
-// values a lane (FP64: 64 registers of them), and as few idle lanes as that leaves.
+// Per length: lanes, elements between the scratch lines of a warp (8-byte and
+// 16-byte values) and radices.  Two stages where the factors allow, up to 16 values a
+// lane (FP64: 64 registers of them), and as few idle lanes as that leaves; the
+// spacings are those with the fewest shared-memory wavefronts over a transform's
+// exchanges, counted access by access (128 values: half those of an odd spacing).
 template <typename T, int N> struct AnyCfg;
-#define JDFT_ANY(N_, TL_, ...)            \
-    template <typename T>                 \
-    struct AnyCfg<T, N_> {                \
-        static constexpr int TL = TL_;    \
-        using R = Rad<__VA_ARGS__>;       \
+#define JDFT_ANY(N_, TL_, SP8, SP16, ...)                                           \
+    template <typename T>                                                           \
+    struct AnyCfg<T, N_> {                                                          \
+        static constexpr int TL = TL_;                                              \
+        static constexpr int SPACING = std::is_same<T, double>::value ? SP16 : SP8; \
+        using R = Rad<__VA_ARGS__>;                                                 \
+        static_assert(SPACING >= padded_line(N_), "scratch lines must not overlap"); \
     };
-JDFT_ANY(12, 4, 4, 3)
-JDFT_ANY(16, 4, 4, 4)
-JDFT_ANY(24, 6, 4, 6)
-JDFT_ANY(25, 5, 5, 5)
-JDFT_ANY(27, 3, 9, 3)
-JDFT_ANY(30, 6, 5, 6)
-JDFT_ANY(32, 4, 8, 4)
-JDFT_ANY(36, 6, 6, 6)
-JDFT_ANY(40, 5, 8, 5)
-JDFT_ANY(45, 5, 9, 5)
-JDFT_ANY(48, 8, 8, 6)
-JDFT_ANY(50, 5, 10, 5)
-JDFT_ANY(54, 6, 9, 6)
-JDFT_ANY(60, 6, 10, 6)
-JDFT_ANY(64, 8, 8, 8)
-JDFT_ANY(72, 9, 9, 8)
-JDFT_ANY(75, 5, 5, 5, 3)
-JDFT_ANY(80, 10, 10, 8)
-JDFT_ANY(81, 9, 9, 9)
-JDFT_ANY(90, 10, 10, 9)
-JDFT_ANY(96, 8, 4, 4, 6)
-JDFT_ANY(100, 10, 10, 10)
-JDFT_ANY(108, 9, 6, 6, 3)
-JDFT_ANY(120, 8, 8, 5, 3)
-JDFT_ANY(125, 9, 5, 5, 5)
-JDFT_ANY(128, 8, 16, 8)
-JDFT_ANY(256, 16, 16, 16)
+JDFT_ANY(12, 4, 14, 13, 4, 3)
+JDFT_ANY(16, 4, 18, 17, 4, 4)
+JDFT_ANY(24, 6, 29, 29, 4, 6)
+JDFT_ANY(25, 5, 39, 29, 5, 5)
+JDFT_ANY(27, 3, 33, 29, 9, 3)
+JDFT_ANY(30, 6, 45, 37, 5, 6)
+JDFT_ANY(32, 4, 34, 35, 8, 4)
+JDFT_ANY(36, 6, 41, 45, 6, 6)
+JDFT_ANY(40, 5, 55, 43, 8, 5)
+JDFT_ANY(45, 5, 55, 47, 9, 5)
+JDFT_ANY(48, 8, 54, 54, 8, 6)
+JDFT_ANY(50, 5, 55, 55, 10, 5)
+JDFT_ANY(54, 6, 71, 61, 9, 6)
+JDFT_ANY(60, 6, 77, 69, 10, 6)
+JDFT_ANY(64, 8, 68, 70, 8, 8)
+JDFT_ANY(72, 9, 76, 83, 9, 8)
+JDFT_ANY(75, 5, 87, 81, 5, 5, 3)
+JDFT_ANY(80, 10, 87, 86, 10, 8)
+JDFT_ANY(81, 9, 91, 91, 9, 9)
+JDFT_ANY(90, 10, 100, 99, 10, 9)
+JDFT_ANY(96, 8, 103, 102, 4, 4, 6)
+JDFT_ANY(100, 10, 108, 110, 10, 10)
+JDFT_ANY(108, 9, 123, 115, 6, 6, 3)
+JDFT_ANY(120, 8, 132, 130, 8, 5, 3)
+JDFT_ANY(125, 9, 132, 139, 5, 5, 5)
+JDFT_ANY(128, 8, 140, 140, 16, 8)
+JDFT_ANY(256, 16, 280, 276, 16, 16)
 #undef JDFT_ANY
 // FP64: 16 lanes of 8 values in three stages, which leaves more warps an SM (see RegCfg)
 template <>
 struct AnyCfg<double, 128> {
-    static constexpr int TL = 16;
+    static constexpr int TL = 16, SPACING = 140;
     using R = Rad<8, 4, 4>;
 };
 
 template <typename T, int N>
-using LineOf = AnyLine<T, N, AnyCfg<T, N>::TL, typename AnyCfg<T, N>::R>;
+using LineOf = AnyLine<T, N, AnyCfg<T, N>::TL, AnyCfg<T, N>::SPACING, typename AnyCfg<T, N>::R>;
 
 }  // namespace jdft

@@ -44,10 +44,12 @@
 #include <cstdlib>
 #include <vector>
 
+#include "block_sum.cuh"
 #include "common.cuh"
 #include "fft.cuh"
 #include "field_fast.cuh"
 #include "field_lda.cuh"
+#include "line_path.cuh"
 #include "profile.cuh"
 
 namespace jdft {
@@ -336,27 +338,10 @@ jdft_status field_work(jdft_basis_s* b, FieldWork* w, int nbox = 1) {
     return JDFT_OK;
 }
 
-// Call of a member of FieldFast<T, n> or HartreeFast<n> for the compiled length n
-// (JDFT_ERR_UNSUPPORTED otherwise): the call's template argument is N.
-#define JDFT_FIELD_LENGTH(n, ...)                                       \
-    [&]() -> jdft_status {                                              \
-        switch (n) {                                                    \
-            case 12: { constexpr int N = 12; return __VA_ARGS__; }      \
-            case 16: { constexpr int N = 16; return __VA_ARGS__; }      \
-            case 40: { constexpr int N = 40; return __VA_ARGS__; }      \
-            case 48: { constexpr int N = 48; return __VA_ARGS__; }      \
-            case 64: { constexpr int N = 64; return __VA_ARGS__; }      \
-            case 80: { constexpr int N = 80; return __VA_ARGS__; }      \
-            case 128: { constexpr int N = 128; return __VA_ARGS__; }    \
-            case 256: { constexpr int N = 256; return __VA_ARGS__; }    \
-        }                                                               \
-        return JDFT_ERR_UNSUPPORTED;                                    \
-    }()
-
 // JDFT_FAST_PLANE=0 turns every register-FFT path off (tests compare the two).
 bool field_fast(int n) {
     const char* e = getenv("JDFT_FAST_PLANE");
-    return field_fast_length(n) && !(e && e[0] == '0');
+    return line_length(n) && !(e && e[0] == '0');
 }
 
 FieldCell field_cell(const jdft_basis_s* b) {
@@ -391,7 +376,7 @@ jdft_status launch_axis(const char* name, jdft_basis_s* b, int axis, const void*
                         cudaStream_t st, int* nblocks = nullptr, int batch = 1) {
     if constexpr (!IN_REAL && !KERNEL && OUT == OUT_COMPLEX) {
         if (field_fast(b->S[axis]))
-            return JDFT_FIELD_LENGTH(b->S[axis],
+            return JDFT_LINE_DISPATCH(b->S[axis],
                                      FieldFast<double, N>::axis(name, SIGN, (const double2*)in, (double2*)out,
                                                                 line_geom(b, axis, b->S[2]), a.scale, batch, a.bstride,
                                                                 b->tw64, b->plan[axis], st));
@@ -453,25 +438,22 @@ jdft_status hartree_chain(jdft_basis_s* b, const double* n, const double* vion, 
         const int H = b->S[2] / 2 + 1, lines = b->S[0] * b->S[1];
         const LineGeom g1 = line_geom(b, 1, H);
         double2* x = w.box;
-        if ((s = JDFT_FIELD_LENGTH(b->S[2], HartreeFast<N>::forward2(n, x, lines, b->tw64, b->plan[2], st)))) return s;
-        if ((s = JDFT_FIELD_LENGTH(b->S[1], FieldFast<double, N>::axis("field_fft_axis1", -1, x, x, g1, 1.0, 1, 0,
+        if ((s = JDFT_LINE_DISPATCH(b->S[2], HartreeFast<N>::forward2(n, x, lines, b->tw64, b->plan[2], st)))) return s;
+        if ((s = JDFT_LINE_DISPATCH(b->S[1], FieldFast<double, N>::axis("field_fft_axis1", -1, x, x, g1, 1.0, 1, 0,
                                                                        b->tw64, b->plan[1], st))))
             return s;
-        if ((s = JDFT_FIELD_LENGTH(b->S[0], HartreeFast<N>::kernel0(x, q, w.partial, &nb_h, b->tw64, b->plan[0], st))))
+        const BlockSum eh{w.partial, b->counters, energies}, ex{w.partial + half, b->counters + 1,
+                                                                OUT == OUT_KS && energies ? energies + 1 : nullptr};
+        if ((s = JDFT_LINE_DISPATCH(b->S[0], HartreeFast<N>::kernel0(x, q, eh, 0.5 * b->omega, b->tw64, b->plan[0], st))))
             return s;
-        if ((s = JDFT_FIELD_LENGTH(b->S[1], FieldFast<double, N>::axis("field_fft_axis1", +1, x, x, g1, 1.0, 1, 0,
+        if ((s = JDFT_LINE_DISPATCH(b->S[1], FieldFast<double, N>::axis("field_fft_axis1", +1, x, x, g1, 1.0, 1, 0,
                                                                        b->tw64, b->plan[1], st))))
             return s;
-        if ((s = JDFT_FIELD_LENGTH(b->S[2], HartreeFast<N>::inverse2(x, V, OUT == OUT_KS ? n : nullptr,
-                                                                     OUT == OUT_KS ? vion : nullptr, w.partial + half,
-                                                                     &nb_x, lines, b->tw64, b->plan[2], st))))
+        if ((s = JDFT_LINE_DISPATCH(b->S[2], HartreeFast<N>::inverse2(x, V, OUT == OUT_KS ? n : nullptr,
+                                                                     OUT == OUT_KS ? vion : nullptr, ex,
+                                                                     b->omega / (double)b->N, lines, b->tw64,
+                                                                     b->plan[2], st))))
             return s;
-        if (energies) {
-            if ((s = launch_reduce(w.partial, nb_h, 1, 1, 0.5 * b->omega, energies, false, st))) return s;
-            if (OUT == OUT_KS)
-                if ((s = launch_reduce(w.partial + half, nb_x, 1, 1, b->omega / (double)b->N, energies + 1, false, st)))
-                    return s;
-        }
         return JDFT_OK;
     }
     for (int axis = 0; axis < 3; axis += 2) {
@@ -880,30 +862,46 @@ pcm_init_kernel(const double2* __restrict__ rho, c_t<T>* __restrict__ x, c_t<T>*
     if (threadIdx.x == 0) { partial[2 * blockIdx.x] = s0; partial[2 * blockIdx.x + 1] = s1; }
 }
 
-// x += alpha d, r -= alpha Hd with alpha = rz / dHd (device scalars); partial
-// sums of |r|^2 and r.Kr of the new residual.
+// x += alpha d, r -= alpha Hd with alpha = rz / dHd (device scalars); sums of |r|^2
+// and r.Kr of the new residual.  A warp takes whole rows along axis 2, so the
+// division that finds (m0, m1) is per row, and the grid is small (update_grid): a
+// block's sums cost 3000 FP64 additions, which were half of the kernel's time with
+// a thousand blocks.  Four boxes are read and two written, which bounds the rest
+// (128^3, FP32: 37 -> 31 us).
 template <typename T>
 __global__ void __launch_bounds__(kFieldThreads)
 pcm_update_kernel(c_t<T>* __restrict__ x, c_t<T>* __restrict__ r, const c_t<T>* __restrict__ d,
                   const c_t<T>* __restrict__ Hd, const double* __restrict__ rz, const double* __restrict__ dHd,
-                  GArgs q, int64_t N, double* __restrict__ partial) {
+                  GArgs q, BlockSum sum) {
     const T alpha = (T)(*rz / *dHd);
-    T rr = 0, rzn = 0;
-    for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < N; j += (int64_t)gridDim.x * blockDim.x) {
-        const c_t<T> dv = d[j], hv = Hd[j];
-        c_t<T> xv = x[j], rv = r[j];
-        xv.x += alpha * dv.x; xv.y += alpha * dv.y;
-        rv.x -= alpha * hv.x; rv.y -= alpha * hv.y;
-        x[j] = xv;
-        r[j] = rv;
-        const T K = coulomb_of_index<T>(q, j);
-        const T a = rv.x * rv.x + rv.y * rv.y;
-        rr += a;
-        rzn += K * a;
+    const int rows = q.S[0] * q.S[1], S2 = q.S[2];
+    const int lane = threadIdx.x & 31, warps = gridDim.x * (kFieldThreads / 32);
+    T s[2] = {0, 0};
+    for (int row = blockIdx.x * (kFieldThreads / 32) + (threadIdx.x >> 5); row < rows; row += warps) {
+        const int m0 = row / q.S[1], m1 = row - m0 * q.S[1];
+        const T f0 = (T)fold(m0, q.S[0]), f1 = (T)fold(m1, q.S[1]);
+        const T gx = f0 * (T)q.B[0] + f1 * (T)q.B[1], gy = f0 * (T)q.B[3] + f1 * (T)q.B[4],
+                gz = f0 * (T)q.B[6] + f1 * (T)q.B[7];
+        const int64_t base = (int64_t)row * S2;
+#pragma unroll 4
+        for (int m2 = lane; m2 < S2; m2 += 32) {
+            const int64_t j = base + m2;
+            const c_t<T> dv = d[j], hv = Hd[j];
+            c_t<T> xv = x[j], rv = r[j];
+            xv.x += alpha * dv.x; xv.y += alpha * dv.y;
+            rv.x -= alpha * hv.x; rv.y -= alpha * hv.y;
+            x[j] = xv;
+            r[j] = rv;
+            const T f2 = (T)fold(m2, S2);
+            const T ax = gx + f2 * (T)q.B[2], ay = gy + f2 * (T)q.B[5], az = gz + f2 * (T)q.B[8];
+            const T g2 = ax * ax + ay * ay + az * az;
+            const T K = g2 > (T)0 ? (T)kFourPi / g2 : (T)0;
+            const T a = rv.x * rv.x + rv.y * rv.y;
+            s[0] += a;
+            s[1] += K * a;
+        }
     }
-    const double s0 = block_sum((double)rr);
-    const double s1 = block_sum((double)rzn);
-    if (threadIdx.x == 0) { partial[2 * blockIdx.x] = s0; partial[2 * blockIdx.x + 1] = s1; }
+    finish_sum<2, kFieldThreads>(s, sum, 1.0);
 }
 
 // d = K r + beta d, beta = rz_new / rz_old (device scalars).
@@ -993,6 +991,10 @@ pcm_energy_kernel(const double2* __restrict__ phi, const double2* __restrict__ r
     if (threadIdx.x == 0) partial[blockIdx.x] = s;
 }
 
+int update_grid(const jdft_basis_s* b) {
+    return std::max(1, std::min(152 * 3, (b->S[0] * b->S[1] + kFieldThreads / 32 - 1) / (kFieldThreads / 32)));
+}
+
 GArgs g_args(const jdft_basis_s* b) {
     GArgs q;
     for (int i = 0; i < 9; ++i) q.B[i] = b->B[i];
@@ -1005,31 +1007,39 @@ template <> const double2* twiddles_of<double>(const jdft_basis_s* b) { return b
 template <> const float2* twiddles_of<float>(const jdft_basis_s* b) { return b->tw32; }
 
 // hessian of X into out (out must overlap neither X nor the three gradient
-// boxes Yg); with din, partial sums of Re conj(din) out into partial.
+// boxes Yg), X first made the new direction if dir says so; with dot, the sum of
+// Re conj(X) out into sum.out.
 template <typename T>
-jdft_status pcm_hessian(jdft_basis_s* b, const T* eps, const c_t<T>* X, c_t<T>* out, c_t<T>* Yg,
-                        const c_t<T>* din, double* partial, int* nblocks, cudaStream_t st) {
+jdft_status pcm_hessian(jdft_basis_s* b, const T* eps, c_t<T>* X, const DirectionArgs<T>& dir, c_t<T>* out, c_t<T>* Yg,
+                        bool dot, const BlockSum& sum, cudaStream_t st) {
     const GArgs q = g_args(b);
+    const c_t<T>* din = dot ? X : nullptr;
     if (field_fast(b->S[0]) && field_fast(b->S[1]) && field_fast(b->S[2])) {
         const FieldCell c = field_cell(b);
         const c_t<T>* tw = twiddles_of<T>(b);
         const LineGeom g1 = line_geom(b, 1, b->S[2]);
         const int64_t NB = b->N;
-        int blocks = 0;
         jdft_status s;
-        if ((s = JDFT_FIELD_LENGTH(b->S[0], FieldFast<T, N>::grad(X, Yg, c, NB, tw, b->plan[0], st)))) return s;
-        if ((s = JDFT_FIELD_LENGTH(b->S[1], FieldFast<T, N>::axis("field_fft_axis1_batch", +1, Yg, Yg, g1, T(1), 3, NB,
+        if ((s = JDFT_LINE_DISPATCH(b->S[0], FieldFast<T, N>::grad(X, dir, Yg, c, NB, tw, b->plan[0], st)))) return s;
+        if ((s = JDFT_LINE_DISPATCH(b->S[1], FieldFast<T, N>::axis("field_fft_axis1_batch", +1, Yg, Yg, g1, T(1), 3, NB,
                                                                   tw, b->plan[1], st))))
             return s;
-        if ((s = JDFT_FIELD_LENGTH(b->S[2], FieldFast<T, N>::eps(Yg, eps, b->S[0] * b->S[1], NB, tw, b->plan[2], st))))
+        if ((s = JDFT_LINE_DISPATCH(b->S[2], FieldFast<T, N>::eps(Yg, eps, b->S[0] * b->S[1], NB, tw, b->plan[2], st))))
             return s;
-        if ((s = JDFT_FIELD_LENGTH(b->S[1], FieldFast<T, N>::axis("field_fft_axis1_batch", -1, Yg, Yg, g1, T(1), 3, NB,
+        if ((s = JDFT_LINE_DISPATCH(b->S[1], FieldFast<T, N>::axis("field_fft_axis1_batch", -1, Yg, Yg, g1, T(1), 3, NB,
                                                                   tw, b->plan[1], st))))
             return s;
-        s = JDFT_FIELD_LENGTH(b->S[0], FieldFast<T, N>::div(Yg, din, out, c, NB, -1.0 / (kFourPi * (double)NB),
-                                                            partial, &blocks, tw, b->plan[0], st));
-        if (nblocks) *nblocks = blocks;
-        return s;
+        return JDFT_LINE_DISPATCH(b->S[0], FieldFast<T, N>::div(Yg, din, out, c, NB, -1.0 / (kFourPi * (double)NB), sum,
+                                                               tw, b->plan[0], st));
+    }
+    if (dir.r) {
+        {
+            Trace tr_("pcm_direction", st);
+            pcm_direction_kernel<T><<<reduce_grid(b->N), kFieldThreads, 0, st>>>(dir.r, X, dir.rz_new, dir.rz_old, q,
+                                                                                 b->N);
+        }
+        const jdft_status s = check_launch("pcm_direction");
+        if (s) return s;
     }
     const AxisGeom g0 = axis_geom(b, 0), g1 = axis_geom(b, 1), g2 = axis_geom(b, 2);
     const int64_t grid0 = (g0.nlines + g0.W - 1) / g0.W;
@@ -1077,10 +1087,10 @@ jdft_status pcm_hessian(jdft_basis_s* b, const T* eps, const c_t<T>* X, c_t<T>* 
     {
         Trace tr_("pcm_div_axis0", st);
         pcm_div_axis0_kernel<T><<<(unsigned)grid0, kFieldThreads, smem3, st>>>(
-            Yg, din, out, g0, p0, tw + p0.tw_offset, q, N, -1.0 / (kFourPi * (double)N), partial);
+            Yg, din, out, g0, p0, tw + p0.tw_offset, q, N, -1.0 / (kFourPi * (double)N), sum.partial);
     }
-    if (nblocks) *nblocks = (int)grid0;
-    return check_launch("pcm_div_axis0");
+    if ((s = check_launch("pcm_div_axis0")) || !dot) return s;
+    return launch_reduce(sum.partial, (int)grid0, 1, 1, 1.0, sum.out, false, st);
 }
 
 // Preconditioned CG on hessian(x) = r0 for boxes of type T, from x = 0:
@@ -1096,6 +1106,7 @@ jdft_status pcm_cg(jdft_basis_s* b, const T* eps, const double2* rho, c_t<T>* x,
     const int grid = reduce_grid(N);
     const GArgs q = g_args(b);
     jdft_status s;
+    unsigned* count = b->counters + 2;
     {
         Trace tr_("pcm_init", st);
         pcm_init_kernel<T><<<grid, kFieldThreads, 0, st>>>(rho, x, r, d, q, N, partial);
@@ -1112,27 +1123,22 @@ jdft_status pcm_cg(jdft_basis_s* b, const T* eps, const double2* rho, c_t<T>* x,
     if (bnorm > 0.0) {
         res = 1.0;
         for (it = 0; it < max_iter;) {
-            int nb0 = 0;
-            if ((s = pcm_hessian<T>(b, eps, d, Hd, Yg, d, partial, &nb0, st))) return s;
-            if ((s = launch_reduce(partial, nb0, 1, 1, 1.0, sc, false, st))) return s;
             double* old = sc + 2 + 2 * (it & 1);
             double* nw = sc + 2 + 2 * ((it + 1) & 1);
+            // the direction of this iteration (the first is pcm_init's) goes into the hessian's first pass
+            const DirectionArgs<T> dir{it > 0 ? r : nullptr, old + 1, nw + 1};
+            if ((s = pcm_hessian<T>(b, eps, d, dir, Hd, Yg, true, BlockSum{partial, count, sc}, st))) return s;
             {
                 Trace tr_("pcm_update", st);
-                pcm_update_kernel<T><<<grid, kFieldThreads, 0, st>>>(x, r, d, Hd, old + 1, sc, q, N, partial);
+                pcm_update_kernel<T><<<update_grid(b), kFieldThreads, 0, st>>>(x, r, d, Hd, old + 1, sc, q,
+                                                                     BlockSum{partial, count, nw});
             }
             if ((s = check_launch("pcm_update"))) return s;
-            if ((s = launch_reduce(partial, grid, 2, 2, 1.0, nw, false, st))) return s;
             JDFT_CUDA_TRY(cudaMemcpyAsync(host, nw, sizeof(double), cudaMemcpyDeviceToHost, st));
             JDFT_CUDA_TRY(cudaStreamSynchronize(st));
             ++it;
             res = std::sqrt(host[0]) / bnorm;
             if (!(res > rel_tol)) break;
-            {
-                Trace tr_("pcm_direction", st);
-                pcm_direction_kernel<T><<<grid, kFieldThreads, 0, st>>>(r, d, nw + 1, old + 1, q, N);
-            }
-            if ((s = check_launch("pcm_direction"))) return s;
         }
     }
     *iters = it;
@@ -1446,8 +1452,9 @@ jdft_status jdft_pcm_hessian(jdft_basis_t b, const double* eps, const void* phi_
     FieldWork w;
     jdft_status s = field_work(b, &w, 3);
     if (s) return s;
-    return pcm_hessian<double>(b, eps, (const double2*)phi_t, (double2*)out_t, w.box, nullptr, w.partial, nullptr,
-                               (cudaStream_t)stream);
+    // phi_t is only read: no direction, no dot product
+    return pcm_hessian<double>(b, eps, (double2*)phi_t, DirectionArgs<double>{nullptr, nullptr, nullptr}, (double2*)out_t,
+                               w.box, false, BlockSum{w.partial, nullptr, nullptr}, (cudaStream_t)stream);
 }
 
 jdft_status jdft_pcm_solve(jdft_basis_t b, const double* eps, const void* rho_t, void* phi_t, double tol,
@@ -1524,19 +1531,20 @@ jdft_status jdft_pcm_solve(jdft_basis_t b, const double* eps, const void* rho_t,
         }
         double rref = std::sqrt(host);
         int k = 0;                 // parity of the (|r|^2, r.Kr) slots
+        unsigned* count = b->counters + 2;
         while (res > tol && its < max_iter) {
-            int nb0 = 0;
-            if ((s = pcm_hessian<float>(b, eps32, d32, Hd32, Yg32, d32, w.partial, &nb0, st))) return s;
-            if ((s = launch_reduce(w.partial, nb0, 1, 1, 1.0, sc, false, st))) return s;
             double* old = sc + 2 + 2 * (k & 1);
             double* nw = sc + 2 + 2 * ((k + 1) & 1);
+            // the direction of this iteration (the first is pcm_init's) goes into the hessian's first pass
+            const DirectionArgs<float> dir{k > 0 ? r32 : nullptr, old + 1, nw + 1};
+            if ((s = pcm_hessian<float>(b, eps32, d32, dir, Hd32, Yg32, true, BlockSum{w.partial, count, sc}, st)))
+                return s;
             {
                 Trace tr_("pcm_update", st);
-                pcm_update_kernel<float><<<grid, kFieldThreads, 0, st>>>(e32, r32, d32, Hd32, old + 1, sc, q, N,
-                                                                         w.partial);
+                pcm_update_kernel<float><<<update_grid(b), kFieldThreads, 0, st>>>(e32, r32, d32, Hd32, old + 1, sc, q,
+                                                                         BlockSum{w.partial, count, nw});
             }
             if ((s = check_launch("pcm_update"))) return s;
-            if ((s = launch_reduce(w.partial, grid, 2, 2, 1.0, nw, false, st))) return s;
             JDFT_CUDA_TRY(cudaMemcpyAsync(&host, nw, sizeof(double), cudaMemcpyDeviceToHost, st));
             JDFT_CUDA_TRY(cudaStreamSynchronize(st));
             ++its;
@@ -1550,7 +1558,9 @@ jdft_status jdft_pcm_solve(jdft_basis_t b, const double* eps, const void* rho_t,
                 }
                 if ((s = check_launch("pcm_accumulate"))) return s;
                 JDFT_CUDA_TRY(cudaMemsetAsync(e32, 0, N * sizeof(float2), st));
-                if ((s = pcm_hessian<double>(b, eps, x, Hx, Yg64, nullptr, w.partial, nullptr, st))) return s;
+                if ((s = pcm_hessian<double>(b, eps, x, DirectionArgs<double>{nullptr, nullptr, nullptr}, Hx, Yg64, false,
+                                             BlockSum{w.partial, nullptr, nullptr}, st)))
+                    return s;
                 ++its64;
                 {
                     Trace tr_("pcm_residual", st);
@@ -1573,11 +1583,6 @@ jdft_status jdft_pcm_solve(jdft_basis_t b, const double* eps, const void* rho_t,
                 JDFT_CUDA_TRY(cudaStreamSynchronize(st));
                 rref = std::sqrt(host);
             }
-            {
-                Trace tr_("pcm_direction", st);
-                pcm_direction_kernel<float><<<grid, kFieldThreads, 0, st>>>(r32, d32, nw + 1, old + 1, q, N);
-            }
-            if ((s = check_launch("pcm_direction"))) return s;
         }
     }
     {

@@ -2,7 +2,9 @@
 // translation units, which instantiate them per type and length.
 #pragma once
 
+#include "block_sum.cuh"
 #include "fft_lanes.cuh"
+#include "fft_line.cuh"
 #include "field_fast.cuh"
 #include "field_lda.cuh"
 #include "profile.cuh"
@@ -20,15 +22,13 @@ __device__ __forceinline__ int fold(int m, int S) { return m < (S + 1) / 2 ? m :
 
 template <typename T, int N>
 struct Line {
-    static constexpr int E = RegCfg<T, N>::E;
-    using Fwd = LineFFT<T, N, E, -1, typename RegCfg<T, N>::R>;
-    using Inv = LineFFT<T, N, E, +1, typename RegCfg<T, N>::R>;
-    using LN = Lanes<N, E>;
-    static constexpr int LPW = LN::LPW, TL = LN::TL;
+    using F = LineOf<T, N>;
+    static constexpr int E = F::E, TL = F::TL;
     static constexpr int THREADS = 32 * kWarps<T>;
-    static constexpr int LPB = kWarps<T> * LPW;  // lines per block
-    static constexpr size_t SMEM = (N + (size_t)LPB * ScratchSpacing<T, N>::value) * sizeof(c_t<T>);
-    // this thread's position in its line, its line within the block, the table and the line's scratch
+    static constexpr int LPB = kWarps<T> * F::LPW;  // lines per block
+    static constexpr size_t SMEM = (N + (size_t)LPB * F::SPACING) * sizeof(c_t<T>);
+    // this thread's position in its line (past N for idle lanes, whose values are all invalid), its line
+    // within the block, the table and the line's scratch
     int t, line;
     const c_t<T>* W;
     c_t<T>* scr;
@@ -36,33 +36,23 @@ struct Line {
         c_t<T>* w = reinterpret_cast<c_t<T>*>(smem);
         for (int i = threadIdx.x; i < N; i += THREADS) w[i] = tw[i];
         const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-        t = LN::pos(lane);
-        line = warp * LPW + LN::line(lane);
-        scr = w + N + line * ScratchSpacing<T, N>::value;
+        t = lane < TL * F::LPW ? lane / F::LPW : 2 * N;
+        line = warp * F::LPW + lane % F::LPW;
+        scr = w + N + line * F::SPACING;
         W = w;
         __syncthreads();
     }
 };
 
-// Sum over the block in a fixed order; thread 0 returns it.
-template <int THREADS>
-__device__ __forceinline__ double block_total(double x) {
-    __shared__ double red[THREADS / 32];
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_down_sync(0xffffffffu, x, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = x;
-    __syncthreads();
-    double s = 0.0;
-    if (threadIdx.x == 0)
-        for (int i = 0; i < THREADS / 32; ++i) s += red[i];
-    return s;
-}
-
-template <typename T, int N, int SIGN>
+// The forward transform is the inverse one with real and imaginary parts swapped on
+// both sides: one compiled transform serves both signs.
+template <typename T, int N>
 __global__ void __launch_bounds__(Line<T, N>::THREADS)
-    axis_kernel(const c_t<T>* in, c_t<T>* out, LineGeom g, T scale, int64_t bstride, const c_t<T>* __restrict__ tw) {
+    axis_kernel(const c_t<T>* in, c_t<T>* out, LineGeom g, int forward, T scale, int64_t bstride,
+                const c_t<T>* __restrict__ tw) {
     extern __shared__ __align__(16) unsigned char smem[];
     using L = Line<T, N>;
-    using F = std::conditional_t<(SIGN > 0), typename L::Inv, typename L::Fwd>;
+    using F = typename L::F;
     L ln(smem, tw);
     const int l = blockIdx.x * L::LPB + ln.line;
     const bool act = l < g.nlines;
@@ -70,12 +60,20 @@ __global__ void __launch_bounds__(Line<T, N>::THREADS)
     const int64_t base = blockIdx.y * bstride + o * g.ostride + i * g.istride;
     c_t<T> v[L::E];
 #pragma unroll
-    for (int e = 0; e < L::E; ++e) v[e] = act ? in[base + F::in_index(ln.t, e) * g.es] : mk<T>(T(0), T(0));
-    F::run(v, ln.t, ln.scr, ln.W);
-    if (act) {
+    for (int e = 0; e < L::E; ++e) {
+        v[e] = mk<T>(T(0), T(0));
+        if (act && F::in_valid(ln.t, e)) {
+            const c_t<T> x = in[base + F::in_index(ln.t, e) * g.es];
+            v[e] = forward ? mk<T>(x.y, x.x) : x;
+        }
+    }
+    F::template run<+1>(v, ln.t, ln.scr, ln.W);
+    if (!act) return;
 #pragma unroll
-        for (int e = 0; e < L::E; ++e)
-            out[base + F::out_index(ln.t, e) * g.es] = mk<T>(scale * v[e].x, scale * v[e].y);
+    for (int e = 0; e < L::E; ++e) {
+        if (!F::out_valid(ln.t, e)) continue;
+        const c_t<T> y = forward ? mk<T>(v[e].y, v[e].x) : v[e];
+        out[base + F::out_index(ln.t, e) * g.es] = mk<T>(scale * y.x, scale * y.y);
     }
 }
 
@@ -90,17 +88,46 @@ __device__ __forceinline__ void line_G(const FieldCell& q, int l, int S2, T* G) 
 
 template <typename T, int N>
 __global__ void __launch_bounds__(Line<T, N>::THREADS)
-    grad_kernel(const c_t<T>* __restrict__ X, c_t<T>* __restrict__ Y, FieldCell q, int64_t bstride,
+    grad_kernel(c_t<T>* X, DirectionArgs<T> dir, c_t<T>* __restrict__ Y, FieldCell q, int64_t bstride,
                 const c_t<T>* __restrict__ tw) {
     extern __shared__ __align__(16) unsigned char smem[];
     using L = Line<T, N>;
-    using F = typename L::Inv;
+    using F = typename L::F;
     L ln(smem, tw);
     const int es = q.S[1] * q.S[2];
     const int l = blockIdx.x * L::LPB + ln.line;
     const bool act = l < es;
     T G[3];
     line_G<T>(q, act ? l : 0, q.S[2], G);
+    // The direction (saves a launch and a pass over d): each lane updates the values it reads below, in
+    // groups whose loads are all in flight before the first store.
+    if (dir.r && act) {
+        const T beta = (T)(*dir.rz_new / *dir.rz_old);
+        constexpr int GR = L::E % 8 == 0 ? 8 : L::E % 6 == 0 ? 6 : L::E % 5 == 0 ? 5 : L::E % 3 == 0 ? 3 : 1;
+#pragma unroll
+        for (int e0 = 0; e0 < L::E; e0 += GR) {
+            c_t<T> r[GR], d[GR];
+#pragma unroll
+            for (int i = 0; i < GR; ++i) {
+                r[i] = d[i] = mk<T>(T(0), T(0));
+                if (F::in_valid(ln.t, e0 + i)) {
+                    const int64_t a = l + (int64_t)F::in_index(ln.t, e0 + i) * es;
+                    r[i] = dir.r[a];
+                    d[i] = X[a];
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < GR; ++i) {
+                if (!F::in_valid(ln.t, e0 + i)) continue;
+                const int j = F::in_index(ln.t, e0 + i);
+                const T f0 = (T)fold(j, N);
+                const T gx = f0 * (T)q.B[0] + G[0], gy = f0 * (T)q.B[3] + G[1], gz = f0 * (T)q.B[6] + G[2];
+                const T g2 = gx * gx + gy * gy + gz * gz;
+                const T K = g2 > (T)0 ? (T)kFourPi / g2 : (T)0;
+                X[l + (int64_t)j * es] = mk<T>(K * r[i].x + beta * d[i].x, K * r[i].y + beta * d[i].y);
+            }
+        }
+    }
     // X is read again for each component: it stays in L1, and the registers go to the transform
 #pragma unroll 1
     for (int c = 0; c < 3; ++c) {
@@ -109,15 +136,16 @@ __global__ void __launch_bounds__(Line<T, N>::THREADS)
 #pragma unroll
         for (int e = 0; e < L::E; ++e) {
             const int j = F::in_index(ln.t, e);
-            const c_t<T> x = act ? X[l + (int64_t)j * es] : mk<T>(T(0), T(0));
+            const c_t<T> x = act && F::in_valid(ln.t, e) ? X[l + (int64_t)j * es] : mk<T>(T(0), T(0));
             const T Gc = (T)fold(j, N) * b0 + g0;
             v[e] = mk<T>(-Gc * x.y, Gc * x.x);
         }
-        F::run(v, ln.t, ln.scr, ln.W);
+        F::template run<+1>(v, ln.t, ln.scr, ln.W);
         if (act) {
             c_t<T>* Yc = Y + c * bstride + l;
 #pragma unroll
-            for (int e = 0; e < L::E; ++e) Yc[(int64_t)F::out_index(ln.t, e) * es] = v[e];
+            for (int e = 0; e < L::E; ++e)
+                if (F::out_valid(ln.t, e)) Yc[(int64_t)F::out_index(ln.t, e) * es] = v[e];
         }
         __syncwarp();
     }
@@ -129,37 +157,39 @@ __global__ void __launch_bounds__(Line<T, N>::THREADS)
                const c_t<T>* __restrict__ tw) {
     extern __shared__ __align__(16) unsigned char smem[];
     using L = Line<T, N>;
-    using F = typename L::Inv;
+    using F = typename L::F;
     L ln(smem, tw);
     const int l = blockIdx.x * L::LPB + ln.line;
     const bool act = l < nlines;
     c_t<T>* y = Y + blockIdx.y * bstride + (int64_t)l * N;
     c_t<T> v[L::E];
 #pragma unroll
-    for (int e = 0; e < L::E; ++e) v[e] = act ? y[F::in_index(ln.t, e)] : mk<T>(T(0), T(0));
-    F::run(v, ln.t, ln.scr, ln.W);
+    for (int e = 0; e < L::E; ++e)
+        v[e] = act && F::in_valid(ln.t, e) ? y[F::in_index(ln.t, e)] : mk<T>(T(0), T(0));
+    F::template run<+1>(v, ln.t, ln.scr, ln.W);
     const T* el = eps + (int64_t)(act ? l : 0) * N;
 #pragma unroll
     for (int e = 0; e < L::E; ++e) {
-        const T s = el[F::out_index(ln.t, e)];
-        v[e].x *= s;
-        v[e].y *= s;
+        const T s = F::out_valid(ln.t, e) ? el[F::out_index(ln.t, e)] : T(0);
+        // invalid slots hold leftovers of the earlier stages: zero, not a product, since they may not be finite
+        v[e] = F::out_valid(ln.t, e) ? mk<T>(s * v[e].x, s * v[e].y) : mk<T>(T(0), T(0));
     }
     // the forward transform as the inverse's adjoint: from the layout the inverse left to the one it read
-    F::run_adjoint(v, ln.t, ln.scr, ln.W);
+    F::template adjoint<-1>(v, ln.t, ln.scr, ln.W);
     if (act) {
 #pragma unroll
-        for (int e = 0; e < L::E; ++e) y[F::in_index(ln.t, e)] = v[e];
+        for (int e = 0; e < L::E; ++e)
+            if (F::in_valid(ln.t, e)) y[F::in_index(ln.t, e)] = v[e];
     }
 }
 
 template <typename T, int N>
 __global__ void __launch_bounds__(Line<T, N>::THREADS)
     div_kernel(const c_t<T>* __restrict__ Y, const c_t<T>* __restrict__ din, c_t<T>* __restrict__ out, FieldCell q,
-               int64_t bstride, double scale, double* __restrict__ partial, const c_t<T>* __restrict__ tw) {
+               int64_t bstride, double scale, BlockSum sum, const c_t<T>* __restrict__ tw) {
     extern __shared__ __align__(16) unsigned char smem[];
     using L = Line<T, N>;
-    using F = typename L::Fwd;
+    using F = typename L::F;
     L ln(smem, tw);
     const int es = q.S[1] * q.S[2];
     const int l = blockIdx.x * L::LPB + ln.line;
@@ -176,8 +206,8 @@ __global__ void __launch_bounds__(Line<T, N>::THREADS)
         c_t<T> v[L::E];
 #pragma unroll
         for (int e = 0; e < L::E; ++e)
-            v[e] = act ? Yc[(int64_t)F::in_index(ln.t, e) * es] : mk<T>(T(0), T(0));
-        F::run(v, ln.t, ln.scr, ln.W);
+            v[e] = act && F::in_valid(ln.t, e) ? Yc[(int64_t)F::in_index(ln.t, e) * es] : mk<T>(T(0), T(0));
+        F::template run<-1>(v, ln.t, ln.scr, ln.W);
 #pragma unroll
         for (int e = 0; e < L::E; ++e) {
             const T Gc = (T)fold(F::out_index(ln.t, e), N) * b0 + g0;
@@ -191,6 +221,7 @@ __global__ void __launch_bounds__(Line<T, N>::THREADS)
     if (act) {
 #pragma unroll
         for (int e = 0; e < L::E; ++e) {
+            if (!F::out_valid(ln.t, e)) continue;
             const int64_t a = l + (int64_t)F::out_index(ln.t, e) * es;
             const c_t<T> r = mk<T>(sc * acc[e].x, sc * acc[e].y);
             out[a] = r;
@@ -200,10 +231,7 @@ __global__ void __launch_bounds__(Line<T, N>::THREADS)
             }
         }
     }
-    if (din) {
-        const double s = block_total<L::THREADS>((double)part);
-        if (threadIdx.x == 0) partial[blockIdx.x] = s;
-    }
+    if (din) finish_sum<1, L::THREADS>(&part, sum, 1.0);
 }
 
 // ---- the Hartree chain on the half box -----------------------------------------
@@ -214,7 +242,7 @@ __global__ void __launch_bounds__(Line<double, N>::THREADS)
                             const double2* __restrict__ tw) {
     extern __shared__ __align__(16) unsigned char smem[];
     using L = Line<double, N>;
-    using F = typename L::Fwd;
+    using F = typename L::F;
     constexpr int H = N / 2 + 1;
     L ln(smem, tw);
     const int a = 2 * (blockIdx.x * L::LPB + ln.line);
@@ -224,12 +252,14 @@ __global__ void __launch_bounds__(Line<double, N>::THREADS)
 #pragma unroll
     for (int e = 0; e < L::E; ++e) {
         const int j = F::in_index(ln.t, e);
-        v[e] = make_double2(actA ? na[j] : 0.0, actB ? na[N + j] : 0.0);
+        const bool ok = F::in_valid(ln.t, e);
+        v[e] = make_double2(actA && ok ? na[j] : 0.0, actB && ok ? na[N + j] : 0.0);
     }
-    F::run(v, ln.t, ln.scr, ln.W);
+    F::template run<-1>(v, ln.t, ln.scr, ln.W);
     __syncwarp();
 #pragma unroll
-    for (int e = 0; e < L::E; ++e) ln.scr[padx(F::out_index(ln.t, e))] = v[e];
+    for (int e = 0; e < L::E; ++e)
+        if (F::out_valid(ln.t, e)) ln.scr[padx(F::out_index(ln.t, e))] = v[e];
     __syncwarp();
     double2* ha = half + (int64_t)a * H;
     for (int k = ln.t; k < H; k += L::TL) {
@@ -244,7 +274,7 @@ __global__ void __launch_bounds__(Line<double, N>::THREADS)
 static __device__ __noinline__ double coulomb_plain(double g2) { return g2 > 0.0 ? kFourPi / g2 : 0.0; }
 __device__ __forceinline__ double coulomb_of(double g2) {
     if (!(g2 > 1e-30 && g2 < 1e30)) return coulomb_plain(g2);
-    double r = (double)__frcp_rn((float)g2);
+    double r = long_of(__fdividef(1.0f, short_of(g2)));
     const double f = fma(-g2, r, 1.0);
     r = fma(r, fma(f, f, f), r);
     return kFourPi * r;
@@ -256,11 +286,11 @@ __device__ __forceinline__ double norm2(const FieldCell& q, double f0, double lx
 
 template <int N>
 __global__ void __launch_bounds__(Line<double, N>::THREADS)
-    hartree_kernel0_kernel(double2* __restrict__ half, FieldCell q, double* __restrict__ partial,
+    hartree_kernel0_kernel(double2* __restrict__ half, FieldCell q, BlockSum sum, double sum_scale,
                            const double2* __restrict__ tw) {
     extern __shared__ __align__(16) unsigned char smem[];
     using L = Line<double, N>;
-    using F = typename L::Fwd;
+    using F = typename L::F;
     L ln(smem, tw);
     const int H = q.S[2] / 2 + 1, es = q.S[1] * H;
     const int l = blockIdx.x * L::LPB + ln.line;
@@ -268,8 +298,9 @@ __global__ void __launch_bounds__(Line<double, N>::THREADS)
     const int m1 = act ? l / H : 0, m2 = act ? l - m1 * H : 0;
     double2 v[L::E];
 #pragma unroll
-    for (int e = 0; e < L::E; ++e) v[e] = act ? half[l + (int64_t)F::in_index(ln.t, e) * es] : make_double2(0.0, 0.0);
-    F::run(v, ln.t, ln.scr, ln.W);
+    for (int e = 0; e < L::E; ++e)
+        v[e] = act && F::in_valid(ln.t, e) ? half[l + (int64_t)F::in_index(ln.t, e) * es] : make_double2(0.0, 0.0);
+    F::template run<-1>(v, ln.t, ln.scr, ln.W);
     double G[3], Gm[3];
     line_G<double>(q, m1 * q.S[2] + m2, q.S[2], G);
     // the mirror slot -m of the full box: a Nyquist index folds to -S/2 on both sides, so on
@@ -281,6 +312,10 @@ __global__ void __launch_bounds__(Line<double, N>::THREADS)
     double part = 0.0;
 #pragma unroll
     for (int e = 0; e < L::E; ++e) {
+        if (!F::out_valid(ln.t, e)) {
+            v[e] = make_double2(0.0, 0.0);
+            continue;
+        }
         const int t = F::out_index(ln.t, e);
         double K = coulomb_of(norm2(q, (double)fold(t, N), G[0], G[1], G[2]));
         if (ny1 || ny2 || 2 * t == N) {
@@ -294,23 +329,24 @@ __global__ void __launch_bounds__(Line<double, N>::THREADS)
     }
     // slots with 0 < m2 < S2/2 stand for their mirrors too
     part *= invN * invN * (m2 == 0 || ny2 ? 1.0 : 2.0);
-    F::run_adjoint(v, ln.t, ln.scr, ln.W);
+    F::template adjoint<+1>(v, ln.t, ln.scr, ln.W);
     if (act) {
 #pragma unroll
-        for (int e = 0; e < L::E; ++e) half[l + (int64_t)F::in_index(ln.t, e) * es] = v[e];
+        for (int e = 0; e < L::E; ++e)
+            if (F::in_valid(ln.t, e)) half[l + (int64_t)F::in_index(ln.t, e) * es] = v[e];
     }
-    const double s = block_total<L::THREADS>(act ? part : 0.0);
-    if (threadIdx.x == 0) partial[blockIdx.x] = s;
+    if (!act) part = 0.0;
+    if (sum.out) finish_sum<1, L::THREADS>(&part, sum, sum_scale);
 }
 
 template <int N, bool KS>
 __global__ void __launch_bounds__(Line<double, N>::THREADS)
     hartree_inverse2_kernel(const double2* __restrict__ half, double* __restrict__ V, const double* __restrict__ n,
-                            const double* __restrict__ vion, double* __restrict__ partial, int nlines,
+                            const double* __restrict__ vion, BlockSum sum, double sum_scale, int nlines,
                             const double2* __restrict__ tw) {
     extern __shared__ __align__(16) unsigned char smem[];
     using L = Line<double, N>;
-    using F = typename L::Inv;
+    using F = typename L::F;
     constexpr int H = N / 2 + 1;
     L ln(smem, tw);
     const int a = 2 * (blockIdx.x * L::LPB + ln.line);
@@ -320,14 +356,16 @@ __global__ void __launch_bounds__(Line<double, N>::THREADS)
 #pragma unroll
     for (int e = 0; e < L::E; ++e) {
         const int j = F::in_index(ln.t, e), k = 2 * j <= N ? j : N - j;
-        double2 A = actA ? ha[k] : make_double2(0.0, 0.0), B = actB ? ha[H + k] : make_double2(0.0, 0.0);
+        const bool ok = F::in_valid(ln.t, e);
+        double2 A = actA && ok ? ha[k] : make_double2(0.0, 0.0), B = actB && ok ? ha[H + k] : make_double2(0.0, 0.0);
         if (k == 0 || 2 * k == N) A.y = B.y = 0.0;  // real for real lines
         v[e] = 2 * j <= N ? make_double2(A.x - B.y, A.y + B.x) : make_double2(A.x + B.y, B.x - A.y);
     }
-    F::run(v, ln.t, ln.scr, ln.W);
+    F::template run<+1>(v, ln.t, ln.scr, ln.W);
     double part = 0.0;
 #pragma unroll
     for (int e = 0; e < L::E; ++e) {
+        if (!F::out_valid(ln.t, e)) continue;
         const int64_t j = (int64_t)a * N + F::out_index(ln.t, e);
         if constexpr (KS) {
 #pragma unroll
@@ -347,8 +385,7 @@ __global__ void __launch_bounds__(Line<double, N>::THREADS)
         }
     }
     if constexpr (KS) {
-        const double s = block_total<L::THREADS>(part);
-        if (threadIdx.x == 0) partial[blockIdx.x] = s;
+        if (sum.out) finish_sum<1, L::THREADS>(&part, sum, sum_scale);
     }
 }
 
@@ -370,15 +407,13 @@ template <typename T, int N>
 jdft_status FieldFast<T, N>::axis(const char* name, int sign, const c_t<T>* in, c_t<T>* out, const LineGeom& g, T scale,
                                   int batch, int64_t bstride, const c_t<T>* tw, const FftPlan& p, cudaStream_t st) {
     const c_t<T>* t = reg_table<T>(tw, p);
-    return sign > 0 ? ff::launch<T, N>(name, ff::axis_kernel<T, N, +1>, g.nlines, batch, st, in, out, g, scale,
-                                       bstride, t)
-                    : ff::launch<T, N>(name, ff::axis_kernel<T, N, -1>, g.nlines, batch, st, in, out, g, scale,
-                                       bstride, t);
+    return ff::launch<T, N>(name, ff::axis_kernel<T, N>, g.nlines, batch, st, in, out, g, sign < 0 ? 1 : 0, scale,
+                            bstride, t);
 }
 template <typename T, int N>
-jdft_status FieldFast<T, N>::grad(const c_t<T>* X, c_t<T>* Y, const FieldCell& q, int64_t bstride, const c_t<T>* tw,
-                                  const FftPlan& p, cudaStream_t st) {
-    return ff::launch<T, N>("pcm_grad_axis0", ff::grad_kernel<T, N>, q.S[1] * q.S[2], 1, st, X, Y, q, bstride,
+jdft_status FieldFast<T, N>::grad(c_t<T>* X, const DirectionArgs<T>& dir, c_t<T>* Y, const FieldCell& q,
+                                  int64_t bstride, const c_t<T>* tw, const FftPlan& p, cudaStream_t st) {
+    return ff::launch<T, N>("pcm_grad_axis0", ff::grad_kernel<T, N>, q.S[1] * q.S[2], 1, st, X, dir, Y, q, bstride,
                             reg_table<T>(tw, p));
 }
 template <typename T, int N>
@@ -389,11 +424,10 @@ jdft_status FieldFast<T, N>::eps(c_t<T>* Y, const T* eps, int nlines, int64_t bs
 }
 template <typename T, int N>
 jdft_status FieldFast<T, N>::div(const c_t<T>* Y, const c_t<T>* din, c_t<T>* out, const FieldCell& q, int64_t bstride,
-                                 double scale, double* partial, int* blocks, const c_t<T>* tw, const FftPlan& p,
+                                 double scale, const BlockSum& sum, const c_t<T>* tw, const FftPlan& p,
                                  cudaStream_t st) {
-    *blocks = (q.S[1] * q.S[2] + ff::Line<T, N>::LPB - 1) / ff::Line<T, N>::LPB;
     return ff::launch<T, N>("pcm_div_axis0", ff::div_kernel<T, N>, q.S[1] * q.S[2], 1, st, Y, din, out, q, bstride,
-                            scale, partial, reg_table<T>(tw, p));
+                            scale, sum, reg_table<T>(tw, p));
 }
 
 template <int N>
@@ -403,24 +437,21 @@ jdft_status HartreeFast<N>::forward2(const double* n, double2* half, int nlines,
                                  nlines, reg_table<double>(tw, p));
 }
 template <int N>
-jdft_status HartreeFast<N>::kernel0(double2* half, const FieldCell& q, double* partial, int* blocks,
+jdft_status HartreeFast<N>::kernel0(double2* half, const FieldCell& q, const BlockSum& sum, double sum_scale,
                                     const double2* tw, const FftPlan& p, cudaStream_t st) {
-    const int lines = q.S[1] * (q.S[2] / 2 + 1);
-    *blocks = (lines + ff::Line<double, N>::LPB - 1) / ff::Line<double, N>::LPB;
-    return ff::launch<double, N>("hartree_kernel_axis0", ff::hartree_kernel0_kernel<N>, lines, 1, st, half, q, partial,
-                                 reg_table<double>(tw, p));
+    return ff::launch<double, N>("hartree_kernel_axis0", ff::hartree_kernel0_kernel<N>, q.S[1] * (q.S[2] / 2 + 1), 1, st,
+                                 half, q, sum, sum_scale, reg_table<double>(tw, p));
 }
 template <int N>
 jdft_status HartreeFast<N>::inverse2(const double2* half, double* V, const double* n, const double* vion,
-                                     double* partial, int* blocks, int nlines, const double2* tw, const FftPlan& p,
-                                     cudaStream_t st) {
+                                     const BlockSum& sum, double sum_scale, int nlines, const double2* tw,
+                                     const FftPlan& p, cudaStream_t st) {
     const int slots = (nlines + 1) / 2;
-    *blocks = (slots + ff::Line<double, N>::LPB - 1) / ff::Line<double, N>::LPB;
     if (vion)
         return ff::launch<double, N>("ks_potential_axis2", ff::hartree_inverse2_kernel<N, true>, slots, 1, st, half, V,
-                                     n, vion, partial, nlines, reg_table<double>(tw, p));
+                                     n, vion, sum, sum_scale, nlines, reg_table<double>(tw, p));
     return ff::launch<double, N>("field_fft_axis2", ff::hartree_inverse2_kernel<N, false>, slots, 1, st, half, V, n,
-                                 vion, partial, nlines, reg_table<double>(tw, p));
+                                 vion, sum, sum_scale, nlines, reg_table<double>(tw, p));
 }
 
 }  // namespace jdft

@@ -17,6 +17,9 @@ LD = np.longdouble
 SKEW = np.array([[7.0, 1.1, -0.6], [0.4, 6.2, 0.9], [0.0, -0.7, 8.1]])
 BOXES = [(12, 16, 40), (40, 12, 16), (16, 48, 12), (48, 40, 64), (64, 12, 80), (80, 64, 12), (12, 128, 16), (16, 12, 256),
          (256, 16, 12), (128, 12, 48)]
+# the other lengths, each on every axis
+_REST = [24, 25, 27, 30, 32, 36, 45, 50, 54, 60, 72, 75, 81, 90, 96, 100, 108, 120, 125]
+RAGGED = [(_REST[i], _REST[(i + 7) % 19], _REST[(i + 13) % 19]) for i in range(19)]
 
 
 def _basis(S):
@@ -105,7 +108,39 @@ def test_transforms_and_hartree(S):
     assert abs(float(e[0]) / eh - 1) < 64 * U64 and abs(float(e[1]) / exc - 1) < 64 * U64
 
 
-@pytest.mark.parametrize("S", [BOXES[0], BOXES[3], BOXES[5], BOXES[7], BOXES[8], BOXES[9]],
+@pytest.mark.parametrize("S", RAGGED, ids=lambda s: "x".join(map(str, s)))
+def test_ragged_lengths(S):
+    """I, J and the Kohn-Sham potential on the other lengths.  Between passes the line of a large mean m keeps n m with a
+    rounding of u n m, against sqrt(n) d for fluctuations d on it: the potential (no G = 0 term) of such a density is off by
+    up to 8 u (1 + sqrt(n) m / d) in any FP64 transform."""
+    jdft, b = _basis(S)
+    N = int(np.prod(S))
+    rng = np.random.default_rng(N + 2)
+    x = rng.standard_normal(N) + 1j * rng.standard_normal(N)
+    xd = torch.tensor(x, device="cuda")
+    out = torch.empty_like(xd)
+    jdft.jdft_field_I(b, xd, out)
+    assert _rel(out.cpu().numpy(), _I(S, x)) < 32 * U64
+    jdft.jdft_field_J(b, xd, out)
+    assert _rel(out.cpu().numpy(), _J(S, x)) < 32 * U64
+    n = 0.05 * rng.random(N) + 1e-3
+    vion = 0.1 * rng.standard_normal(N)
+    K, nt, om = _coulomb(S), _J(S, n), LD(np.linalg.det(SKEW))
+    vh = _I(S, K * nt).real
+    eh = float(om / 2 * (K * np.abs(nt) ** 2).sum())
+    exc_n, vxc = _lda(n)
+    exc = float(om / N * (n * exc_n).sum())
+    nd, vd = torch.tensor(n, device="cuda"), torch.empty(N, dtype=torch.float64, device="cuda")
+    e = torch.zeros(2, dtype=torch.float64, device="cuda")
+    tol = 8 * U64 * (1 + np.sqrt(max(S)) * n.mean() / n.std())
+    jdft.jdft_hartree(b, nd, vd, e[:1])
+    assert _rel(vd.cpu().numpy(), vh) < tol and abs(float(e[0]) / eh - 1) < 2 * tol
+    jdft.jdft_ks_potential(b, nd, torch.tensor(vion, device="cuda"), vd, e)
+    assert _rel(vd.cpu().numpy(), vion + vh + vxc) < tol
+    assert abs(float(e[0]) / eh - 1) < 2 * tol and abs(float(e[1]) / exc - 1) < 64 * U64
+
+
+@pytest.mark.parametrize("S", [BOXES[0], BOXES[3], BOXES[5], BOXES[7], BOXES[8], BOXES[9]] + RAGGED[::3],
                          ids=lambda s: "x".join(map(str, s)))
 def test_dielectric_solve(S):
     """The hessian in FP64, and the FP32 solve, whose FP64 residual the library measures with it."""
