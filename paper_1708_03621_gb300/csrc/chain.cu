@@ -693,19 +693,34 @@ static jdft_status run_apply_H(jdft_basis_s* b, int ik, const void* C, int ldc, 
     jdft_status s = ensure_workspace(b, ch.bytes + nlbytes);
     if (s != JDFT_OK) return s;
     ch.bind(b->work.ptr);
+    void* nlwork = (char*)b->work.ptr + ch.bytes;
     const T omega = (T)b->omega, invN = (T)(1.0 / (double)b->N);
-    for (int b0 = 0; b0 < nb; b0 += ch.nc) {
+    // D P^dag C needs C alone: where neither it nor the chain fills the GPU it runs beside the chain on the
+    // basis's side stream and joins before P (D P^dag C) is added (FP64 H C of 16 bands with 32 projectors on
+    // 48^3: OVERLAP64; FP32, 13 bands on 60 x 54 x 72: OVERLAP32).
+    const bool beside = sp.nproj > 0 && nonlocal_small(sp, nb, prec);
+    auto nonlocal = [&](cudaStream_t on, int phases) {
+        return nonlocal_accumulate<T>(sp, C, ldc, HC, ldhc, nb, prec, nlwork, on, true, nullptr, true, &b->prodwork, phases);
+    };
+    if (beside) {
+        if ((s = side_stream(b))) return s;
+        JDFT_CUDA_TRY(cudaEventRecord(b->ev_fork, st));
+        JDFT_CUDA_TRY(cudaStreamWaitEvent(b->side, b->ev_fork, 0));
+        s = nonlocal(b->side, kNonlocalProject);
+        // joined whatever happened, so that nothing of this call outlives it on the side stream
+        JDFT_CUDA_TRY(cudaEventRecord(b->ev_join, b->side));
+    }
+    for (int b0 = 0; b0 < nb && s == JDFT_OK; b0 += ch.nc) {
         const int n = std::min(ch.nc, nb - b0);
         const c_t<T>* Cc = (const c_t<T>*)C + (size_t)b0 * ldc;
         c_t<T>* Hc = (c_t<T>*)HC + (size_t)b0 * ldhc;
-        if ((s = ch.inverse(Cc, ldc, n, st))) return s;
-        if ((s = ch.apply(n, st))) return s;
-        if ((s = ch.forward(Cc, ldc, Hc, ldhc, kinetic<T>(sp), omega, invN, n, st))) return s;
+        if ((s = ch.inverse(Cc, ldc, n, st))) break;
+        if ((s = ch.apply(n, st))) break;
+        s = ch.forward(Cc, ldc, Hc, ldhc, kinetic<T>(sp), omega, invN, n, st);
     }
-    if (sp.nproj > 0)
-        return nonlocal_accumulate<T>(sp, C, ldc, HC, ldhc, nb, prec, (char*)b->work.ptr + ch.bytes, st, true, nullptr,
-                                      true, &b->prodwork);
-    return JDFT_OK;
+    if (beside) JDFT_CUDA_TRY(cudaStreamWaitEvent(st, b->ev_join, 0));
+    if (s != JDFT_OK || sp.nproj == 0) return s;
+    return nonlocal(st, beside ? kNonlocalAdd : kNonlocalBoth);
 }
 
 // H C and the density of the same block: per chunk one pass in, then the fused

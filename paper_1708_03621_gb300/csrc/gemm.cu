@@ -26,6 +26,9 @@ namespace jdft {
 // ---------------------------------------------------------------------------
 constexpr int CN_BK = 32, CN_WARPS = 4;
 
+__device__ __forceinline__ double mad(double a, double b, double c) { return fma(a, b, c); }
+__device__ __forceinline__ float mad(float a, float b, float c) { return fmaf(a, b, c); }
+
 template <typename T, int TM, int TN>
 __global__ void __launch_bounds__(32 * CN_WARPS)
     zgemm_cn_kernel(int M, int N, int K, int kchunk, const c_t<T>* __restrict__ A, int lda,
@@ -72,9 +75,9 @@ __global__ void __launch_bounds__(32 * CN_WARPS)
             for (int i = 0; i < PM; ++i)
 #pragma unroll
                 for (int j = 0; j < PN; ++j) {
-                    // conj(a) * b
-                    acc[i][j].x += a[i].x * b[j].x + a[i].y * b[j].y;
-                    acc[i][j].y += a[i].x * b[j].y - a[i].y * b[j].x;
+                    // conj(a) * b, as four multiply-adds (summing the two products first would make six)
+                    acc[i][j].x = mad(a[i].y, b[j].y, mad(a[i].x, b[j].x, acc[i][j].x));
+                    acc[i][j].y = mad(-a[i].y, b[j].x, mad(a[i].x, b[j].y, acc[i][j].y));
                 }
         }
         __syncthreads();
@@ -168,8 +171,8 @@ __global__ void __launch_bounds__(32 * NN_WARPS)
 #pragma unroll
                 for (int j = 0; j < NN_PN; ++j) {
                     const c_t<T> b = Bs[kk][warp * NN_PN + j];
-                    acc[j].x += a.x * b.x - a.y * b.y;
-                    acc[j].y += a.x * b.y + a.y * b.x;
+                    acc[j].x = mad(-a.y, b.y, mad(a.x, b.x, acc[j].x));
+                    acc[j].y = mad(a.y, b.x, mad(a.x, b.y, acc[j].y));
                 }
             }
         }
@@ -244,43 +247,51 @@ static const c_t<T>* proj_ptr(const KSphere& sp);
 template <> const double2* proj_ptr<double>(const KSphere& sp) { return (const double2*)sp.P; }
 template <> const float2* proj_ptr<float>(const KSphere& sp) { return (const float2*)sp.P32; }
 
+bool nonlocal_small(const KSphere& sp, int nb, jdft_prec prec) {
+    if (prec == JDFT_FP64) return !sl_eligible(sp.nproj, nb, sp.npw) && !sl_eligible(sp.npw, nb, sp.nproj);
+    return !tcx_eligible(prec, sp.nproj, nb) && (size_t)sp.nproj * nb * sp.npw < (size_t)64 << 20;
+}
+
 template <typename T>
 jdft_status nonlocal_accumulate(const KSphere& sp, const void* C, int ldc, void* HC, int ldhc, int nb,
                                 jdft_prec prec, void* work, cudaStream_t st, bool split_c, const void* Csplit,
-                                bool partials, ProductScratch* scratch) {
+                                bool partials, ProductScratch* scratch, int phases) {
     if (sp.nproj == 0 || nb == 0) return JDFT_OK;
     double2* Bc = (double2*)work;
     const size_t abytes = ((size_t)sp.nproj * nb * sizeof(double2) + 255) / 256 * 256;
     const size_t bbytes = ((size_t)sp.nproj * nb * sizeof(c_t<T>) + 255) / 256 * 256;
     c_t<T>* Bd = (c_t<T>*)((char*)work + abytes);
-    JDFT_CUDA_TRY(cudaMemsetAsync(Bc, 0, (size_t)sp.nproj * nb * sizeof(double2), st));
     jdft_status s;
     const bool split_ops = std::is_same<T, float>::value && (split_c || Csplit) && sp.Psplit &&
                            tcx_eligible(prec, sp.nproj, nb);
     const size_t cbytes = split_c && tcx_eligible(prec, sp.nproj, nb)
                               ? (tcx_split_bytes(nb, sp.npw) + 255) / 256 * 256 : 0;
-    if (split_ops) {
-        const void* Cs = Csplit;
-        if (!Cs) {
-            void* own = (char*)work + abytes + bbytes;
-            if ((s = tcx_split((const float2*)C, ldc, nb, sp.npw, own, st))) return s;
-            Cs = own;
+    if (phases & kNonlocalProject) {
+        JDFT_CUDA_TRY(cudaMemsetAsync(Bc, 0, (size_t)sp.nproj * nb * sizeof(double2), st));
+        if (split_ops) {
+            const void* Cs = Csplit;
+            if (!Cs) {
+                void* own = (char*)work + abytes + bbytes;
+                if ((s = tcx_split((const float2*)C, ldc, nb, sp.npw, own, st))) return s;
+                Cs = own;
+            }
+            const size_t dbytes = (tcx_split_bytes(nb, sp.nproj) + 255) / 256 * 256;
+            void* part = partials ? (char*)work + abytes + bbytes + cbytes + dbytes : nullptr;
+            s = tcx_cn(sp.nproj, nb, sp.npw, sp.Psplit, Cs, Bc, nb, 1.0, st, part,
+                       partials ? tcx_cn_partial_bytes(sp.nproj, nb, sp.npw) : 0);
+        } else {
+            s = gemm_cn<T>(prec, sp.nproj, nb, sp.npw, proj_ptr<T>(sp), sp.npw, (const c_t<T>*)C, ldc, Bc, nb, 1.0, st,
+                           scratch);
         }
-        const size_t dbytes = (tcx_split_bytes(nb, sp.nproj) + 255) / 256 * 256;
-        void* part = partials ? (char*)work + abytes + bbytes + cbytes + dbytes : nullptr;
-        s = tcx_cn(sp.nproj, nb, sp.npw, sp.Psplit, Cs, Bc, nb, 1.0, st, part,
-                   partials ? tcx_cn_partial_bytes(sp.nproj, nb, sp.npw) : 0);
-    } else {
-        s = gemm_cn<T>(prec, sp.nproj, nb, sp.npw, proj_ptr<T>(sp), sp.npw, (const c_t<T>*)C, ldc, Bc, nb, 1.0, st,
-                       scratch);
+        if (s != JDFT_OK) return s;
+        {
+            Trace tr_("dmul", st);
+            dmul_kernel<T><<<std::min(152 * 8, (sp.nproj * nb + 255) / 256), 256, 0, st>>>(sp.nproj, nb, sp.Dw, sp.Dcol,
+                                                                                            sp.Dval, Bc, Bd);
+        }
+        if ((s = check_launch("dmul"))) return s;
     }
-    if (s != JDFT_OK) return s;
-    {
-        Trace tr_("dmul", st);
-        dmul_kernel<T><<<std::min(152 * 8, (sp.nproj * nb + 255) / 256), 256, 0, st>>>(sp.nproj, nb, sp.Dw, sp.Dcol,
-                                                                                        sp.Dval, Bc, Bd);
-    }
-    if ((s = check_launch("dmul"))) return s;
+    if (!(phases & kNonlocalAdd)) return JDFT_OK;
     if (split_ops && sp.Psplit_t) {
         // HC += P (D P^dag C): P's transposed split (made with the projectors) and that of D P^dag C
         void* Bt = (char*)work + abytes + bbytes + cbytes;
@@ -332,9 +343,9 @@ template jdft_status zgemm_nn_acc<double>(int, int, int, const double2*, int, co
 template jdft_status zgemm_nn_acc<float>(int, int, int, const float2*, int, const float2*, int, float2*, int,
                                          cudaStream_t, bool);
 template jdft_status nonlocal_accumulate<double>(const KSphere&, const void*, int, void*, int, int, jdft_prec, void*,
-                                                 cudaStream_t, bool, const void*, bool, ProductScratch*);
+                                                 cudaStream_t, bool, const void*, bool, ProductScratch*, int);
 template jdft_status nonlocal_accumulate<float>(const KSphere&, const void*, int, void*, int, int, jdft_prec, void*,
-                                                cudaStream_t, bool, const void*, bool, ProductScratch*);
+                                                cudaStream_t, bool, const void*, bool, ProductScratch*, int);
 
 }  // namespace jdft
 

@@ -90,6 +90,8 @@ bool gemm_nn_inplace_ok(jdft_prec prec, int N);
 size_t nonlocal_workspace_bytes(int nproj, int nb, size_t elem, int npw = 0, jdft_prec prec = JDFT_FP64,
                                 bool split_c = false, bool partials = false);
 
+// The two halves of the nonlocal term: D P^dag C into the workspace, and HC += P (that).
+constexpr int kNonlocalProject = 1, kNonlocalAdd = 2, kNonlocalBoth = 3;
 // HC += P D P^dag C for the sphere's projectors (no-op when nproj == 0).
 // split_c: take the projection from split operands (tcx_cn) when it is
 // eligible, splitting C in the workspace, which must then hold
@@ -103,6 +105,9 @@ template <typename T>
 jdft_status nonlocal_accumulate(const KSphere& sp, const void* C, int ldc, void* HC, int ldhc, int nb,
                                 jdft_prec prec, void* work, cudaStream_t st, bool split_c = false,
                                 const void* Csplit = nullptr, bool partials = false,
-                                ProductScratch* scratch = nullptr);
+                                ProductScratch* scratch = nullptr, int phases = kNonlocalBoth);
+// Whether both products of the nonlocal term are too small for the split-operand and
+// sliced kernels: then neither part of H C fills the GPU.
+bool nonlocal_small(const KSphere& sp, int nb, jdft_prec prec);
 
 }  // namespace jdft

@@ -850,8 +850,7 @@ namespace jdft {
 
 static size_t r256(size_t x) { return (x + 255) / 256 * 256; }
 
-// Side stream and fork / join events of a basis (created on first use).
-static jdft_status step_streams(jdft_basis_s* b) {
+jdft_status side_stream(jdft_basis_s* b) {
     if (!b->side) {
         JDFT_CUDA_TRY(cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking));
         JDFT_CUDA_TRY(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
@@ -921,7 +920,7 @@ static jdft_status hamiltonian_step_impl(jdft_basis_s* b, int ik, void* C, int l
     }
     c_t<T>* W = nullptr;
     if (ortho) {
-        if ((s = step_streams(b))) return s;
+        if ((s = side_stream(b))) return s;
         JDFT_CUDA_TRY(cudaEventRecord(b->ev_fork, st));
         JDFT_CUDA_TRY(cudaStreamWaitEvent(b->side, b->ev_fork, 0));
         if ((s = overlap_factor<T>(b, COC, nb, sticky, b->side, &W))) return s;

@@ -38,9 +38,11 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
 }
 // Bounded wait: true once the phase with the given parity has completed;
 // false if limit_ns nanoseconds pass first.  A limit of 0 gives up without
-// trying (the failure path's tests rely on that).
+// trying (the failure path's tests rely on that).  The timer is read only when
+// the first try fails: reading it costs more than a short product.
 __device__ __forceinline__ bool mbar_wait_ns(uint64_t* bar, uint32_t parity, uint64_t limit_ns) {
     if (limit_ns == 0) return false;
+    if (mbar_try_wait(bar, parity)) return true;
     const uint64_t t0 = globaltimer_ns();
     do {
         if (mbar_try_wait(bar, parity)) return true;

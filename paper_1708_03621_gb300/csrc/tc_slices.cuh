@@ -159,6 +159,34 @@ struct SlLayout {
     static_assert(NCOLS <= 512 && SMEM <= 227 * 1024, "one block per SM");
 };
 
+// The pieces of the issuing thread's loop, on shared-memory addresses and descriptor words.
+__device__ __forceinline__ bool sl_wait(uint32_t bar, uint32_t parity, uint64_t* generic, uint64_t wait_ns) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    if (ok && wait_ns) return true;
+    return tc::mbar_wait_ns(generic, parity, wait_ns);
+}
+__device__ __forceinline__ void sl_mma(uint32_t d_tmem, uint32_t alo, uint32_t blo, uint32_t hi, uint32_t idesc,
+                                       uint32_t accumulate) {
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b64 da, db;\n\t"
+        "mov.b64 da, {%1, %3};\n\t"
+        "mov.b64 db, {%2, %3};\n\t"
+        "setp.ne.b32 p, %5, 0;\n\t"
+        "tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %4, p;\n\t}"
+        ::"r"(d_tmem), "r"(alo), "r"(blo), "r"(hi), "r"(idesc), "r"(accumulate)
+        : "memory");
+}
+__device__ __forceinline__ void sl_commit(uint32_t bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+}
+
 // CONJ: Re = Ar.Br + Ai.Bi, Im = Ar.Bi - Ai.Br (conj(A) B); else Re = Ar.Br - Ai.Bi, Im = Ar.Bi + Ai.Br.
 // part: [tile][unit][column][row] of (Re, Im) integers, S_D + 2^7 S_(D-1).
 template <int NT, bool CONJ>
@@ -201,58 +229,78 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
     const unsigned long long wait_ns = g_tc_wait_ns;
     if (tid == 0) {
         // step j of a chunk: slice j of A and slice D - j of B (1-based)
-        int it = 0;
+        const size_t aplane = (size_t)rpA * (TCX_KC * 2), bplane = (size_t)rpB * (TCX_KC * 2);
+        int it = 0, s = 0;
+        uint32_t par = 1;
         for (int kc = c0; kc < c1 && !flags[0]; ++kc) {
+            const char* pa = As + (size_t)kc * SL_PLANES * aplane + (size_t)m0 * (TCX_KC * 2);
+            const char* pb = Bs + ((size_t)kc * SL_PLANES + 2 * (D - 2)) * bplane + (size_t)n0 * (TCX_KC * 2);
             for (int j = 1; j <= steps; ++j, ++it) {
-                const int s = it % SL_STAGES;
-                if (!tc::mbar_wait_ns(&empty[s], (uint32_t)((it / SL_STAGES) & 1) ^ 1u, wait_ns)) {
+                if (!tc::mbar_wait_ns(&empty[s], par, wait_ns)) {
                     flags[0] = 1;
                     break;
                 }
                 unsigned char* st = smem + s * L::STAGE;
                 tc::mbar_arrive_expect_tx(&full[s], (uint32_t)L::STAGE);
-#pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    bulk_load(st + c * L::A_PL,
-                              As + ((size_t)(kc * SL_PLANES + 2 * (j - 1) + c) * rpA + m0) * (TCX_KC * 2), L::A_PL,
-                              &full[s]);
-                    bulk_load(st + 2 * L::A_PL + c * L::B_PL,
-                              Bs + ((size_t)(kc * SL_PLANES + 2 * (D - j - 1) + c) * rpB + n0) * (TCX_KC * 2), L::B_PL,
-                              &full[s]);
+                bulk_load(st, pa, L::A_PL, &full[s]);
+                bulk_load(st + L::A_PL, pa + aplane, L::A_PL, &full[s]);
+                bulk_load(st + 2 * L::A_PL, pb, L::B_PL, &full[s]);
+                bulk_load(st + 2 * L::A_PL + L::B_PL, pb + bplane, L::B_PL, &full[s]);
+                pa += 2 * aplane;
+                pb -= 2 * bplane;
+                if (++s == SL_STAGES) {
+                    s = 0;
+                    par ^= 1u;
                 }
             }
         }
         flags[1] = it;
     } else if (tid == 32) {
+        // One thread issues every product, and its instructions are what the loop waits for (descriptors
+        // built anew for each product took 1100 clocks a step of 8 products; these, 64 clocks each at
+        // NT = 128): a descriptor differs from stage to stage in its low word alone.
         constexpr uint32_t idesc = tc::instr_desc(1u, TCX_M, NT);
         constexpr uint32_t idesc_neg = idesc | (1u << 13);  // negate A
+        const uint64_t d0 = tc::smem_desc(tc::smem_addr(smem), 128, 256);
+        const uint32_t dhi = (uint32_t)(d0 >> 32);
+        constexpr uint32_t AI = L::A_PL >> 4, B0 = (2 * L::A_PL) >> 4, BI = L::B_PL >> 4, ST = L::STAGE >> 4;
+        const uint32_t fullbar = tc::smem_addr(full), emptybar = tc::smem_addr(empty);
+        const uint32_t re = tmem, im = tmem + NT, re1 = tmem + 2 * NT, im1 = tmem + 3 * NT;
+        uint32_t a = (uint32_t)d0, prev = 0, s = 0, sp = 0, par = 0, acc = 0, acc1 = 0;
         int it = 0;
         for (int kc = c0; kc < c1 && !flags[0]; ++kc) {
             for (int j = 1; j <= steps; ++j, ++it) {
-                const int s = it % SL_STAGES, sp = (it + SL_STAGES - 1) % SL_STAGES;
-                if (!tc::mbar_wait_ns(&full[s], (uint32_t)((it / SL_STAGES) & 1), wait_ns)) {
+                if (!sl_wait(fullbar + 8 * s, par, &full[s], wait_ns)) {
                     flags[0] = 1;
                     break;
                 }
                 tc::tc_fence_after_sync();
-                const uint32_t base = tc::smem_addr(smem + s * L::STAGE);
-                const uint32_t prev = tc::smem_addr(smem + sp * L::STAGE);
-                const uint64_t br = tc::smem_desc(base + 2 * L::A_PL, 128, 256);
-                const uint64_t bi = tc::smem_desc(base + 2 * L::A_PL + L::B_PL, 128, 256);
-                // q = 0: this step's slice of A into the sum D; q = 1: the previous one's into D - 1
-                for (int q = 0; q < 2 && (q == 0 || j > 1); ++q) {
-                    const uint32_t ab = q == 0 ? base : prev;
-                    const uint64_t ar = tc::smem_desc(ab, 128, 256), ai = tc::smem_desc(ab + L::A_PL, 128, 256);
-                    const uint32_t re = tmem + 2 * q * NT, im = re + NT;
-                    const uint32_t acc = (kc > c0 || j > 1 + q) ? 1u : 0u;
-                    tc::mma_bf16(re, ar, br, idesc, acc);
-                    tc::mma_bf16(re, ai, bi, CONJ ? idesc : idesc_neg, 1u);
-                    tc::mma_bf16(im, ar, bi, idesc, acc);
-                    tc::mma_bf16(im, ai, br, CONJ ? idesc_neg : idesc, 1u);
+                const uint32_t b = a + B0;
+                // this step's slice of A into the sum D, the previous one's into D - 1
+                sl_mma(re, a, b, dhi, idesc, acc);
+                sl_mma(im, a, b + BI, dhi, idesc, acc);
+                sl_mma(re, a + AI, b + BI, dhi, CONJ ? idesc : idesc_neg, 1u);
+                sl_mma(im, a + AI, b, dhi, CONJ ? idesc_neg : idesc, 1u);
+                acc = 1u;
+                if (j > 1) {
+                    sl_mma(re1, prev, b, dhi, idesc, acc1);
+                    sl_mma(im1, prev, b + BI, dhi, idesc, acc1);
+                    sl_mma(re1, prev + AI, b + BI, dhi, CONJ ? idesc : idesc_neg, 1u);
+                    sl_mma(im1, prev + AI, b, dhi, CONJ ? idesc_neg : idesc, 1u);
+                    acc1 = 1u;
+                    // the previous slice of A has been used twice now
+                    sl_commit(emptybar + 8 * sp);
                 }
-                // the previous slice of A has been used twice now; the chunk's last one is not needed again
-                if (j > 1) tc::mma_commit(&empty[sp]);
-                if (j == steps) tc::mma_commit(&empty[s]);
+                if (j == steps) sl_commit(emptybar + 8 * s);  // the chunk's last slice is not needed again
+                prev = a;
+                sp = s;
+                if (++s == SL_STAGES) {
+                    s = 0;
+                    par ^= 1u;
+                    a = (uint32_t)d0;
+                } else {
+                    a += ST;
+                }
             }
         }
         flags[2] = it;
@@ -385,21 +433,31 @@ __global__ void __launch_bounds__(TCX_M* RZ)
 }
 
 // ---- host ---------------------------------------------------------------------------
+// Units of the largest size the sums allow, or up to four times smaller: the
+// choice whose waves of blocks, each as long as its largest unit, end first.
 static SlPlan sl_plan(int nkc, int tiles) {
-    SlPlan p;
-    // steps of the whole product (2 (D - 1) - 1 products a chunk and group), cut into about three waves of blocks
-    int64_t all = 0;
-    for (int g = 0; g < SL_GROUPS; ++g) all += (int64_t)nkc * (2 * sl_top(g) - 3);
-    const int64_t want = std::max<int64_t>(1, all * tiles / (3 * 152));
-    p.first[0] = 0;
-    for (int g = 0; g < SL_GROUPS; ++g) {
-        int per = (int)std::min<int64_t>(sl_limit(g), std::max<int64_t>(4, want / (2 * sl_top(g) - 3)));
-        const int n = (nkc + per - 1) / per;
-        per = (nkc + n - 1) / n;
-        p.per[g] = per;
-        p.first[g + 1] = p.first[g] + (nkc + per - 1) / per;
+    constexpr int kOverhead = 180;  // of a unit, in products: barriers, tensor memory, the integers out
+    SlPlan best{};
+    int64_t best_cost = -1;
+    for (int f = 16; f >= 4; --f) {
+        SlPlan p;
+        p.first[0] = 0;
+        int64_t longest = 0;
+        for (int g = 0; g < SL_GROUPS; ++g) {
+            const int top = std::max(1, std::min(sl_limit(g), nkc) * f / 16);
+            const int n = (nkc + top - 1) / top;
+            p.per[g] = (nkc + n - 1) / n;
+            p.first[g + 1] = p.first[g] + (nkc + p.per[g] - 1) / p.per[g];
+            longest = std::max<int64_t>(longest, (int64_t)p.per[g] * 4 * (2 * sl_top(g) - 3));
+        }
+        const int64_t waves = ((int64_t)p.first[SL_GROUPS] * tiles + 151) / 152;
+        const int64_t cost = waves * (longest + kOverhead);
+        if (best_cost < 0 || cost < best_cost) {
+            best = p;
+            best_cost = cost;
+        }
     }
-    return p;
+    return best;
 }
 static int sl_units_max(int nkc, int tiles) { return sl_plan(nkc, tiles).first[SL_GROUPS]; }
 static int sl_nt(int N) { return N <= 32 ? 32 : N <= 64 ? 64 : 128; }
