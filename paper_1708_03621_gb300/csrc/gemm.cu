@@ -22,7 +22,8 @@ namespace jdft {
 // 8 x 4, TM/8 x TN/4 outputs each), so one shared-memory read feeds 5 to 11
 // multiply-adds.  The warps' sums meet in shared memory, the blocks' in FP64 atomics.
 // Against a 32 x 32 tile of 256 threads with 2 x 2 outputs each and at least 64
-// K to a block, 16 x 16 over 4 259 plane waves took 142 us and takes 27 (event times).
+// K to a block, 16 x 16 over 4 259 plane waves took 142 us and takes 22 (event times),
+// 27 before a complex multiply-add was written as four fused instructions (mad).
 // ---------------------------------------------------------------------------
 constexpr int CN_BK = 32, CN_WARPS = 4;
 
@@ -142,7 +143,7 @@ jdft_status zgemm_cn(int M, int N, int K, const c_t<T>* A, int lda, const c_t<T>
 // (32 consecutive values a warp, sixteen rows in flight) and Bm, staged 64 rows deep, by broadcast.
 // Small blocks, because N is small where this kernel is used and M/32 of them
 // just fill the SMs: 16 x 16 over 4 259 rows 40 -> 23 us in FP64 against 64 m to a
-// block, which used 67 SMs.
+// block, which used 67 SMs, and 18 with four fused instructions a multiply-add.
 // ---------------------------------------------------------------------------
 constexpr int NN_BM = 32, NN_PN = 4, NN_WARPS = 4, NN_BN = NN_PN * NN_WARPS, NN_BK = 64;
 

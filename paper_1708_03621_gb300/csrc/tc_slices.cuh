@@ -23,14 +23,14 @@
 // A unit of work (block) is a 128 x NT output tile, a pair of digit sums (D, D - 1)
 // and a range of K: at step j it adds A_j B_(D-j) to the first and
 // A_(j-1) B_(D-j) to the second accumulator, so each slice is staged once for
-// two products (33 bytes a clock and SM; one sum alone would need 64).  Tensor
-// memory holds 2 x 2 x NT columns.
+// two products; three steps share a stage, copied by one bulk copy per operand.
+// Tensor memory holds 2 x 2 x NT columns.
 //
-// Measured: overlap, subspace matrix and rotation of 120 bands of 27 000 plane
-// waves 19.86 -> 1.51 ms, error against 64-bit references 6.7e-16 -> 5.9e-16 (the
-// Cholesky factorisation between them takes 0.4 ms); H C of 64 bands on a 128^3
-// box with 256 projectors 28.06 -> 7.64 ms, its two projector products 22.4 ms of
-// the former.
+// Measured (event times, against the CUDA-core products): overlap, subspace matrix
+// and rotation of 120 bands of 27 000 plane waves 19.86 -> 1.32 ms, error against
+// 64-bit references 6.7e-16 -> 5.9e-16 (the Cholesky factorisation between them
+// takes 0.35 ms); H C of 64 bands on a 128^3 box with 256 projectors 28.06 -> 7.64 ms
+// when they came in, their two launches of products 0.65 ms each then and 0.58 now.
 #pragma once
 
 namespace jdft {
@@ -39,7 +39,8 @@ constexpr int SL_N = 9;                 // slices of an operand
 constexpr int SL_BITS = 7;
 constexpr int SL_GROUPS = 5;            // digit sums (10, 9), (8, 7), (6, 5), (4, 3), (2)
 constexpr int SL_PLANES = 2 * SL_N;     // Re and Im of each slice
-constexpr int SL_STAGES = 12;
+constexpr int SL_STAGES = 4;
+constexpr int SL_RUN = 3;               // slices per stage and operand, one copy each
 constexpr int SL_THREADS = 128;
 constexpr int SL_BAD = 1 << 20;         // row exponent of a row with an infinity or NaN
 __host__ __device__ constexpr int sl_top(int g) { return 10 - 2 * g; }              // larger digit sum of group g
@@ -87,15 +88,22 @@ __device__ __forceinline__ int sl_exponent(int maxhi, bool& up) {
 }
 
 // ---- slices -------------------------------------------------------------------
+// Layout: [chunk of 16 K][block of RB rows][plane][RB x 16 values], the rows of a
+// plane as core matrices (as in the split blocks above).  The planes of consecutive
+// slices of a row block are one contiguous run, so a stage of three steps takes one
+// bulk copy per operand and one barrier, in place of four copies and a barrier a step
+// (products of 120 x 120 over 27 000: 162 -> 147 us a launch; of 256 x 64 over a 128^3
+// box's plane waves: 651 -> 582 us).
 // One thread per row and 8 consecutive K values: a 16-byte core-matrix row of
-// each of the 18 planes (layout of the split blocks above, 18 planes a chunk).
+// each of the 18 planes.
 template <bool TRANS>
 __global__ void __launch_bounds__(256) sl_slice_kernel(const double2* __restrict__ X, size_t ld, int rows, int K,
-                                                       int rows_pad, int nkc, const int* __restrict__ maxhi,
+                                                       int rows_pad, int RB, int nkc, const int* __restrict__ maxhi,
                                                        __nv_bfloat16* __restrict__ out) {
     const int per_chunk = rows_pad * 2;
     const int64_t total = (int64_t)per_chunk * nkc;
-    const size_t P = (size_t)rows_pad * TCX_KC;  // elements between planes of one chunk
+    const size_t P = (size_t)RB * TCX_KC;  // elements between planes
+    const int nrb = rows_pad / RB;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
         const int kc = (int)(i / per_chunk), u = (int)(i - (int64_t)kc * per_chunk);
         const int r8 = u & 7, h = (u >> 3) & 1, g = u >> 4;
@@ -125,7 +133,9 @@ __global__ void __launch_bounds__(256) sl_slice_kernel(const double2* __restrict
                 d[c][j] = (uint64_t)((t ^ s) - s) + kOffset;
             }
         }
-        __nv_bfloat16* o = out + (size_t)kc * SL_PLANES * P + (size_t)(r & ~7) * TCX_KC + h * 64 + r8 * 8;
+        const int rb = r / RB;
+        __nv_bfloat16* o = out + ((size_t)kc * nrb + rb) * SL_PLANES * P + (size_t)((r - rb * RB) & ~7) * TCX_KC + h * 64 +
+                           r8 * 8;
         const __nv_bfloat162 off = __floats2bfloat162_rn(192.f, 192.f);
 #pragma unroll
         for (int s = 0; s < SL_N; ++s) {
@@ -152,7 +162,9 @@ template <int NT>
 struct SlLayout {
     static constexpr int A_PL = TCX_PLANE;
     static constexpr int B_PL = NT * TCX_KC * 2;
-    static constexpr int STAGE = 2 * A_PL + 2 * B_PL;
+    static constexpr int A_SL = 2 * A_PL, B_SL = 2 * B_PL;  // one slice: Re and Im
+    static constexpr int B_OFF = SL_RUN * A_SL;
+    static constexpr int STAGE = SL_RUN * (A_SL + B_SL);
     static constexpr int BAR_OFF = SL_STAGES * STAGE;
     static constexpr int SMEM = BAR_OFF + 512 + 1024;
     static constexpr uint32_t NCOLS = 4 * NT;
@@ -191,7 +203,7 @@ __device__ __forceinline__ void sl_commit(uint32_t bar) {
 // part: [tile][unit][column][row] of (Re, Im) integers, S_D + 2^7 S_(D-1).
 template <int NT, bool CONJ>
 __global__ void __launch_bounds__(SL_THREADS, 1)
-    sl_mma_kernel(const char* __restrict__ As, const char* __restrict__ Bs, int rpA, int rpB, int nkc, int mtiles,
+    sl_mma_kernel(const char* __restrict__ As, const char* __restrict__ Bs, int nrbA, int nrbB, int nkc, int mtiles,
                   SlPlan plan, int2* __restrict__ part) {
     using L = SlLayout<NT>;
     extern __shared__ unsigned char smem_raw[];
@@ -208,8 +220,9 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
     while (g + 1 < SL_GROUPS && unit >= plan.first[g + 1]) ++g;
     const int D = sl_top(g), steps = D - 1;
     const int c0 = (unit - plan.first[g]) * plan.per[g], c1 = min(nkc, c0 + plan.per[g]);
-    const int m0 = (tile % mtiles) * TCX_M, n0 = (tile / mtiles) * NT;
-    const int total = (c1 - c0) * steps;  // at least one: the plan has no empty units
+    const int mt = tile % mtiles, nt = tile / mtiles;
+    const int runs = (steps + SL_RUN - 1) / SL_RUN;  // stages per chunk
+    const int total = (c1 - c0) * runs;              // at least one: the plan has no empty units
     if (tid == 0) {
         for (int s = 0; s < SL_STAGES; ++s) {
             tc::mbar_init(&full[s], 1);
@@ -228,26 +241,23 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
     const uint32_t tmem = *tslot;
     const unsigned long long wait_ns = g_tc_wait_ns;
     if (tid == 0) {
-        // step j of a chunk: slice j of A and slice D - j of B (1-based)
-        const size_t aplane = (size_t)rpA * (TCX_KC * 2), bplane = (size_t)rpB * (TCX_KC * 2);
+        // steps j = j0 .. j0 + n - 1 of a chunk to a stage: slices j of A (ascending) and D - j of B
+        // (1-based; copied ascending, so step i of the stage finds its slice of B at place n - 1 - i)
         int it = 0, s = 0;
         uint32_t par = 1;
         for (int kc = c0; kc < c1 && !flags[0]; ++kc) {
-            const char* pa = As + (size_t)kc * SL_PLANES * aplane + (size_t)m0 * (TCX_KC * 2);
-            const char* pb = Bs + ((size_t)kc * SL_PLANES + 2 * (D - 2)) * bplane + (size_t)n0 * (TCX_KC * 2);
-            for (int j = 1; j <= steps; ++j, ++it) {
+            const char* pa = As + ((size_t)kc * nrbA + mt) * SL_N * L::A_SL;
+            const char* pb = Bs + ((size_t)kc * nrbB + nt) * SL_N * L::B_SL;
+            for (int j0 = 1; j0 <= steps; j0 += SL_RUN, ++it) {
+                const int n = min(SL_RUN, steps - j0 + 1);
                 if (!tc::mbar_wait_ns(&empty[s], par, wait_ns)) {
                     flags[0] = 1;
                     break;
                 }
                 unsigned char* st = smem + s * L::STAGE;
-                tc::mbar_arrive_expect_tx(&full[s], (uint32_t)L::STAGE);
-                bulk_load(st, pa, L::A_PL, &full[s]);
-                bulk_load(st + L::A_PL, pa + aplane, L::A_PL, &full[s]);
-                bulk_load(st + 2 * L::A_PL, pb, L::B_PL, &full[s]);
-                bulk_load(st + 2 * L::A_PL + L::B_PL, pb + bplane, L::B_PL, &full[s]);
-                pa += 2 * aplane;
-                pb -= 2 * bplane;
+                tc::mbar_arrive_expect_tx(&full[s], (uint32_t)(n * (L::A_SL + L::B_SL)));
+                bulk_load(st, pa + (size_t)(j0 - 1) * L::A_SL, n * L::A_SL, &full[s]);
+                bulk_load(st + L::B_OFF, pb + (size_t)(D - j0 - n) * L::B_SL, n * L::B_SL, &full[s]);
                 if (++s == SL_STAGES) {
                     s = 0;
                     par ^= 1u;
@@ -256,50 +266,53 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
         }
         flags[1] = it;
     } else if (tid == 32) {
-        // One thread issues every product, and its instructions are what the loop waits for (descriptors
-        // built anew for each product took 1100 clocks a step of 8 products; these, 64 clocks each at
-        // NT = 128): a descriptor differs from stage to stage in its low word alone.
+        // One thread issues every product: its loop works on descriptor words, of which only the low one
+        // differs from slice to slice (descriptors built anew for each product: 120 x 120 over 27 000 took
+        // 203 us a launch, with these words 162).
         constexpr uint32_t idesc = tc::instr_desc(1u, TCX_M, NT);
         constexpr uint32_t idesc_neg = idesc | (1u << 13);  // negate A
         const uint64_t d0 = tc::smem_desc(tc::smem_addr(smem), 128, 256);
         const uint32_t dhi = (uint32_t)(d0 >> 32);
-        constexpr uint32_t AI = L::A_PL >> 4, B0 = (2 * L::A_PL) >> 4, BI = L::B_PL >> 4, ST = L::STAGE >> 4;
+        constexpr uint32_t AI = L::A_PL >> 4, BI = L::B_PL >> 4, AS = L::A_SL >> 4, BS = L::B_SL >> 4, ST = L::STAGE >> 4;
         const uint32_t fullbar = tc::smem_addr(full), emptybar = tc::smem_addr(empty);
         const uint32_t re = tmem, im = tmem + NT, re1 = tmem + 2 * NT, im1 = tmem + 3 * NT;
-        uint32_t a = (uint32_t)d0, prev = 0, s = 0, sp = 0, par = 0, acc = 0, acc1 = 0;
+        uint32_t stage = (uint32_t)d0, prev = 0, s = 0, sp = 0, par = 0, acc = 0, acc1 = 0;
         int it = 0;
         for (int kc = c0; kc < c1 && !flags[0]; ++kc) {
-            for (int j = 1; j <= steps; ++j, ++it) {
+            for (int j0 = 1; j0 <= steps; j0 += SL_RUN, ++it) {
+                const int n = min(SL_RUN, steps - j0 + 1);
                 if (!sl_wait(fullbar + 8 * s, par, &full[s], wait_ns)) {
                     flags[0] = 1;
                     break;
                 }
                 tc::tc_fence_after_sync();
-                const uint32_t b = a + B0;
-                // this step's slice of A into the sum D, the previous one's into D - 1
-                sl_mma(re, a, b, dhi, idesc, acc);
-                sl_mma(im, a, b + BI, dhi, idesc, acc);
-                sl_mma(re, a + AI, b + BI, dhi, CONJ ? idesc : idesc_neg, 1u);
-                sl_mma(im, a + AI, b, dhi, CONJ ? idesc_neg : idesc, 1u);
-                acc = 1u;
-                if (j > 1) {
-                    sl_mma(re1, prev, b, dhi, idesc, acc1);
-                    sl_mma(im1, prev, b + BI, dhi, idesc, acc1);
-                    sl_mma(re1, prev + AI, b + BI, dhi, CONJ ? idesc : idesc_neg, 1u);
-                    sl_mma(im1, prev + AI, b, dhi, CONJ ? idesc_neg : idesc, 1u);
-                    acc1 = 1u;
-                    // the previous slice of A has been used twice now
-                    sl_commit(emptybar + 8 * sp);
+                uint32_t a = stage, b = stage + (L::B_OFF >> 4) + (n - 1) * BS;
+                for (int i = 0; i < n; ++i, a += AS, b -= BS) {
+                    // this step's slice of A into the sum D, the previous one's into D - 1
+                    sl_mma(re, a, b, dhi, idesc, acc);
+                    sl_mma(im, a, b + BI, dhi, idesc, acc);
+                    sl_mma(re, a + AI, b + BI, dhi, CONJ ? idesc : idesc_neg, 1u);
+                    sl_mma(im, a + AI, b, dhi, CONJ ? idesc_neg : idesc, 1u);
+                    acc = 1u;
+                    if (j0 + i > 1) {
+                        sl_mma(re1, prev, b, dhi, idesc, acc1);
+                        sl_mma(im1, prev, b + BI, dhi, idesc, acc1);
+                        sl_mma(re1, prev + AI, b + BI, dhi, CONJ ? idesc : idesc_neg, 1u);
+                        sl_mma(im1, prev + AI, b, dhi, CONJ ? idesc_neg : idesc, 1u);
+                        acc1 = 1u;
+                        // the previous stage's last slice of A has been used twice now
+                        if (i == 0) sl_commit(emptybar + 8 * sp);
+                    }
+                    prev = a;
                 }
-                if (j == steps) sl_commit(emptybar + 8 * s);  // the chunk's last slice is not needed again
-                prev = a;
+                if (j0 + SL_RUN > steps) sl_commit(emptybar + 8 * s);  // the chunk's last stage is not needed again
                 sp = s;
                 if (++s == SL_STAGES) {
                     s = 0;
                     par ^= 1u;
-                    a = (uint32_t)d0;
+                    stage = (uint32_t)d0;
                 } else {
-                    a += ST;
+                    stage += ST;
                 }
             }
         }
@@ -480,7 +493,7 @@ bool sl_eligible(int M, int N, int K) {
 }
 
 template <int NT, bool CONJ>
-static jdft_status sl_launch_nt(const void* As, const void* Bs, int rpA, int rpB, int nkc, int mtiles, int tiles,
+static jdft_status sl_launch_nt(const void* As, const void* Bs, int nrbA, int nrbB, int nkc, int mtiles, int tiles,
                                 const SlPlan& plan, int2* part, cudaStream_t st) {
     auto kern = sl_mma_kernel<NT, CONJ>;
     cudaError_t e = set_smem_attr((const void*)kern, SlLayout<NT>::SMEM);
@@ -488,23 +501,22 @@ static jdft_status sl_launch_nt(const void* As, const void* Bs, int rpA, int rpB
     {
         Trace tr_("sl_mma", st);
         kern<<<dim3(plan.first[SL_GROUPS], tiles), SL_THREADS, SlLayout<NT>::SMEM, st>>>(
-            (const char*)As, (const char*)Bs, rpA, rpB, nkc, mtiles, plan, part);
+            (const char*)As, (const char*)Bs, nrbA, nrbB, nkc, mtiles, plan, part);
     }
     return check_launch("sl_mma");
 }
 
 template <bool CONJ>
-static jdft_status sl_product(const void* As, const void* Bs, int rpB, int M, int N, int NT, int nkc, const int* maxA,
+static jdft_status sl_product(const void* As, const void* Bs, int M, int N, int NT, int nkc, const int* maxA,
                               const int* maxB, void* partial, double2* out, size_t sm, size_t sn, double scale,
                               bool accumulate, cudaStream_t st) {
-    const int rpA = tcx_rows_pad(M);
-    const int mtiles = rpA / TCX_M, tiles = mtiles * ((N + NT - 1) / NT);
+    const int mtiles = tcx_rows_pad(M) / TCX_M, ntiles = (N + NT - 1) / NT, tiles = mtiles * ntiles;
     const SlPlan plan = sl_plan(nkc, tiles);
     int2* part = (int2*)partial;
     jdft_status s;
-    if (NT == 32) s = sl_launch_nt<32, CONJ>(As, Bs, rpA, rpB, nkc, mtiles, tiles, plan, part, st);
-    else if (NT == 64) s = sl_launch_nt<64, CONJ>(As, Bs, rpA, rpB, nkc, mtiles, tiles, plan, part, st);
-    else s = sl_launch_nt<128, CONJ>(As, Bs, rpA, rpB, nkc, mtiles, tiles, plan, part, st);
+    if (NT == 32) s = sl_launch_nt<32, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, st);
+    else if (NT == 64) s = sl_launch_nt<64, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, st);
+    else s = sl_launch_nt<128, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, st);
     if (s != JDFT_OK) return s;
     {
         Trace tr_("sl_reduce", st);
@@ -519,11 +531,12 @@ static jdft_status sl_product(const void* As, const void* Bs, int rpB, int M, in
     return check_launch("sl_reduce");
 }
 
-// Row maxima and slices of an operand (K values a row; trans: X[k * ld + r]).
-static jdft_status sl_slice(const double2* X, size_t ld, int rows, int rows_pad, int K, bool trans, int* maxhi,
+// Row maxima and slices of an operand (K values a row; trans: X[k * ld + r]), its
+// rows padded to blocks of RB.
+static jdft_status sl_slice(const double2* X, size_t ld, int rows, int RB, int K, bool trans, int* maxhi,
                             void* slices, cudaStream_t st) {
     JDFT_CUDA_TRY(cudaMemsetAsync(maxhi, 0, (size_t)rows * sizeof(int), st));
-    const int nkc = tcx_chunks(K);
+    const int nkc = tcx_chunks(K), rows_pad = (rows + RB - 1) / RB * RB;
     const int64_t total = (int64_t)rows_pad * 2 * nkc;
     const int grid = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
     {
@@ -541,9 +554,11 @@ static jdft_status sl_slice(const double2* X, size_t ld, int rows, int rows_pad,
     {
         Trace tr_("sl_slice", st);
         if (trans)
-            sl_slice_kernel<true><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, nkc, maxhi, (__nv_bfloat16*)slices);
+            sl_slice_kernel<true><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, RB, nkc, maxhi,
+                                                        (__nv_bfloat16*)slices);
         else
-            sl_slice_kernel<false><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, nkc, maxhi, (__nv_bfloat16*)slices);
+            sl_slice_kernel<false><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, RB, nkc, maxhi,
+                                                         (__nv_bfloat16*)slices);
     }
     return check_launch("sl_slice");
 }
@@ -551,8 +566,8 @@ static jdft_status sl_slice(const double2* X, size_t ld, int rows, int rows_pad,
 jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* out,
                         int ldo, double scale, ProductScratch& scratch, cudaStream_t st) {
     const int NT = sl_nt(N);
-    const bool same = A == B && lda == ldb && M == N;  // one set of slices (rows padded to 128, a multiple of NT)
-    const int rpA = tcx_rows_pad(M), rpB = same ? rpA : (N + NT - 1) / NT * NT;
+    const bool same = A == B && lda == ldb && M == N && NT == TCX_M;  // one set of slices
+    const int rpA = tcx_rows_pad(M), rpB = (N + NT - 1) / NT * NT;
     const int tiles = rpA / TCX_M * ((N + NT - 1) / NT);
     const size_t mx = sl_align((size_t)(M + N) * sizeof(int));
     auto bytes = [&](int k) {
@@ -571,9 +586,9 @@ jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const do
         char* As = (char*)ws + mx;
         char* Bs = same ? As : As + sl_block_bytes(rpA, k);
         char* part = Bs + sl_block_bytes(rpB, k);
-        if ((s = sl_slice(A + k0, lda, M, rpA, k, false, maxA, As, st))) return s;
-        if (!same && (s = sl_slice(B + k0, ldb, N, rpB, k, false, maxB, Bs, st))) return s;
-        if ((s = sl_product<true>(As, Bs, rpB, M, N, NT, tcx_chunks(k), maxA, maxB, part, out, ldo, 1, scale, true, st)))
+        if ((s = sl_slice(A + k0, lda, M, TCX_M, k, false, maxA, As, st))) return s;
+        if (!same && (s = sl_slice(B + k0, ldb, N, NT, k, false, maxB, Bs, st))) return s;
+        if ((s = sl_product<true>(As, Bs, M, N, NT, tcx_chunks(k), maxA, maxB, part, out, ldo, 1, scale, true, st)))
             return s;
     }
     return JDFT_OK;
@@ -603,9 +618,9 @@ jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const do
         char* Bs = (char*)ws + sl_align((size_t)(m + N) * sizeof(int));
         char* As = Bs + sl_block_bytes(rpB, K);
         char* part = As + sl_block_bytes(rpA, K);
-        if ((s = sl_slice(Bm, ldb, N, rpB, K, true, maxB, Bs, st))) return s;
-        if ((s = sl_slice(A + m0, lda, m, rpA, K, true, maxA, As, st))) return s;
-        if ((s = sl_product<false>(As, Bs, rpB, m, N, NT, nkc, maxA, maxB, part, out + m0, 1, ldo, 1.0, accumulate, st)))
+        if ((s = sl_slice(Bm, ldb, N, NT, K, true, maxB, Bs, st))) return s;
+        if ((s = sl_slice(A + m0, lda, m, TCX_M, K, true, maxA, As, st))) return s;
+        if ((s = sl_product<false>(As, Bs, m, N, NT, nkc, maxA, maxB, part, out + m0, 1, ldo, 1.0, accumulate, st)))
             return s;
     }
     return JDFT_OK;
