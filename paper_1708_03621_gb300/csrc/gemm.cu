@@ -249,7 +249,7 @@ template <> const double2* proj_ptr<double>(const KSphere& sp) { return (const d
 template <> const float2* proj_ptr<float>(const KSphere& sp) { return (const float2*)sp.P32; }
 
 bool nonlocal_small(const KSphere& sp, int nb, jdft_prec prec) {
-    if (prec == JDFT_FP64) return !sl_eligible(sp.nproj, nb, sp.npw) && !sl_eligible(sp.npw, nb, sp.nproj);
+    if (prec == JDFT_FP64) return !sl_eligible(sp.nproj, nb, sp.npw);
     return !tcx_eligible(prec, sp.nproj, nb) && (size_t)sp.nproj * nb * sp.npw < (size_t)64 << 20;
 }
 

@@ -106,8 +106,9 @@ jdft_status nonlocal_accumulate(const KSphere& sp, const void* C, int ldc, void*
                                 jdft_prec prec, void* work, cudaStream_t st, bool split_c = false,
                                 const void* Csplit = nullptr, bool partials = false,
                                 ProductScratch* scratch = nullptr, int phases = kNonlocalBoth);
-// Whether both products of the nonlocal term are too small for the split-operand and
-// sliced kernels: then neither part of H C fills the GPU.
+// Whether D P^dag C is too small for the split-operand and sliced kernels: it then
+// does not fill the GPU, and runs beside the chain (FP64: whatever adds P (D P^dag C);
+// 16 bands and 64 projectors of 19 778 plane waves 605 -> 562 us).
 bool nonlocal_small(const KSphere& sp, int nb, jdft_prec prec);
 
 }  // namespace jdft

@@ -484,12 +484,19 @@ static size_t sl_block_bytes(int rows_pad, int K) {
 constexpr size_t SL_BUDGET = size_t(1) << 30;
 
 // Whether the slices are the faster way: estimated times of both (microseconds).
-// Slices: the launches, 52 bytes a value of both operands at 3.5 TB/s, and 360 MK N
-// flops of the padded tiles at 1 PFLOP/s; CUDA cores: 8 M N K flops at 0.9 TFLOP/s.
+// Slices: 54 for the launches, reading both operands twice and writing their padded
+// slices at 3.5 TB/s, and per tile of 128 rows 3.6 ns a K and, for five blocks' start
+// and end, 4 us on each of 152 SMs.  CUDA cores: 10 for the launch and 8 flops a padded
+// output and K at 1 TFLOP/s.  Measured (conj(A) B of 4 259 plane waves, CUDA cores /
+// slices): 32 x 32 50 / 67, 40 x 40 108 / 67; of 19 778: 16 x 16 53 / 154, 32 x 32
+// 165 / 160; H C with 128 projectors on 4 259: 16 bands 193 / 225, 32 bands 364 / 274.
 bool sl_eligible(int M, int N, int K) {
-    const double NT = sl_nt(N), m = tcx_rows_pad(M), n = (N + NT - 1) / NT * NT, k = K;
-    const double slices = 25.0 + (m + n) * k * 52.0 / 3.5e6 + m * n * k * 360.0 / 1e9;
-    return slices < 8.0 * M * (double)N * k / 0.9e6;
+    const int NT = sl_nt(N), ntiles = (N + NT - 1) / NT;
+    const double m = tcx_rows_pad(M), n = (double)ntiles * NT, k = K, tiles = m / TCX_M * ntiles;
+    const double slices = 54.0 + (36.0 * (m + n) + 32.0 * ((double)M + N)) * k / 3.5e6 +
+                          tiles * (3.6e-3 * k + 5 * 4.0 / 152);
+    const double M16 = (M + 15) / 16 * 16, N16 = (N + 15) / 16 * 16;
+    return slices < 10.0 + 8.0 * M16 * N16 * k / 1.0e6;
 }
 
 template <int NT, bool CONJ>
