@@ -390,6 +390,7 @@ jdft_status jdft_basis_create(const jdft_cell_desc* desc, jdft_basis_t* out) {
     jdft_status st = JDFT_OK;
     for (int ik = 0; ik < b->nk && st == JDFT_OK; ++ik) st = build_sphere(b, ik);
     if (st == JDFT_OK) st = build_twiddles(b);
+    if (st == JDFT_OK) st = side_stream(b);  // H C of small blocks uses it: 14 us of a first call otherwise
     if (st != JDFT_OK) {
         std::string msg = jdft_last_error();
         jdft_basis_destroy(b);

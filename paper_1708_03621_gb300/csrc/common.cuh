@@ -189,7 +189,7 @@ struct jdft_basis_s {
 namespace jdft {
 // Grows the basis workspace to at least `bytes` (synchronous cudaMalloc).
 jdft_status ensure_workspace(jdft_basis_s* b, size_t bytes);
-// Creates the basis's side stream and its fork and join events on first use.
+// Creates the basis's side stream and its fork and join events where they are missing.
 jdft_status side_stream(jdft_basis_s* b);
 // The same for any library-owned workspace of the basis.
 jdft_status ensure_ws(Workspace& w, size_t bytes);

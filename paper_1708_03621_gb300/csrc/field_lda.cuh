@@ -47,37 +47,38 @@ static __device__ __noinline__ void lda_pz_plain(double n, double& e, double& v)
     v = (4.0 * third) * ex + vc;
 }
 
-// The same with the FP64 pipe's work cut to about 30 instructions where r_s >= 1
+// The same with the FP64 pipe's work cut to about 25 instructions where r_s >= 1
 // (n <= 0.2387, nearly every point of a cell): t = n^(-1/6) from an FP32 estimate
-// with one step of Householder's method (e = 1 - n t^6 is below 2^-16, the terms
-// kept reach e^3), from which n^(1/3), r_s and its square root are products, and
-// the reciprocal of the fit's denominator from an FP32 one with two terms of the
-// geometric series.  What bounds the epilogue is still the FP64 pipe: 30
-// instructions for each of two million points are 107 us of a 128^3 box.
+// with one step of Householder's method (d = 1 - n t^6 is below 2^-16, the terms
+// kept reach d^3), from which n^(1/3) and the fit in t (sqrt(r_s) and r_s are
+// multiples of t and t^2) are products, and the reciprocal of the fit's denominator
+// from an FP32 one with two terms of the geometric series.  What bounds the epilogue
+// is still the FP64 pipe: 25 instructions for each of two million points are 90 us of
+// a 128^3 box.  Emulated against 80 bits, e and v are off by 0.7 to 0.9 units of 2^-53
+// (root mean square), as the plain form is with a correctly rounded cube root.
 __device__ __forceinline__ void lda_pz(double n, double& e, double& v) {
     if (!(n > 1e-30 && n < 0.23)) { lda_pz_plain(n, e, v); return; }
     const double cx = -0.73855876638202240588423003065;
-    const double kr = 0.62035049089940001666800681204778;
-    const double ks = 0.7876233178997433;  // sqrt(kr)
-    const double g = -0.1423, b1 = 1.0529, b2 = 0.3334;
+    const double g = -0.1423;
+    const double p1 = 0.82928859141663966846;  // b1 sqrt(kr) and b2 kr of the plain form
+    const double p2 = 0.20682485366585996556;
     const double t0 = long_of(exp2f(__log2f(short_of(n)) * (-1.0f / 6.0f)));
-    const double s0 = t0 * t0;  // exact: t0 has 24 bits
-    const double t3 = s0 * t0;
-    const double d = fma(-(n * t3), t3, 1.0);
+    const double t3 = (t0 * t0) * t0;  // the square is exact: t0 has 24 bits
+    const double w = n * t3;
+    const double d = fma(-w, t3, 1.0);
     // t = t0 (1 - d)^(-1/6) and n^(1/3) = n t0^4 (1 - d)^(-2/3), each by its own series: the
-    // fourth power of t would multiply its rounding by four
+    // fourth power of t would multiply its rounding by four.  n t0^4 is formed from d's own
+    // n t0^3, whose roundings d takes out again but for a third.
     const double t = fma(t0, d * fma(d, fma(d, 91.0 / 1296.0, 7.0 / 72.0), 1.0 / 6.0), t0);
-    const double c0 = n * (s0 * s0);
+    const double c0 = w * t0;
     const double c = fma(c0, d * fma(d, fma(d, 40.0 / 81.0, 5.0 / 9.0), 2.0 / 3.0), c0);
-    const double t2 = t * t;
-    const double sq = ks * t, rb = b2 * (kr * t2);
-    const double den = fma(b1, sq, 1.0 + rb);
+    const double den = fma(fma(t, p2, p1), t, 1.0);
     double r = long_of(__fdividef(1.0f, short_of(den)));
     const double f = fma(-den, r, 1.0);
     r = fma(r, fma(f, f, f), r);
     const double ec = g * r;
     // v_c = e_c - (r_s/3) de_c/dr_s = e_c (1 + (b1 sqrt(r_s)/2 + b2 r_s) / (3 den))
-    const double vc = ec * fma((1.0 / 3.0) * fma(0.5 * b1, sq, rb), r, 1.0);
+    const double vc = fma(ec * (t * r), fma(t, p2 / 3.0, p1 / 6.0), ec);
     e = fma(cx, c, ec);
     v = fma((4.0 / 3.0) * cx, c, vc);
 }

@@ -851,11 +851,9 @@ namespace jdft {
 static size_t r256(size_t x) { return (x + 255) / 256 * 256; }
 
 jdft_status side_stream(jdft_basis_s* b) {
-    if (!b->side) {
-        JDFT_CUDA_TRY(cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking));
-        JDFT_CUDA_TRY(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
-        JDFT_CUDA_TRY(cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming));
-    }
+    if (!b->ev_fork) JDFT_CUDA_TRY(cudaEventCreateWithFlags(&b->ev_fork, cudaEventDisableTiming));
+    if (!b->ev_join) JDFT_CUDA_TRY(cudaEventCreateWithFlags(&b->ev_join, cudaEventDisableTiming));
+    if (!b->side) JDFT_CUDA_TRY(cudaStreamCreateWithFlags(&b->side, cudaStreamNonBlocking));
     return JDFT_OK;
 }
 
