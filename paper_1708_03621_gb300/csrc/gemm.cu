@@ -14,7 +14,7 @@ namespace jdft {
 
 // ---------------------------------------------------------------------------
 // C^dag-style product with split K, for the shapes whose FP64 products are too
-// small for the sliced ones and for FP32 blocks.  FP64: bound by the FP64 pipe (2
+// small for the sliced ones.  FP64: bound by the FP64 pipe (2
 // multiply-adds per clock and SM), so what counts is that every SM has work and
 // no lane multiplies padding.  A block of four warps holds a TM x TN tile (16 or
 // 32 each way, whichever pads less) and a range of K in chunks of 32; each warp
@@ -125,9 +125,108 @@ static jdft_status launch_zgemm_cn(int M, int N, int K, const c_t<T>* A, int lda
     return check_launch("zgemm_cn");
 }
 
-template <typename T>
-jdft_status zgemm_cn(int M, int N, int K, const c_t<T>* A, int lda, const c_t<T>* B, int ldb, double2* out, int ldo,
-                     double scale, cudaStream_t st) {
+// FP32 blocks: the multiply-adds are cheap and latency counts, so a block of eight
+// warps shares its staged K (16 deep), each thread with P x P outputs of a 16 P square
+// tile, four blocks to an SM.  The tiles above, with four warps a block and two blocks
+// an SM, tie with P = 2 at 44 x 13 over 6 600 plane waves (18.6 us) and lose on large
+// blocks (spinor H C of 64 bands on 128^3 with 256 projectors 3.29 ms; with P = 4 here
+// and cgemm_nn_kernel below 2.08 ms).
+constexpr int CNF_BK = 16;
+
+template <int P>
+__global__ void __launch_bounds__(256)
+    cgemm_cn_kernel(int M, int N, int K, int kchunk, const float2* __restrict__ A, int lda, const float2* __restrict__ B,
+                    int ldb, double2* __restrict__ out, int ldo, double scale) {
+    constexpr int TILE = 16 * P;
+    __shared__ float2 As[CNF_BK][TILE + 1];
+    __shared__ float2 Bs[CNF_BK][TILE + 1];
+    const int m0 = blockIdx.x * TILE, n0 = blockIdx.y * TILE;
+    const int kA = blockIdx.z * kchunk, kB = min(K, kA + kchunk);
+    const int tm = threadIdx.x / 16, tn = threadIdx.x % 16;
+    float2 acc[P][P];
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+#pragma unroll
+        for (int j = 0; j < P; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    for (int k0 = kA; k0 < kB; k0 += CNF_BK) {
+#pragma unroll
+        for (int e = threadIdx.x; e < TILE * CNF_BK; e += 256) {
+            const int r = e / CNF_BK, kk = e % CNF_BK;
+            const int m = m0 + r, n = n0 + r, k = k0 + kk;
+            As[kk][r] = (m < M && k < kB) ? A[(size_t)m * lda + k] : make_float2(0.f, 0.f);
+            Bs[kk][r] = (n < N && k < kB) ? B[(size_t)n * ldb + k] : make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < CNF_BK; ++kk) {
+            float2 a[P], b[P];
+#pragma unroll
+            for (int i = 0; i < P; ++i) a[i] = As[kk][tm + 16 * i];
+#pragma unroll
+            for (int j = 0; j < P; ++j) b[j] = Bs[kk][tn + 16 * j];
+#pragma unroll
+            for (int i = 0; i < P; ++i)
+#pragma unroll
+                for (int j = 0; j < P; ++j) {
+                    if constexpr (P == 2) {
+                        // the shorter chain: four outputs a thread hardly hide two additions in a row (two
+                        // products of 32 x 32 over 19 808: 41.5 us, 47.9 with the form below; H C of 4 bands
+                        // with 256 projectors on 62 759 the other way, 308 and 280)
+                        acc[i][j].x += a[i].x * b[j].x + a[i].y * b[j].y;
+                        acc[i][j].y += a[i].x * b[j].y - a[i].y * b[j].x;
+                    } else {
+                        acc[i][j].x = mad(a[i].y, b[j].y, mad(a[i].x, b[j].x, acc[i][j].x));
+                        acc[i][j].y = mad(-a[i].y, b[j].x, mad(a[i].x, b[j].y, acc[i][j].y));
+                    }
+                }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < P; ++i)
+#pragma unroll
+        for (int j = 0; j < P; ++j) {
+            const int m = m0 + tm + 16 * i, n = n0 + tn + 16 * j;
+            if (m < M && n < N) {
+                atomicAdd(&out[(size_t)m * ldo + n].x, scale * (double)acc[i][j].x);
+                atomicAdd(&out[(size_t)m * ldo + n].y, scale * (double)acc[i][j].y);
+            }
+        }
+}
+
+template <int P>
+static jdft_status launch_cgemm_cn(int M, int N, int K, const float2* A, int lda, const float2* B, int ldb, double2* out,
+                                   int ldo, double scale, cudaStream_t st) {
+    constexpr int TILE = 16 * P;
+    const int mt = (M + TILE - 1) / TILE, nt = (N + TILE - 1) / TILE;
+    // enough K splits for about 4 blocks per SM, each at least 64 deep
+    int splits = std::max(1, (152 * 4 + mt * nt - 1) / (mt * nt));
+    splits = std::min(splits, std::max(1, K / 64));
+    int kchunk = (K + splits - 1) / splits;
+    kchunk = (kchunk + CNF_BK - 1) / CNF_BK * CNF_BK;
+    splits = (K + kchunk - 1) / kchunk;
+    {
+        Trace tr_("zgemm_cn", st);
+        cgemm_cn_kernel<P><<<dim3(mt, nt, splits), 256, 0, st>>>(M, N, K, kchunk, A, lda, B, ldb, out, ldo, scale);
+    }
+    return check_launch("zgemm_cn");
+}
+
+template <>
+jdft_status zgemm_cn<float>(int M, int N, int K, const float2* A, int lda, const float2* B, int ldb, double2* out,
+                            int ldo, double scale, cudaStream_t st) {
+    if (M == 0 || N == 0 || K == 0) return JDFT_OK;
+    // 64-wide tiles where they are more than half full both ways and the product is long enough for
+    // their larger blocks (two products, P = 2 / 4: 64 x 64 over 4 259 34 / 49 us, over 19 808 67 / 74,
+    // over 62 759 156 / 154; 128 x 128 over 19 808 190 / 155, over 62 759 604 / 436)
+    if (M > 32 && N > 32 && (double)M * N * K > 1e8) return launch_cgemm_cn<4>(M, N, K, A, lda, B, ldb, out, ldo, scale, st);
+    return launch_cgemm_cn<2>(M, N, K, A, lda, B, ldb, out, ldo, scale, st);
+}
+
+template <>
+jdft_status zgemm_cn<double>(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* out,
+                             int ldo, double scale, cudaStream_t st) {
+    using T = double;
     if (M == 0 || N == 0 || K == 0) return JDFT_OK;
     // 16-wide tiles where a 32-wide one would be at most half full at the edge
     const bool m16 = (M - 1) % 32 < 16, n16 = (N - 1) % 32 < 16;
@@ -188,6 +287,65 @@ __global__ void __launch_bounds__(32 * NN_WARPS)
     }
 }
 
+// FP32 blocks on many plane waves: A's tile staged as well, 256 threads of 2 m x 8 n
+// each (128 x 32 outputs a block), so that A is read once per 32 columns instead of
+// once per 16 and a shared-memory read feeds 6 multiply-adds (FP32 H C of 64 bands with
+// 256 projectors on 62 759 plane waves, both products: 1 179 -> 993 us against 64 m x
+// 16 n a block).
+constexpr int NNF_BM = 128, NNF_BN = 32, NNF_BK = 16;
+
+__global__ void __launch_bounds__(256)
+    cgemm_nn_kernel(int M, int N, int K, const float2* __restrict__ A, int lda, const float2* __restrict__ Bm, int ldb,
+                    float2* __restrict__ out, int ldo, bool accumulate) {
+    __shared__ float2 As[NNF_BK][NNF_BM];
+    __shared__ float2 Bs[NNF_BK][NNF_BN];
+    const int m0 = blockIdx.x * NNF_BM, n0 = blockIdx.y * NNF_BN;
+    const int tm = threadIdx.x % 64, tq = threadIdx.x / 64;  // rows tm and tm + 64, columns 8 tq .. 8 tq + 7
+    float2 acc[2][8];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) acc[i][j] = make_float2(0.f, 0.f);
+    for (int k0 = 0; k0 < K; k0 += NNF_BK) {
+#pragma unroll
+        for (int e = threadIdx.x; e < NNF_BK * NNF_BM; e += 256) {
+            const int kk = e / NNF_BM, r = e % NNF_BM;
+            const int m = m0 + r, k = k0 + kk;
+            As[kk][r] = (m < M && k < K) ? A[(size_t)k * lda + m] : make_float2(0.f, 0.f);
+        }
+#pragma unroll
+        for (int e = threadIdx.x; e < NNF_BK * NNF_BN; e += 256) {
+            const int kk = e / NNF_BN, c = e % NNF_BN;
+            const int n = n0 + c, k = k0 + kk;
+            Bs[kk][c] = (n < N && k < K) ? Bm[(size_t)k * ldb + n] : make_float2(0.f, 0.f);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int kk = 0; kk < NNF_BK; ++kk) {
+            const float2 a0 = As[kk][tm], a1 = As[kk][tm + 64];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const float2 b = Bs[kk][tq * 8 + j];
+                acc[0][j].x = mad(-a0.y, b.y, mad(a0.x, b.x, acc[0][j].x));
+                acc[0][j].y = mad(a0.y, b.x, mad(a0.x, b.y, acc[0][j].y));
+                acc[1][j].x = mad(-a1.y, b.y, mad(a1.x, b.x, acc[1][j].x));
+                acc[1][j].y = mad(a1.y, b.x, mad(a1.x, b.y, acc[1][j].y));
+            }
+        }
+        __syncthreads();
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const int m = m0 + tm + 64 * i;
+        if (m >= M) continue;
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            const int n = n0 + tq * 8 + j;
+            if (n < N) out[(size_t)n * ldo + m] = accumulate ? cadd(out[(size_t)n * ldo + m], acc[i][j]) : acc[i][j];
+        }
+    }
+}
+
 template <typename T>
 jdft_status zgemm_nn_acc(int M, int N, int K, const c_t<T>* A, int lda, const c_t<T>* Bm, int ldb, c_t<T>* out,
                          int ldo, cudaStream_t st, bool accumulate) {
@@ -197,6 +355,17 @@ jdft_status zgemm_nn_acc(int M, int N, int K, const c_t<T>* A, int lda, const c_
             for (int n = 0; n < N; ++n)
                 JDFT_CUDA_TRY(cudaMemsetAsync(out + (size_t)n * ldo, 0, (size_t)M * sizeof(c_t<T>), st));
         return JDFT_OK;
+    }
+    if constexpr (std::is_same<T, float>::value) {
+        // two blocks for every SM, and more than half of the 32 columns
+        const int mt = (M + NNF_BM - 1) / NNF_BM, nt = (N + NNF_BN - 1) / NNF_BN;
+        if (N > 16 && (int64_t)mt * nt >= 304) {
+            {
+                Trace tr_("zgemm_nn", st);
+                cgemm_nn_kernel<<<dim3(mt, nt), 256, 0, st>>>(M, N, K, A, lda, Bm, ldb, out, ldo, accumulate);
+            }
+            return check_launch("zgemm_nn");
+        }
     }
     dim3 grid((M + NN_BM - 1) / NN_BM, (N + NN_BN - 1) / NN_BN);
     {
@@ -335,10 +504,6 @@ jdft_status gemm_nn_acc<float>(jdft_prec prec, int M, int N, int K, const float2
     return zgemm_nn_acc<float>(M, N, K, A, lda, Bm, ldb, out, ldo, st, accumulate);
 }
 
-template jdft_status zgemm_cn<double>(int, int, int, const double2*, int, const double2*, int, double2*, int, double,
-                                      cudaStream_t);
-template jdft_status zgemm_cn<float>(int, int, int, const float2*, int, const float2*, int, double2*, int, double,
-                                     cudaStream_t);
 template jdft_status zgemm_nn_acc<double>(int, int, int, const double2*, int, const double2*, int, double2*, int,
                                           cudaStream_t, bool);
 template jdft_status zgemm_nn_acc<float>(int, int, int, const float2*, int, const float2*, int, float2*, int,
