@@ -42,7 +42,8 @@ constexpr int SL_PLANES = 2 * SL_N;     // Re and Im of each slice
 constexpr int SL_STAGES = 4;
 constexpr int SL_RUN = 3;               // slices per stage and operand, one copy each
 constexpr int SL_THREADS = 128;
-constexpr int SL_BAD = 1 << 20;         // row exponent of a row with an infinity or NaN
+constexpr int SL_BIAS = 1 << 13;        // of stored exponents (0: none)
+constexpr int SL_BAD = 1 << 20;         // exponent of a row with an infinity or NaN
 __host__ __device__ constexpr int sl_top(int g) { return 10 - 2 * g; }              // larger digit sum of group g
 __host__ __device__ constexpr int sl_limit(int g) { return 2048 / (sl_top(g) - 1) / TCX_KC; }  // K chunks per unit
 
@@ -54,37 +55,45 @@ struct SlPlan {
 };
 
 // ---- row maxima -------------------------------------------------------------
-// maxhi[r] = largest high word of |Re|, |Im| over the row's K values.
+// Exponents are exponent fields (1 for zeros and denormals, whose significands have no
+// implicit bit) plus SL_BIAS, so that 0 means none.  `shift` scales the summed index: value
+// k counts as 2^(sign (shift[k] - SL_BIAS)) times itself, with sign -1 for one operand and
+// +1 for the other (see sl_zgemm_nn).
+__device__ __forceinline__ int sl_field(int hi) { return max((hi >> 20) & 0x7ff, 1); }
+__device__ __forceinline__ int sl_shift(const int* __restrict__ shift, int sign, int k) {
+    return shift ? sign * (shift[k] - SL_BIAS) : 0;
+}
+// The exponent that a row of largest component v has at least: SL_BAD for an infinity or NaN.
+__device__ __forceinline__ int sl_exponent(double2 v, int shift) {
+    const int x = __double2hiint(v.x) & 0x7fffffff, y = __double2hiint(v.y) & 0x7fffffff, hi = max(x, y);
+    if ((hi >> 20) == 0x7ff) return SL_BAD;
+    return (hi | __double2loint(v.x) | __double2loint(v.y)) == 0 ? 0 : sl_field(hi) + shift + SL_BIAS;
+}
+
+// ex[r] = largest exponent over the row's K values (FINITE: of those without an infinity or NaN).
+template <bool FINITE>
 __global__ void __launch_bounds__(256) sl_rowmax_kernel(const double2* __restrict__ X, size_t ld, int K,
-                                                        int* __restrict__ maxhi) {
+                                                        const int* __restrict__ shift, int sign,
+                                                        int* __restrict__ ex) {
     const double2* x = X + (size_t)blockIdx.x * ld;
     int m = 0;
     for (int k = blockIdx.y * blockDim.x + threadIdx.x; k < K; k += gridDim.y * blockDim.x) {
-        const double2 v = x[k];
-        m = max(m, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
+        const int e = sl_exponent(x[k], sl_shift(shift, sign, k));
+        if (!FINITE || e != SL_BAD) m = max(m, e);
     }
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(&maxhi[blockIdx.x], m);
+    if ((threadIdx.x & 31) == 0) atomicMax(&ex[blockIdx.x], m);
 }
 // The same of the transpose: row r, value k at X[k * ld + r]; blockIdx.y strides over k.
 __global__ void __launch_bounds__(256) sl_rowmax_t_kernel(const double2* __restrict__ X, size_t ld, int rows, int K,
-                                                          int* __restrict__ maxhi) {
+                                                          const int* __restrict__ shift, int sign,
+                                                          int* __restrict__ ex) {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= rows) return;
     int m = 0;
-    for (int k = blockIdx.y; k < K; k += gridDim.y) {
-        const double2 v = X[(size_t)k * ld + r];
-        m = max(m, max(__double2hiint(v.x) & 0x7fffffff, __double2hiint(v.y) & 0x7fffffff));
-    }
-    atomicMax(&maxhi[r], m);
-}
-
-// Biased exponent of a row's largest value and whether its values are scaled
-// by 2^512 first (rows below 2^-959, whose products would lose bits otherwise).
-__device__ __forceinline__ int sl_exponent(int maxhi, bool& up) {
-    const int e = maxhi >> 20;
-    up = maxhi > 0 && e < 64;
-    return up ? max(e, 1) + 512 : max(e, 64);
+    for (int k = blockIdx.y; k < K; k += gridDim.y)
+        m = max(m, sl_exponent(X[(size_t)k * ld + r], sl_shift(shift, sign, k)));
+    atomicMax(&ex[r], m);
 }
 
 // ---- slices -------------------------------------------------------------------
@@ -98,7 +107,8 @@ __device__ __forceinline__ int sl_exponent(int maxhi, bool& up) {
 // each of the 18 planes.
 template <bool TRANS>
 __global__ void __launch_bounds__(256) sl_slice_kernel(const double2* __restrict__ X, size_t ld, int rows, int K,
-                                                       int rows_pad, int RB, int nkc, const int* __restrict__ maxhi,
+                                                       int rows_pad, int RB, int nkc, const int* __restrict__ ex,
+                                                       const int* __restrict__ shift, int sign,
                                                        __nv_bfloat16* __restrict__ out) {
     const int per_chunk = rows_pad * 2;
     const int64_t total = (int64_t)per_chunk * nkc;
@@ -112,23 +122,23 @@ __global__ void __launch_bounds__(256) sl_slice_kernel(const double2* __restrict
         // the digits' offsets: 64 in each place makes them non-negative
         constexpr uint64_t kOffset = 64ull * ((1ull << 0) + (1ull << 7) + (1ull << 14) + (1ull << 21) + (1ull << 28) +
                                               (1ull << 35) + (1ull << 42) + (1ull << 49) + (1ull << 56));
-        bool up;
-        const int emax = sl_exponent(r < rows ? maxhi[r] : 0, up);
-        const double f = up ? __hiloint2double((1023 + 512) << 20, 0) : 1.0;
+        const int emax = r < rows ? ex[r] - SL_BIAS : 0;
 #pragma unroll
         for (int j = 0; j < 8; ++j) {
             double2 v = make_double2(0.0, 0.0);
-            if (r < rows && k0 + j < K) v = TRANS ? X[(size_t)(k0 + j) * ld + r] : X[(size_t)r * ld + k0 + j];
-            if (up) {
-                v.x *= f;
-                v.y *= f;
+            int sh = 0;
+            if (r < rows && k0 + j < K) {
+                v = TRANS ? X[(size_t)(k0 + j) * ld + r] : X[(size_t)r * ld + k0 + j];
+                sh = sl_shift(shift, sign, k0 + j);
             }
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
                 const double x = c ? v.y : v.x;
                 const int hi = __double2hiint(x);
-                const int n = min(emax - ((hi >> 20) & 0x7ff), 63);
-                const uint64_t m = ((uint64_t)(uint32_t)((hi & 0xfffff) | 0x100000) << 32) | (uint32_t)__double2loint(x);
+                // (a zero may lie above its row's exponent: as unsigned, the shift is then 63 too)
+                const int n = (int)min((uint32_t)(emax - sl_field(hi) - sh), 63u);
+                const uint64_t m = ((uint64_t)(uint32_t)((hi & 0xfffff) | ((hi & 0x7ff00000) ? 0x100000 : 0)) << 32) |
+                                   (uint32_t)__double2loint(x);
                 const int64_t t = (int64_t)((m << 8) >> n), s = (int64_t)(hi >> 31);
                 d[c][j] = (uint64_t)((t ^ s) - s) + kOffset;
             }
@@ -392,7 +402,7 @@ __device__ __forceinline__ double sl_to_double(__int128 t, int q) {
 template <int RZ>
 __global__ void __launch_bounds__(TCX_M* RZ)
     sl_reduce_kernel(const int2* __restrict__ part, SlPlan plan, int NT, int mtiles, int M, int N,
-                     const int* __restrict__ maxA, const int* __restrict__ maxB, double2* __restrict__ out, size_t sm,
+                     const int* __restrict__ exA, const int* __restrict__ exB, double2* __restrict__ out, size_t sm,
                      size_t sn, double scale, int accumulate) {
     __shared__ longlong2 sum[RZ > 1 ? RZ : 1][2][RZ > 1 ? TCX_M : 1];
     const int r = threadIdx.x, q = threadIdx.y;
@@ -429,13 +439,11 @@ __global__ void __launch_bounds__(TCX_M* RZ)
         }
     }
     if (m >= M) return;
-    bool upA, upB;
-    const int hA = maxA[m], hB = maxB[n];
-    // rows scaled so that 2^(e - 61) is the unit, e = biased exponent - 1022; sums in units of 2^56 of their product
-    const int eA = sl_exponent(hA, upA) - 1022, eB = sl_exponent(hB, upB) - 1022;
-    const int w = eA + eB - 2 * 61 + 56 - (upA ? 512 : 0) - (upB ? 512 : 0);
+    // a slice's last digit is worth 2^(exponent - 1083) of its row, the sums are in units of 2^56 of their product
+    const int eA = exA[m], eB = exB[n];
+    const int w = (eA - SL_BIAS - 1083) + (eB - SL_BIAS - 1083) + 56;
     double2 v = make_double2(scale * sl_to_double(re, w), scale * sl_to_double(im, w));
-    if ((hA >> 20) == 0x7ff || (hB >> 20) == 0x7ff) v.x = v.y = __hiloint2double(0x7ff80000, 0);
+    if (eA == SL_BAD || eB == SL_BAD) v.x = v.y = __hiloint2double(0x7ff80000, 0);
     double2* o = out + (size_t)m * sm + (size_t)n * sn;
     if (accumulate) {
         const double2 old = *o;
@@ -514,8 +522,8 @@ static jdft_status sl_launch_nt(const void* As, const void* Bs, int nrbA, int nr
 }
 
 template <bool CONJ>
-static jdft_status sl_product(const void* As, const void* Bs, int M, int N, int NT, int nkc, const int* maxA,
-                              const int* maxB, void* partial, double2* out, size_t sm, size_t sn, double scale,
+static jdft_status sl_product(const void* As, const void* Bs, int M, int N, int NT, int nkc, const int* exA,
+                              const int* exB, void* partial, double2* out, size_t sm, size_t sn, double scale,
                               bool accumulate, cudaStream_t st) {
     const int mtiles = tcx_rows_pad(M) / TCX_M, ntiles = (N + NT - 1) / NT, tiles = mtiles * ntiles;
     const SlPlan plan = sl_plan(nkc, tiles);
@@ -529,44 +537,45 @@ static jdft_status sl_product(const void* As, const void* Bs, int M, int N, int 
         Trace tr_("sl_reduce", st);
         const dim3 grid(std::min(NT, N), tiles);
         if (plan.first[SL_GROUPS] > 24)
-            sl_reduce_kernel<8><<<grid, dim3(TCX_M, 8), 0, st>>>(part, plan, NT, mtiles, M, N, maxA, maxB, out, sm, sn,
+            sl_reduce_kernel<8><<<grid, dim3(TCX_M, 8), 0, st>>>(part, plan, NT, mtiles, M, N, exA, exB, out, sm, sn,
                                                                  scale, accumulate);
         else
-            sl_reduce_kernel<1><<<grid, dim3(TCX_M, 1), 0, st>>>(part, plan, NT, mtiles, M, N, maxA, maxB, out, sm, sn,
+            sl_reduce_kernel<1><<<grid, dim3(TCX_M, 1), 0, st>>>(part, plan, NT, mtiles, M, N, exA, exB, out, sm, sn,
                                                                  scale, accumulate);
     }
     return check_launch("sl_reduce");
 }
 
-// Row maxima and slices of an operand (K values a row; trans: X[k * ld + r]), its
-// rows padded to blocks of RB.
-static jdft_status sl_slice(const double2* X, size_t ld, int rows, int RB, int K, bool trans, int* maxhi,
-                            void* slices, cudaStream_t st) {
-    JDFT_CUDA_TRY(cudaMemsetAsync(maxhi, 0, (size_t)rows * sizeof(int), st));
+// Exponents of an operand's rows (K values a row; trans: X[k * ld + r]).
+static jdft_status sl_exponents(const double2* X, size_t ld, int rows, int K, bool trans, const int* shift, int sign,
+                                int* ex, cudaStream_t st, bool finite = false) {
+    JDFT_CUDA_TRY(cudaMemsetAsync(ex, 0, (size_t)rows * sizeof(int), st));
+    Trace tr_("sl_rowmax", st);
+    if (trans) {
+        const int bx = (rows + 255) / 256;
+        sl_rowmax_t_kernel<<<dim3(bx, std::max(1, std::min(K, 152 * 8 / bx))), 256, 0, st>>>(X, ld, rows, K, shift,
+                                                                                            sign, ex);
+    } else {
+        const dim3 grid(rows, std::max(1, std::min((K + 1023) / 1024, 152 * 8 / rows)));
+        if (finite) sl_rowmax_kernel<true><<<grid, 256, 0, st>>>(X, ld, K, shift, sign, ex);
+        else sl_rowmax_kernel<false><<<grid, 256, 0, st>>>(X, ld, K, shift, sign, ex);
+    }
+    return check_launch("sl_rowmax");
+}
+
+// Slices of an operand from its rows' exponents, its rows padded to blocks of RB.
+static jdft_status sl_slice(const double2* X, size_t ld, int rows, int RB, int K, bool trans, const int* shift,
+                            int sign, const int* ex, void* slices, cudaStream_t st) {
     const int nkc = tcx_chunks(K), rows_pad = (rows + RB - 1) / RB * RB;
     const int64_t total = (int64_t)rows_pad * 2 * nkc;
     const int grid = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
-    {
-        Trace tr_("sl_rowmax", st);
-        if (trans) {
-            const int bx = (rows + 255) / 256;
-            sl_rowmax_t_kernel<<<dim3(bx, std::max(1, std::min(K, 152 * 8 / bx))), 256, 0, st>>>(X, ld, rows, K, maxhi);
-        } else {
-            sl_rowmax_kernel<<<dim3(rows, std::max(1, std::min((K + 1023) / 1024, 152 * 8 / rows))), 256, 0, st>>>(
-                X, ld, K, maxhi);
-        }
-    }
-    jdft_status s = check_launch("sl_rowmax");
-    if (s != JDFT_OK) return s;
-    {
-        Trace tr_("sl_slice", st);
-        if (trans)
-            sl_slice_kernel<true><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, RB, nkc, maxhi,
-                                                        (__nv_bfloat16*)slices);
-        else
-            sl_slice_kernel<false><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, RB, nkc, maxhi,
-                                                         (__nv_bfloat16*)slices);
-    }
+    Trace tr_("sl_slice", st);
+    if (trans)
+        sl_slice_kernel<true><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, RB, nkc, ex, shift, sign,
+                                                    (__nv_bfloat16*)slices);
+    else
+        sl_slice_kernel<false><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, RB, nkc, ex, shift, sign,
+                                                     (__nv_bfloat16*)slices);
     return check_launch("sl_slice");
 }
 
@@ -586,29 +595,41 @@ jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const do
     void* ws = scratch.get(std::max(bytes(kp), K % kp ? bytes(K % kp) : 0));
     if (!ws) return JDFT_ERR_UNSUPPORTED;
     jdft_status s;
-    int* maxA = (int*)ws;
-    int* maxB = same ? maxA : maxA + M;
+    int* exA = (int*)ws;
+    int* exB = same ? exA : exA + M;
     for (int k0 = 0; k0 < K; k0 += kp) {
         const int k = std::min(kp, K - k0);
         char* As = (char*)ws + mx;
         char* Bs = same ? As : As + sl_block_bytes(rpA, k);
         char* part = Bs + sl_block_bytes(rpB, k);
-        if ((s = sl_slice(A + k0, lda, M, TCX_M, k, false, maxA, As, st))) return s;
-        if (!same && (s = sl_slice(B + k0, ldb, N, NT, k, false, maxB, Bs, st))) return s;
-        if ((s = sl_product<true>(As, Bs, M, N, NT, tcx_chunks(k), maxA, maxB, part, out, ldo, 1, scale, true, st)))
+        if ((s = sl_exponents(A + k0, lda, M, k, false, nullptr, 0, exA, st))) return s;
+        if ((s = sl_slice(A + k0, lda, M, TCX_M, k, false, nullptr, 0, exA, As, st))) return s;
+        if (!same) {
+            if ((s = sl_exponents(B + k0, ldb, N, k, false, nullptr, 0, exB, st))) return s;
+            if ((s = sl_slice(B + k0, ldb, N, NT, k, false, nullptr, 0, exB, Bs, st))) return s;
+        }
+        if ((s = sl_product<true>(As, Bs, M, N, NT, tcx_chunks(k), exA, exB, part, out, ldo, 1, scale, true, st)))
             return s;
     }
     return JDFT_OK;
 }
 
+// The summed index is scaled first: column k of A by 2^-s_k and row k of B by 2^s_k, s_k the
+// exponent of the column's largest value (exponents only, so exact).  A row of A is one plane
+// wave over all bands or projectors, and their norms may be anything: cut against the largest
+// of them, a small band's coefficients would lose the bits that its large entries of B bring
+// back (bands with norms spread over 1e12, rotated by L^-dag, came out orthonormal to 7e-7).
+// Scaled, the columns of A are alike, and each column of the output is off by 2^-60 of its own
+// largest contributions, whatever the scales.  It costs one more reading of A.
 jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const double2* Bm, int ldb, double2* out,
                         int ldo, bool accumulate, ProductScratch& scratch, cudaStream_t st) {
     const int NT = sl_nt(N);
     const int rpB = (N + NT - 1) / NT * NT;
     const int nkc = tcx_chunks(K);
+    const size_t head = sl_align((size_t)(M + N + K) * sizeof(int));  // exponents
     auto bytes = [&](int m) {
         const int rpA = tcx_rows_pad(m), tiles = rpA / TCX_M * (rpB / NT);
-        return sl_align((size_t)(m + N) * sizeof(int)) + sl_block_bytes(rpA, K) + sl_block_bytes(rpB, K) +
+        return head + sl_block_bytes(rpA, K) + sl_block_bytes(rpB, K) +
                sl_align((size_t)tiles * sl_units_max(nkc, tiles) * NT * TCX_M * sizeof(int2));
     };
     int mp = M;
@@ -618,16 +639,20 @@ jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const do
     void* ws = scratch.get(std::max(bytes(mp), last ? bytes(last) : 0));
     if (!ws) return JDFT_ERR_UNSUPPORTED;
     jdft_status s;
+    int* shift = (int*)ws;
+    int* exB = shift + K;
+    int* exA = exB + N;
+    char* Bs = (char*)ws + head;
+    char* As = Bs + sl_block_bytes(rpB, K);
+    if ((s = sl_exponents(A, lda, K, M, false, nullptr, 0, shift, st, true))) return s;
+    if ((s = sl_exponents(Bm, ldb, N, K, true, shift, +1, exB, st))) return s;
+    if ((s = sl_slice(Bm, ldb, N, NT, K, true, shift, +1, exB, Bs, st))) return s;
     for (int m0 = 0; m0 < M; m0 += mp) {
-        const int m = std::min(mp, M - m0), rpA = tcx_rows_pad(m);
-        int* maxB = (int*)ws;
-        int* maxA = maxB + N;
-        char* Bs = (char*)ws + sl_align((size_t)(m + N) * sizeof(int));
-        char* As = Bs + sl_block_bytes(rpB, K);
-        char* part = As + sl_block_bytes(rpA, K);
-        if ((s = sl_slice(Bm, ldb, N, NT, K, true, maxB, Bs, st))) return s;
-        if ((s = sl_slice(A + m0, lda, m, TCX_M, K, true, maxA, As, st))) return s;
-        if ((s = sl_product<false>(As, Bs, m, N, NT, nkc, maxA, maxB, part, out + m0, 1, ldo, 1.0, accumulate, st)))
+        const int m = std::min(mp, M - m0);
+        char* part = As + sl_block_bytes(tcx_rows_pad(m), K);
+        if ((s = sl_exponents(A + m0, lda, m, K, true, shift, -1, exA, st))) return s;
+        if ((s = sl_slice(A + m0, lda, m, TCX_M, K, true, shift, -1, exA, As, st))) return s;
+        if ((s = sl_product<false>(As, Bs, m, N, NT, nkc, exA, exB, part, out + m0, 1, ldo, 1.0, accumulate, st)))
             return s;
     }
     return JDFT_OK;
