@@ -44,6 +44,9 @@ constexpr int SL_RUN = 3;               // slices per stage and operand, one cop
 constexpr int SL_THREADS = 128;
 constexpr int SL_BIAS = 1 << 13;        // of stored exponents (0: none)
 constexpr int SL_BAD = 1 << 20;         // exponent of a row with an infinity or NaN
+// Cut against the rows as they are, an entry is off by about 2^-61 |a| |b| of its rows' norms, FP64 sums by 2^-53
+// of their terms: equal where the terms are 2^-8 of the product of the rows' maxima.  Scaled from 2^-4 down.
+constexpr int SL_NEAR = 2 * SL_BIAS - 4;
 __host__ __device__ constexpr int sl_top(int g) { return 10 - 2 * g; }              // larger digit sum of group g
 __host__ __device__ constexpr int sl_limit(int g) { return 2048 / (sl_top(g) - 1) / TCX_KC; }  // K chunks per unit
 
@@ -54,37 +57,59 @@ struct SlPlan {
     int first[SL_GROUPS + 1];
 };
 
-// ---- row maxima -------------------------------------------------------------
+// ---- exponents of the rows ------------------------------------------------------
 // Exponents are exponent fields (1 for zeros and denormals, whose significands have no
-// implicit bit) plus SL_BIAS, so that 0 means none.  `shift` scales the summed index: value
-// k counts as 2^(sign (shift[k] - SL_BIAS)) times itself, with sign -1 for one operand and
-// +1 for the other (see sl_zgemm_nn).
+// implicit bit) plus SL_BIAS, so that 0 means none.  The summed index may be scaled first:
+// value k of one operand counts as 2^-s_k and of the other as 2^s_k times itself, with
+// shift[k] = s_k + SL_BIAS.
+struct SlScale {
+    const int* shift;  // null: no scaling
+    const int* near;   // null: scale; else only where the word is below SL_NEAR (see sl_balance_kernel)
+    __device__ __forceinline__ bool on() const { return shift && (!near || *near < SL_NEAR); }
+};
+// An operand's rows: exponents, and where the index is scaled those of the scaled rows.
+struct SlRows {
+    const int *ex, *scaled;  // scaled null: ex are the scaled rows' already
+    SlScale scale;
+    int sign;  // of s_k
+    __device__ __forceinline__ const int* pick(bool on) const { return on && scaled ? scaled : ex; }
+};
 __device__ __forceinline__ int sl_field(int hi) { return max((hi >> 20) & 0x7ff, 1); }
-__device__ __forceinline__ int sl_shift(const int* __restrict__ shift, int sign, int k) {
-    return shift ? sign * (shift[k] - SL_BIAS) : 0;
-}
-// The exponent that a row of largest component v has at least: SL_BAD for an infinity or NaN.
+// The exponent that a row holding v has at least: SL_BAD for an infinity or NaN.
 __device__ __forceinline__ int sl_exponent(double2 v, int shift) {
     const int x = __double2hiint(v.x) & 0x7fffffff, y = __double2hiint(v.y) & 0x7fffffff, hi = max(x, y);
     if ((hi >> 20) == 0x7ff) return SL_BAD;
     return (hi | __double2loint(v.x) | __double2loint(v.y)) == 0 ? 0 : sl_field(hi) + shift + SL_BIAS;
 }
 
-// ex[r] = largest exponent over the row's K values (FINITE: of those without an infinity or NaN).
+// ex[r] = largest exponent over the K values of row r: first A's rows, then B's (signs -1
+// and +1 of the shift).  FINITE: of the values without an infinity or NaN.  at (or null):
+// the exponent and the place of such a value, as one word.
 template <bool FINITE>
-__global__ void __launch_bounds__(256) sl_rowmax_kernel(const double2* __restrict__ X, size_t ld, int K,
-                                                        const int* __restrict__ shift, int sign,
-                                                        int* __restrict__ ex) {
-    const double2* x = X + (size_t)blockIdx.x * ld;
-    int m = 0;
+__global__ void __launch_bounds__(256) sl_rowmax_kernel(const double2* __restrict__ A, size_t lda, int rowsA,
+                                                        const double2* __restrict__ B, size_t ldb, int K, SlScale sc,
+                                                        int* __restrict__ ex, unsigned long long* __restrict__ at) {
+    const bool on = sc.on();
+    if (sc.shift && !on) return;
+    const int r = blockIdx.x;
+    const double2* x = r < rowsA ? A + (size_t)r * lda : B + (size_t)(r - rowsA) * ldb;
+    const int sign = r < rowsA ? -1 : 1;
+    int m = 0, place = 0;
     for (int k = blockIdx.y * blockDim.x + threadIdx.x; k < K; k += gridDim.y * blockDim.x) {
-        const int e = sl_exponent(x[k], sl_shift(shift, sign, k));
-        if (!FINITE || e != SL_BAD) m = max(m, e);
+        const int e = sl_exponent(x[k], on ? sign * (sc.shift[k] - SL_BIAS) : 0);
+        if (e > m && (!FINITE || e != SL_BAD)) {
+            m = e;
+            place = k;
+        }
     }
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) atomicMax(&ex[blockIdx.x], m);
+    const int top = __reduce_max_sync(0xffffffffu, m);
+    const unsigned who = __ballot_sync(0xffffffffu, m == top);
+    if ((threadIdx.x & 31) == __ffs(who) - 1) {
+        atomicMax(&ex[r], top);
+        if (at) atomicMax(&at[r], (unsigned long long)top << 32 | (unsigned)place);
+    }
 }
-// The same of the transpose: row r, value k at X[k * ld + r]; blockIdx.y strides over k.
+// The same of a transpose: row r, value k at X[k * ld + r]; blockIdx.y strides over k.
 __global__ void __launch_bounds__(256) sl_rowmax_t_kernel(const double2* __restrict__ X, size_t ld, int rows, int K,
                                                           const int* __restrict__ shift, int sign,
                                                           int* __restrict__ ex) {
@@ -92,8 +117,72 @@ __global__ void __launch_bounds__(256) sl_rowmax_t_kernel(const double2* __restr
     if (r >= rows) return;
     int m = 0;
     for (int k = blockIdx.y; k < K; k += gridDim.y)
-        m = max(m, sl_exponent(X[(size_t)k * ld + r], sl_shift(shift, sign, k)));
+        m = max(m, sl_exponent(X[(size_t)k * ld + r], sign * (shift[k] - SL_BIAS)));
     atomicMax(&ex[r], m);
+}
+
+// The scaling of the summed index of conj(A) B: s_k half the difference of the columns'
+// largest exponents a_k and b_k, each value's taken relative to its row's.  Scaled, value k
+// of a row is at most 2^((a_k + b_k) / 2) of the row's largest, so max (a_k + b_k), kept
+// in *near (plus 2 SL_BIAS), is what the scaling gains over cutting the rows as they are.
+// sl_near_kernel looks at the columns of the rows' largest values first: in an ordinary
+// product one of them holds a large value of the other operand too, and nothing else is
+// read (H C of 64 bands with 256 projectors on 62 759 plane waves: 6 237 us with both operands
+// read a second time, 6 190 so).  One warp a row.
+__global__ void __launch_bounds__(256) sl_near_kernel(const double2* __restrict__ A, size_t lda, int rowsA,
+                                                      const double2* __restrict__ B, size_t ldb, int rowsB,
+                                                      const int* __restrict__ ex,
+                                                      const unsigned long long* __restrict__ at,
+                                                      int* __restrict__ near) {
+    const int r = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (r >= rowsA + rowsB || ex[r] == 0 || ex[r] == SL_BAD) return;
+    const bool ofA = r < rowsA;
+    const double2* x = (ofA ? B : A) + (unsigned)at[r];
+    const size_t ld = ofA ? ldb : lda;
+    const int* e = ex + (ofA ? rowsA : 0);
+    int g = 0;
+    for (int n = lane; n < (ofA ? rowsB : rowsA); n += 32) {
+        const int v = sl_exponent(x[n * ld], 0);
+        if (v != 0 && e[n] != SL_BAD) g = max(g, v - e[n] + 2 * SL_BIAS);
+    }
+    g = __reduce_max_sync(0xffffffffu, g);
+    if (lane == 0) atomicMax(near, g);
+}
+// 32 columns a block, its warps sharing the rows.
+__global__ void __launch_bounds__(256) sl_balance_kernel(const double2* __restrict__ A, size_t lda, int rowsA,
+                                                         const double2* __restrict__ B, size_t ldb, int rowsB, int K,
+                                                         const int* __restrict__ ex, int* __restrict__ shift,
+                                                         int* __restrict__ near) {
+    __shared__ int top[2][8][32];
+    constexpr int kNone = -(1 << 24);
+    if (*(volatile const int*)near >= SL_NEAR) return;  // only rises: the same to whoever reads it later
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = blockIdx.x * 32 + lane;
+    int m[2] = {kNone, kNone};
+#pragma unroll
+    for (int o = 0; o < 2; ++o) {
+        const double2* x = (o ? B : A) + k;
+        const size_t ld = o ? ldb : lda;
+        const int rows = k < K ? (o ? rowsB : rowsA) : 0;
+        const int* e = ex + (o ? rowsA : 0);
+#pragma unroll 4
+        for (int r = warp; r < rows; r += 8) {
+            const int v = sl_exponent(x[r * ld], 0), row = e[r];
+            if (v != 0 && row != SL_BAD) m[o] = max(m[o], v - row);
+        }
+        top[o][warp][lane] = m[o];
+    }
+    __syncthreads();
+    if (warp) return;
+#pragma unroll
+    for (int w = 1; w < 8; ++w) {
+        m[0] = max(m[0], top[0][w][lane]);
+        m[1] = max(m[1], top[1][w][lane]);
+    }
+    const bool both = m[0] > kNone && m[1] > kNone;
+    if (k < K) shift[k] = (both ? (m[0] - m[1]) >> 1 : 0) + SL_BIAS;
+    int g = both ? m[0] + m[1] + 2 * SL_BIAS : 0;
+    for (int o = 16; o > 0; o >>= 1) g = max(g, __shfl_xor_sync(0xffffffffu, g, o));
+    if (lane == 0) atomicMax(near, g);
 }
 
 // ---- slices -------------------------------------------------------------------
@@ -107,9 +196,11 @@ __global__ void __launch_bounds__(256) sl_rowmax_t_kernel(const double2* __restr
 // each of the 18 planes.
 template <bool TRANS>
 __global__ void __launch_bounds__(256) sl_slice_kernel(const double2* __restrict__ X, size_t ld, int rows, int K,
-                                                       int rows_pad, int RB, int nkc, const int* __restrict__ ex,
-                                                       const int* __restrict__ shift, int sign,
+                                                       int rows_pad, int RB, int nkc, SlRows sr,
                                                        __nv_bfloat16* __restrict__ out) {
+    const bool on = sr.scale.on();
+    const int* __restrict__ ex = sr.pick(on);
+    const int* __restrict__ shift = sr.scale.shift;
     const int per_chunk = rows_pad * 2;
     const int64_t total = (int64_t)per_chunk * nkc;
     const size_t P = (size_t)RB * TCX_KC;  // elements between planes
@@ -129,7 +220,7 @@ __global__ void __launch_bounds__(256) sl_slice_kernel(const double2* __restrict
             int sh = 0;
             if (r < rows && k0 + j < K) {
                 v = TRANS ? X[(size_t)(k0 + j) * ld + r] : X[(size_t)r * ld + k0 + j];
-                sh = sl_shift(shift, sign, k0 + j);
+                if (on) sh = sr.sign * (shift[k0 + j] - SL_BIAS);
             }
 #pragma unroll
             for (int c = 0; c < 2; ++c) {
@@ -402,7 +493,7 @@ __device__ __forceinline__ double sl_to_double(__int128 t, int q) {
 template <int RZ>
 __global__ void __launch_bounds__(TCX_M* RZ)
     sl_reduce_kernel(const int2* __restrict__ part, SlPlan plan, int NT, int mtiles, int M, int N,
-                     const int* __restrict__ exA, const int* __restrict__ exB, double2* __restrict__ out, size_t sm,
+                     SlRows ra, SlRows rb, double2* __restrict__ out, size_t sm,
                      size_t sn, double scale, int accumulate) {
     __shared__ longlong2 sum[RZ > 1 ? RZ : 1][2][RZ > 1 ? TCX_M : 1];
     const int r = threadIdx.x, q = threadIdx.y;
@@ -440,7 +531,8 @@ __global__ void __launch_bounds__(TCX_M* RZ)
     }
     if (m >= M) return;
     // a slice's last digit is worth 2^(exponent - 1083) of its row, the sums are in units of 2^56 of their product
-    const int eA = exA[m], eB = exB[n];
+    const bool on = ra.scale.on();
+    const int eA = ra.pick(on)[m], eB = rb.pick(on)[n];
     const int w = (eA - SL_BIAS - 1083) + (eB - SL_BIAS - 1083) + 56;
     double2 v = make_double2(scale * sl_to_double(re, w), scale * sl_to_double(im, w));
     if (eA == SL_BAD || eB == SL_BAD) v.x = v.y = __hiloint2double(0x7ff80000, 0);
@@ -522,8 +614,8 @@ static jdft_status sl_launch_nt(const void* As, const void* Bs, int nrbA, int nr
 }
 
 template <bool CONJ>
-static jdft_status sl_product(const void* As, const void* Bs, int M, int N, int NT, int nkc, const int* exA,
-                              const int* exB, void* partial, double2* out, size_t sm, size_t sn, double scale,
+static jdft_status sl_product(const void* As, const void* Bs, int M, int N, int NT, int nkc, const SlRows& ra,
+                              const SlRows& rb, void* partial, double2* out, size_t sm, size_t sn, double scale,
                               bool accumulate, cudaStream_t st) {
     const int mtiles = tcx_rows_pad(M) / TCX_M, ntiles = (N + NT - 1) / NT, tiles = mtiles * ntiles;
     const SlPlan plan = sl_plan(nkc, tiles);
@@ -537,57 +629,66 @@ static jdft_status sl_product(const void* As, const void* Bs, int M, int N, int 
         Trace tr_("sl_reduce", st);
         const dim3 grid(std::min(NT, N), tiles);
         if (plan.first[SL_GROUPS] > 24)
-            sl_reduce_kernel<8><<<grid, dim3(TCX_M, 8), 0, st>>>(part, plan, NT, mtiles, M, N, exA, exB, out, sm, sn,
+            sl_reduce_kernel<8><<<grid, dim3(TCX_M, 8), 0, st>>>(part, plan, NT, mtiles, M, N, ra, rb, out, sm, sn,
                                                                  scale, accumulate);
         else
-            sl_reduce_kernel<1><<<grid, dim3(TCX_M, 1), 0, st>>>(part, plan, NT, mtiles, M, N, exA, exB, out, sm, sn,
+            sl_reduce_kernel<1><<<grid, dim3(TCX_M, 1), 0, st>>>(part, plan, NT, mtiles, M, N, ra, rb, out, sm, sn,
                                                                  scale, accumulate);
     }
     return check_launch("sl_reduce");
 }
 
-// Exponents of an operand's rows (K values a row; trans: X[k * ld + r]).
-static jdft_status sl_exponents(const double2* X, size_t ld, int rows, int K, bool trans, const int* shift, int sign,
-                                int* ex, cudaStream_t st, bool finite = false) {
-    JDFT_CUDA_TRY(cudaMemsetAsync(ex, 0, (size_t)rows * sizeof(int), st));
+// Exponents of an operand's rows (K values a row) into ex, zeroed before; `finite` and sc as in the kernel.
+static jdft_status sl_exponents(const double2* A, size_t lda, int rowsA, const double2* B, size_t ldb, int rowsB, int K,
+                                SlScale sc, int* ex, cudaStream_t st, bool finite = false,
+                                unsigned long long* at = nullptr) {
+    const int rows = rowsA + rowsB;
+    const dim3 grid(rows, std::max(1, std::min((K + 1023) / 1024, 152 * 8 / rows)));
     Trace tr_("sl_rowmax", st);
-    if (trans) {
-        const int bx = (rows + 255) / 256;
-        sl_rowmax_t_kernel<<<dim3(bx, std::max(1, std::min(K, 152 * 8 / bx))), 256, 0, st>>>(X, ld, rows, K, shift,
-                                                                                            sign, ex);
-    } else {
-        const dim3 grid(rows, std::max(1, std::min((K + 1023) / 1024, 152 * 8 / rows)));
-        if (finite) sl_rowmax_kernel<true><<<grid, 256, 0, st>>>(X, ld, K, shift, sign, ex);
-        else sl_rowmax_kernel<false><<<grid, 256, 0, st>>>(X, ld, K, shift, sign, ex);
-    }
+    if (finite) sl_rowmax_kernel<true><<<grid, 256, 0, st>>>(A, lda, rowsA, B, ldb, K, sc, ex, at);
+    else sl_rowmax_kernel<false><<<grid, 256, 0, st>>>(A, lda, rowsA, B, ldb, K, sc, ex, at);
+    return check_launch("sl_rowmax");
+}
+static jdft_status sl_exponents_t(const double2* X, size_t ld, int rows, int K, const int* shift, int sign, int* ex,
+                                  cudaStream_t st) {
+    const int bx = (rows + 255) / 256;
+    Trace tr_("sl_rowmax", st);
+    sl_rowmax_t_kernel<<<dim3(bx, std::max(1, std::min(K, 152 * 8 / bx))), 256, 0, st>>>(X, ld, rows, K, shift, sign,
+                                                                                        ex);
     return check_launch("sl_rowmax");
 }
 
-// Slices of an operand from its rows' exponents, its rows padded to blocks of RB.
-static jdft_status sl_slice(const double2* X, size_t ld, int rows, int RB, int K, bool trans, const int* shift,
-                            int sign, const int* ex, void* slices, cudaStream_t st) {
+// Slices of an operand (trans: X[k * ld + r]) from its rows' exponents, its rows padded to blocks of RB.
+static jdft_status sl_slice(const double2* X, size_t ld, int rows, int RB, int K, bool trans, const SlRows& sr,
+                            void* slices, cudaStream_t st) {
     const int nkc = tcx_chunks(K), rows_pad = (rows + RB - 1) / RB * RB;
     const int64_t total = (int64_t)rows_pad * 2 * nkc;
     const int grid = (int)std::min<int64_t>((total + 255) / 256, 152 * 16);
     Trace tr_("sl_slice", st);
     if (trans)
-        sl_slice_kernel<true><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, RB, nkc, ex, shift, sign,
-                                                    (__nv_bfloat16*)slices);
+        sl_slice_kernel<true><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, RB, nkc, sr, (__nv_bfloat16*)slices);
     else
-        sl_slice_kernel<false><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, RB, nkc, ex, shift, sign,
-                                                     (__nv_bfloat16*)slices);
+        sl_slice_kernel<false><<<grid, 256, 0, st>>>(X, ld, rows, K, rows_pad, RB, nkc, sr, (__nv_bfloat16*)slices);
     return check_launch("sl_slice");
 }
 
+// Rows are cut against their own largest value, so the error of an entry is relative to the
+// product of the two rows' norms, as that of FP64 sums is where the rows' large values meet.
+// Where they do not (C falling and H C rising over the plane waves: the products of the
+// terms are far below the product of the rows' maxima), the summed index is scaled first
+// (sl_balance_kernel).  One product C^dag C needs none: its operands are alike.
 jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const double2* B, int ldb, double2* out,
                         int ldo, double scale, ProductScratch& scratch, cudaStream_t st) {
     const int NT = sl_nt(N);
-    const bool same = A == B && lda == ldb && M == N && NT == TCX_M;  // one set of slices
+    const bool twin = A == B && lda == ldb && M == N;
+    const bool same = twin && NT == TCX_M;  // one set of slices
     const int rpA = tcx_rows_pad(M), rpB = (N + NT - 1) / NT * NT;
     const int tiles = rpA / TCX_M * ((N + NT - 1) / NT);
-    const size_t mx = sl_align((size_t)(M + N) * sizeof(int));
+    // places of the rows' largest values, exponents of the rows, of the scaled rows, the gain, the shifts
+    const int rows = M + N, words = 2 * rows + (twin ? 0 : 2 * rows + 1);
+    const size_t head = sl_align(((size_t)words + (twin ? 0 : K)) * sizeof(int));
     auto bytes = [&](int k) {
-        return mx + sl_block_bytes(rpA, k) + (same ? 0 : sl_block_bytes(rpB, k)) +
+        return head + sl_block_bytes(rpA, k) + (same ? 0 : sl_block_bytes(rpB, k)) +
                sl_align((size_t)tiles * sl_units_max(tcx_chunks(k), tiles) * NT * TCX_M * sizeof(int2));
     };
     int kp = K;
@@ -595,20 +696,31 @@ jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const do
     void* ws = scratch.get(std::max(bytes(kp), K % kp ? bytes(K % kp) : 0));
     if (!ws) return JDFT_ERR_UNSUPPORTED;
     jdft_status s;
-    int* exA = (int*)ws;
-    int* exB = same ? exA : exA + M;
+    unsigned long long* at = twin ? nullptr : (unsigned long long*)ws;
+    int* ex = (int*)ws + (twin ? 0 : 2 * rows);
+    int *scaled = ex + rows, *near = scaled + rows, *shift = near + 1;
+    const SlScale none{nullptr, nullptr}, sc = twin ? none : SlScale{shift, near};
+    const SlRows ra{ex, twin ? nullptr : scaled, sc, -1};
+    const SlRows rb = twin ? ra : SlRows{ex + M, scaled + M, sc, +1};
     for (int k0 = 0; k0 < K; k0 += kp) {
         const int k = std::min(kp, K - k0);
-        char* As = (char*)ws + mx;
+        char* As = (char*)ws + head;
         char* Bs = same ? As : As + sl_block_bytes(rpA, k);
         char* part = Bs + sl_block_bytes(rpB, k);
-        if ((s = sl_exponents(A + k0, lda, M, k, false, nullptr, 0, exA, st))) return s;
-        if ((s = sl_slice(A + k0, lda, M, TCX_M, k, false, nullptr, 0, exA, As, st))) return s;
-        if (!same) {
-            if ((s = sl_exponents(B + k0, ldb, N, k, false, nullptr, 0, exB, st))) return s;
-            if ((s = sl_slice(B + k0, ldb, N, NT, k, false, nullptr, 0, exB, Bs, st))) return s;
+        JDFT_CUDA_TRY(cudaMemsetAsync(ws, 0, words * sizeof(int), st));
+        if ((s = sl_exponents(A + k0, lda, M, B + k0, ldb, twin ? 0 : N, k, none, ex, st, false, at))) return s;
+        if (!twin) {
+            {
+                Trace tr_("sl_balance", st);
+                sl_near_kernel<<<(rows + 7) / 8, 256, 0, st>>>(A + k0, lda, M, B + k0, ldb, N, ex, at, near);
+                sl_balance_kernel<<<(k + 31) / 32, 256, 0, st>>>(A + k0, lda, M, B + k0, ldb, N, k, ex, shift, near);
+            }
+            if ((s = check_launch("sl_balance"))) return s;
+            if ((s = sl_exponents(A + k0, lda, M, B + k0, ldb, N, k, sc, scaled, st))) return s;
         }
-        if ((s = sl_product<true>(As, Bs, M, N, NT, tcx_chunks(k), exA, exB, part, out, ldo, 1, scale, true, st)))
+        if ((s = sl_slice(A + k0, lda, M, TCX_M, k, false, ra, As, st))) return s;
+        if (!same && (s = sl_slice(B + k0, ldb, N, NT, k, false, rb, Bs, st))) return s;
+        if ((s = sl_product<true>(As, Bs, M, N, NT, tcx_chunks(k), ra, rb, part, out, ldo, 1, scale, true, st)))
             return s;
     }
     return JDFT_OK;
@@ -644,15 +756,19 @@ jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const do
     int* exA = exB + N;
     char* Bs = (char*)ws + head;
     char* As = Bs + sl_block_bytes(rpB, K);
-    if ((s = sl_exponents(A, lda, K, M, false, nullptr, 0, shift, st, true))) return s;
-    if ((s = sl_exponents(Bm, ldb, N, K, true, shift, +1, exB, st))) return s;
-    if ((s = sl_slice(Bm, ldb, N, NT, K, true, shift, +1, exB, Bs, st))) return s;
+    JDFT_CUDA_TRY(cudaMemsetAsync(ws, 0, head, st));
+    const SlScale none{nullptr, nullptr}, sc{shift, nullptr};
+    const SlRows ra{exA, nullptr, sc, -1}, rb{exB, nullptr, sc, +1};
+    if ((s = sl_exponents(A, lda, K, nullptr, 0, 0, M, none, shift, st, true))) return s;
+    if ((s = sl_exponents_t(Bm, ldb, N, K, shift, +1, exB, st))) return s;
+    if ((s = sl_slice(Bm, ldb, N, NT, K, true, rb, Bs, st))) return s;
     for (int m0 = 0; m0 < M; m0 += mp) {
         const int m = std::min(mp, M - m0);
         char* part = As + sl_block_bytes(tcx_rows_pad(m), K);
-        if ((s = sl_exponents(A + m0, lda, m, K, true, shift, -1, exA, st))) return s;
-        if ((s = sl_slice(A + m0, lda, m, TCX_M, K, true, shift, -1, exA, As, st))) return s;
-        if ((s = sl_product<false>(As, Bs, m, N, NT, nkc, exA, exB, part, out + m0, 1, ldo, 1.0, accumulate, st)))
+        if (m0) JDFT_CUDA_TRY(cudaMemsetAsync(exA, 0, (size_t)m * sizeof(int), st));
+        if ((s = sl_exponents_t(A + m0, lda, m, K, shift, -1, exA, st))) return s;
+        if ((s = sl_slice(A + m0, lda, m, TCX_M, K, true, ra, As, st))) return s;
+        if ((s = sl_product<false>(As, Bs, m, N, NT, nkc, ra, rb, part, out + m0, 1, ldo, 1.0, accumulate, st)))
             return s;
     }
     return JDFT_OK;

@@ -85,6 +85,32 @@ def test_projectors_of_different_norms(spread):
     assert np.all(np.abs(got - ref) <= 8 * U * scale + 3 * U * np.abs(ref))
 
 
+@pytest.mark.parametrize("nb, spread, norms", [(64, 0, 0), (64, 6, 0), (96, 10, 0), (64, 10, 8), (96, 40, 20)])
+def test_subspace_of_oppositely_graded_blocks(nb, spread, norms):
+    """C^dag H C where C falls by 10^spread over the plane waves (in random order) and H C rises by as much, bands of
+    different norms among them: every term is of one size, far below the product of the rows' maxima.  With r the rows'
+    largest components and a_k, b_k the columns' largest relative to them, the scaled rows stay below 2 sqrt(a_k b_k)
+    r each (halves and exponents rounded down); a component's two products lose 2^-60 of the scaled maxima for either
+    operand and 2^-58 in the digits left out: npw 2^-54 max(a_k b_k) r r', and the entry is rounded three times."""
+    jdft, b, npw = _basis()
+    rng = np.random.default_rng(nb + spread + norms)
+    x = _power(rng, spread, npw)[None, :]
+    s = _power(rng, norms, nb)[:, None]
+    C, H = _normal(rng, nb, npw) * x * s, _normal(rng, nb, npw) / x / s
+    out = torch.empty((nb, nb), dtype=torch.complex128, device="cuda")
+    Cd, Hd = torch.tensor(C, device="cuda"), torch.tensor(H, device="cuda")
+    names = _profiled(jdft, lambda: jdft.jdft_subspace(b, 0, Cd, Hd, out, None))
+    assert names["sl_mma"][0] == 1
+    got = out.cpu().numpy()
+    ref = C.conj().astype(LD) @ H.astype(LD).T
+    big = [np.maximum(np.abs(z.real), np.abs(z.imag)) for z in (C, H)]
+    r = [z.max(1) for z in big]
+    a, bk = ((z / q[:, None]).max(0) for z, q in zip(big, r))
+    tol = npw * 2.0 ** -54 * (a * bk).max() * r[0][:, None] * r[1][None, :]
+    assert np.all(np.abs(got.real - ref.real) <= tol + 3 * U * np.abs(ref))
+    assert np.all(np.abs(got.imag - ref.imag) <= tol + 3 * U * np.abs(ref))
+
+
 def test_rotation_keeps_a_non_finite_coefficient_to_its_plane_wave():
     """With the overlap given, a NaN or infinity among the coefficients of one plane wave reaches that plane wave's
     outputs only; the others are the same bits."""
