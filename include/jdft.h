@@ -34,7 +34,8 @@
  *     kernel launch error is reported as JDFT_ERR_CUDA.
  *   - A basis handle owns device copies of its maps, potential and
  *     projectors, and a workspace that grows on demand (growth calls
- *     cudaMalloc, which synchronises the device).  One basis must not be used
+ *     cudaMalloc, which synchronises the device).  Large FP64 products (on the
+ *     tensor cores, see jdft_subspace) have scratch of their own that grows so.  One basis must not be used
  *     from two host threads at once.
  *   - On any status other than JDFT_OK, jdft_last_error() returns a message
  *     (thread-local, valid until the next call on that thread).
@@ -186,7 +187,13 @@ jdft_status jdft_apply_H_density(jdft_basis_t basis, int ik, const void* C, int 
 /* CHC = C^dag (HC), COC = C^dag O C = Omega C^dag C: the subspace matrices of a
  * ColumnBundle for the variational minimiser (Sec. 2.1, Minimize).  Device
  * complex128 nb x nb, row-major, both triangles written, accumulated in FP64.
- * Either output may be NULL to skip it. */
+ * Either output may be NULL to skip it.  Calls of one basis may be queued on
+ * several streams: this call does not use the basis workspace (JDFT_BF16X3 with
+ * more than 32 bands does).  Large JDFT_FP64 products run on the tensor cores
+ * from slices of their operands in scratch that the basis owns; calls on
+ * different streams then run one after the other.  A product of a stream that is
+ * being captured allocates nothing and runs on the CUDA cores instead (in the
+ * calls that use the basis workspace, unless an earlier call left enough). */
 jdft_status jdft_subspace(jdft_basis_t basis, int ik, const void* C, int ldc, const void* HC,
                           int ldhc, int nb, void* CHC, void* COC, jdft_prec prec, void* stream);
 

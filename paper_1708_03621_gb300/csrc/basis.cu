@@ -59,7 +59,21 @@ jdft_status ensure_ws(Workspace& w, size_t bytes) {
     return JDFT_OK;
 }
 
-void* ProductScratch::get(size_t need) {
+void* ProductScratch::get(size_t need, cudaStream_t st) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &cap) != cudaSuccess) {  // the legacy stream beside a capture
+        cudaGetLastError();
+        return nullptr;
+    }
+    if (cap != cudaStreamCaptureStatusNone) return !ordered && bytes >= need ? ptr : nullptr;
+    if (ordered) {
+        if (!done && cudaEventCreateWithFlags(&done, cudaEventDisableTiming) != cudaSuccess) {
+            cudaGetLastError();
+            done = nullptr;
+            return nullptr;
+        }
+        if (bytes >= need) return cudaStreamWaitEvent(st, done, 0) == cudaSuccess ? ptr : nullptr;
+    }
     if (bytes >= need) return ptr;
     // half again, so that the blocks outgrown stay few; the plain size where that much is not left
     for (const size_t want : {std::max(need, bytes + bytes / 2), need}) {
@@ -75,11 +89,17 @@ void* ProductScratch::get(size_t need) {
     return nullptr;
 }
 
+void ProductScratch::finish(cudaStream_t st) {
+    if (ordered) cudaEventRecord(done, st);
+}
+
 void ProductScratch::release() {
     cudaFree(ptr);
     for (void* p : retired) cudaFree(p);
+    if (done) cudaEventDestroy(done);
     retired.clear();
     ptr = nullptr;
+    done = nullptr;
     bytes = 0;
 }
 
@@ -408,6 +428,7 @@ jdft_status jdft_basis_destroy(jdft_basis_t b) {
     for (auto& s : b->ks) free_sphere(s);
     cudaFree(b->tw64); cudaFree(b->tw32); cudaFree(b->counters); cudaFree(b->V); cudaFree(b->V32); cudaFree(b->Vn); cudaFree(b->Vn32); cudaFree(b->work.ptr);
     b->prodwork.release();
+    b->subwork.release();
     if (b->side) {
         cudaStreamSynchronize(b->side);
         cudaStreamDestroy(b->side);

@@ -132,13 +132,26 @@ struct Workspace {
 // Scratch of the sliced FP64 products.  It grows by at least half again and keeps the
 // blocks it has outgrown until the basis goes (their sizes add up to less than
 // twice the last one), so that a captured graph that holds a pointer to one
-// stays valid.  get() returns nullptr when the device has no room.
+// stays valid.
+// ordered: for calls that nothing else keeps apart.  A product then waits on the device
+// for the one before it, on whatever stream that ran, and no graph takes a pointer.
 struct ProductScratch {
+    bool ordered = false;
     void* ptr = nullptr;
     size_t bytes = 0;
     std::vector<void*> retired;
-    void* get(size_t need);
+    cudaEvent_t done = nullptr;
+    // `need` bytes for work on st, or nullptr where the device has no room or st is
+    // being captured and they are not there already (ordered: at all)
+    void* get(size_t need, cudaStream_t st);
+    // after the last launch that uses them
+    void finish(cudaStream_t st);
     void release();
+};
+struct ScratchUse {  // of a product, to its end on every path
+    ProductScratch& scratch;
+    cudaStream_t st;
+    ~ScratchUse() { scratch.finish(st); }
 };
 
 }  // namespace jdft
@@ -177,7 +190,8 @@ struct jdft_basis_s {
     // full-box field transforms (Hartree, Kohn-Sham potential): a complex FP64
     // box and per-block partial sums (grown on first use)
     jdft::Workspace fieldwork;
-    jdft::ProductScratch prodwork;
+    jdft::ProductScratch prodwork;  // of calls that use the basis workspace as well
+    jdft::ProductScratch subwork{true};  // of jdft_subspace, which does not (ordered)
     // block counters of sums finished by their launch's last block (zero between launches)
     unsigned* counters = nullptr;
     // spinor calls: real-space boxes and sphere blocks of a band chunk

@@ -557,7 +557,7 @@ extern "C" jdft_status jdft_subspace(jdft_basis_t b, int ik, const void* C, int 
         JDFT_CUDA_TRY(cudaMemsetAsync(CHC, 0, (size_t)nb * nb * sizeof(double2), st));
         s = (prec == JDFT_FP64)
                 ? gemm_cn<double>(prec, nb, nb, npw, (const double2*)C, ldc, (const double2*)HC, ldhc, (double2*)CHC,
-                                  nb, 1.0, st, &b->prodwork)
+                                  nb, 1.0, st, &b->subwork)
                 : gemm_cn<float>(prec, nb, nb, npw, (const float2*)C, ldc, (const float2*)HC, ldhc, (double2*)CHC, nb, 1.0,
                                   st);
         if (s != JDFT_OK) return s;
@@ -566,7 +566,7 @@ extern "C" jdft_status jdft_subspace(jdft_basis_t b, int ik, const void* C, int 
         JDFT_CUDA_TRY(cudaMemsetAsync(COC, 0, (size_t)nb * nb * sizeof(double2), st));
         s = (prec == JDFT_FP64)
                 ? gemm_cn<double>(prec, nb, nb, npw, (const double2*)C, ldc, (const double2*)C, ldc, (double2*)COC, nb,
-                                  b->omega, st, &b->prodwork)
+                                  b->omega, st, &b->subwork)
                 : gemm_cn<float>(prec, nb, nb, npw, (const float2*)C, ldc, (const float2*)C, ldc, (double2*)COC, nb,
                                   b->omega, st);
     }

@@ -693,8 +693,9 @@ jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const do
     };
     int kp = K;
     while (kp > 2048 && bytes(kp) > SL_BUDGET) kp = (kp / 2 + TCX_KC - 1) / TCX_KC * TCX_KC;
-    void* ws = scratch.get(std::max(bytes(kp), K % kp ? bytes(K % kp) : 0));
+    void* ws = scratch.get(std::max(bytes(kp), K % kp ? bytes(K % kp) : 0), st);
     if (!ws) return JDFT_ERR_UNSUPPORTED;
+    const ScratchUse use{scratch, st};
     jdft_status s;
     unsigned long long* at = twin ? nullptr : (unsigned long long*)ws;
     int* ex = (int*)ws + (twin ? 0 : 2 * rows);
@@ -748,8 +749,9 @@ jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const do
     while (mp > 4096 && bytes(mp) > SL_BUDGET) mp = (mp / 2 + TCX_M - 1) / TCX_M * TCX_M;
     // smaller panels cut K finer: the last panel may need as much as a full one
     const int last = M % mp;
-    void* ws = scratch.get(std::max(bytes(mp), last ? bytes(last) : 0));
+    void* ws = scratch.get(std::max(bytes(mp), last ? bytes(last) : 0), st);
     if (!ws) return JDFT_ERR_UNSUPPORTED;
+    const ScratchUse use{scratch, st};
     jdft_status s;
     int* shift = (int*)ws;
     int* exB = shift + K;
