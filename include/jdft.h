@@ -705,11 +705,14 @@ jdft_status jdft_profile_read(char* buf, int buflen);
 jdft_status jdft_device_status(void* stream);
 
 /* Limit, in seconds, of each device-side wait of the tensor-core products
- * (large FP64 products run on the tensor cores too) on the current device (default 2 s; kernels launched after the call use it).
+ * (large FP64 products run on the tensor cores too) on the current device
+ * (default 2 s; kernels launched after the call use it).
  * A wait that runs out records JDFT_ERR_TIMEOUT for jdft_device_status, stops
  * issuing products, waits (under a fixed 2 s limit of its own) for the products
  * it already committed, and frees its tensor memory; the product's output is
- * then incomplete.  0 makes every such product give up at its first wait,
+ * then incomplete: NaN throughout for JDFT_FP64.  Calls that wait for their
+ * JDFT_FP64 products (jdft_orthonormalize, jdft_minimize_bands, the generalised
+ * calls, jdft_mlp_rows, jdft_scf) also return JDFT_ERR_TIMEOUT.  0 makes every such product give up at its first wait,
  * which tests of the failure path use.  JDFT_ERR_ARG outside [0, 60].  The
  * paper has no counterpart. */
 jdft_status jdft_set_wait_limit(double seconds);

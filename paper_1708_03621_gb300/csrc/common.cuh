@@ -141,12 +141,21 @@ struct ProductScratch {
     size_t bytes = 0;
     std::vector<void*> retired;
     cudaEvent_t done = nullptr;
+    int* failed = nullptr;  // device word (or null) that a product whose waits ran out sets to JDFT_ERR_TIMEOUT
     // `need` bytes for work on st, or nullptr where the device has no room or st is
     // being captured and they are not there already (ordered: at all)
     void* get(size_t need, cudaStream_t st);
     // after the last launch that uses them
     void finish(cudaStream_t st);
     void release();
+};
+// The device word of a call that waits for its products and then returns their timeout.
+struct ProductStatus {
+    ProductScratch& scratch;
+    int* outer;
+    ProductStatus(ProductScratch& s, int* word) : scratch(s), outer(s.failed) { s.failed = word; }
+    ~ProductStatus() { scratch.failed = outer; }
+    ProductStatus(const ProductStatus&) = delete;
 };
 struct ScratchUse {  // of a product, to its end on every path
     ProductScratch& scratch;

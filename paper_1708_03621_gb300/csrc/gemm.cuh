@@ -66,6 +66,11 @@ jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const do
 jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const double2* Bm, int ldb, double2* out,
                         int ldo, bool accumulate, ProductScratch& scratch, cudaStream_t st);
 
+// What a call that waits returns when one of its sliced products gave up (ProductStatus).
+inline jdft_status product_timeout() {
+    return set_error(JDFT_ERR_TIMEOUT, "a wait of an FP64 product on the tensor cores gave up");
+}
+
 // Precision dispatch: JDFT_TF32X3 and JDFT_BF16X3 run the tensor-core
 // versions (T = float only), the other precisions the CUDA-core ones; FP64
 // products large enough run from slices when the caller has scratch for them.

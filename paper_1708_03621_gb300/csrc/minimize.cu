@@ -480,7 +480,7 @@ struct MinState {
     c_t<T>* W;
     double *Tb, *scal;
     float* bf;  // per-band features of the learned preconditioner
-    int* status;
+    int* status;  // of the factorisations, and of the sliced products
     DevBuf mem;
     const double* kin;
     const float* kin32;
@@ -520,7 +520,7 @@ struct MinState {
             spw = (char*)take(sw);
             spp = (char*)take(spp_bytes);
         }
-        JDFT_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), st));
+        JDFT_CUDA_TRY(cudaMemsetAsync(status, 0, 2 * sizeof(int), st));
         return JDFT_OK;
     }
 
@@ -581,10 +581,11 @@ struct MinState {
         return JDFT_OK;
     }
     jdft_status read_status() {
-        int s = 0;
-        JDFT_CUDA_TRY(cudaMemcpyAsync(&s, status, sizeof(int), cudaMemcpyDeviceToHost, st));
+        int s[2] = {0, 0};
+        JDFT_CUDA_TRY(cudaMemcpyAsync(s, status, sizeof s, cudaMemcpyDeviceToHost, st));
         JDFT_CUDA_TRY(cudaStreamSynchronize(st));
-        if (s != 0) return set_error((jdft_status)s, "overlap matrix not positive definite in the minimiser");
+        if (s[1] != 0) return product_timeout();
+        if (s[0] != 0) return set_error((jdft_status)s[0], "overlap matrix not positive definite in the minimiser");
         return JDFT_OK;
     }
     // Orthonormalise X -> C (Cholesky of Omega X^dag X), then HC = H C, Hs = C^dag HC.
@@ -803,8 +804,9 @@ static jdft_status orthonormalize_impl(jdft_basis_s* b, int ik, void* C, int ldc
     c_t<T>* W = (c_t<T>*)(q + sm);
     double2* work = (double2*)(q + sm + wbytes);
     c_t<T>* tmp = (c_t<T>*)(q + sm + wbytes + lab);
-    int* status = (int*)(q + sm + wbytes + lab + blk);
-    JDFT_CUDA_TRY(cudaMemsetAsync(status, 0, sizeof(int), st));
+    int* status = (int*)(q + sm + wbytes + lab + blk);  // of the factorisation, and of the sliced products
+    JDFT_CUDA_TRY(cudaMemsetAsync(status, 0, 2 * sizeof(int), st));
+    const ProductStatus watch(b->prodwork, sticky ? b->prodwork.failed : status + 1);
     if (Ugiven) {
         U = const_cast<double2*>(Ugiven);  // read only
     } else {
@@ -838,10 +840,11 @@ static jdft_status orthonormalize_impl(jdft_basis_s* b, int ik, void* C, int ldc
         }
         return check_launch("status_merge");
     }
-    int hs = 0;
-    JDFT_CUDA_TRY(cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st));
+    int hs[2] = {0, 0};
+    JDFT_CUDA_TRY(cudaMemcpyAsync(hs, status, sizeof hs, cudaMemcpyDeviceToHost, st));
     JDFT_CUDA_TRY(cudaStreamSynchronize(st));
-    if (hs) return set_error(JDFT_ERR_NOT_POSDEF, "C^dag O C is not positive definite");
+    if (hs[1]) return product_timeout();
+    if (hs[0]) return set_error(JDFT_ERR_NOT_POSDEF, "C^dag O C is not positive definite");
     return JDFT_OK;
 }
 }  // namespace jdft
@@ -1038,6 +1041,7 @@ jdft_status jdft_minimize_bands(jdft_basis_t b, int ik, void* C, int ldc, int nb
     jdft_status s;
     MinState<double> M64;
     if ((s = setup_state(M64, b, ik, nb, JDFT_FP64, f, st))) return s;
+    const ProductStatus watch(b->prodwork, M64.status + 1);
     JDFT_CUDA_TRY(cudaMemcpy2DAsync(M64.Y, (size_t)npw * sizeof(double2), C, (size_t)ldc * sizeof(double2),
                                     (size_t)npw * sizeof(double2), nb, cudaMemcpyDeviceToDevice, st));
     if (opts->prec != JDFT_FP64) {
@@ -1076,7 +1080,8 @@ jdft_status jdft_minimize_bands(jdft_basis_t b, int ik, void* C, int ldc, int nb
         jdft_status s2 = small_jacobi_eigs(nb, M64.Hs, M64.lawork, eigs, st);
         if (s2 != JDFT_OK) return s2;
     }
-    JDFT_CUDA_TRY(cudaStreamSynchronize(st));
+    const jdft_status last = M64.read_status();  // waits
+    if (last != JDFT_OK) return last;
     report->seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     if (!report->converged) return set_error(JDFT_ERR_NOT_CONVERGED, "band minimiser reached its iteration limit");
     return JDFT_OK;

@@ -647,12 +647,15 @@ jdft_status jdft_mlp_rows(jdft_basis_t b, int ik, const void* C, const void* Cst
     double2* Bm = (double2*)alloc((size_t)nb * nb * sizeof(double2));
     double* Tb = (double*)alloc(nb * sizeof(double));
     float* bf = (float*)alloc(3 * (size_t)nb * sizeof(float));
-    double* sums = (double*)alloc(2 * sizeof(double));
+    double* sums = (double*)alloc(3 * sizeof(double));  // and the status word of the sliced products
     if (!HC || !G || !Tt || !Hs || !M || !Bm || !Tb || !bf || !sums)
         return done(set_error(JDFT_ERR_OOM, "jdft_mlp_rows"));
     const double2* Cd = (const double2*)C;
     const double2* Cs = (const double2*)Cstar;
     jdft_status s;
+    int* failed = (int*)(sums + 2);
+    if (cudaMemsetAsync(failed, 0, sizeof(int), st) != cudaSuccess) return done(set_error(JDFT_ERR_CUDA, "memset"));
+    const ProductStatus watch(b->prodwork, failed);
     // residual block G = HC - Omega C (C^dag H C)
     if ((s = jdft_apply_H(b, ik, Cd, npw, HC, npw, nb, JDFT_FP64, stream))) return done(s);
     if (cudaMemsetAsync(Hs, 0, (size_t)nb * nb * sizeof(double2), st) != cudaSuccess)
@@ -704,6 +707,11 @@ jdft_status jdft_mlp_rows(jdft_basis_t b, int ik, const void* C, const void* Cst
         }
         if ((s = check_launch("rows_normalize"))) return done(s);
     }
+    int gave_up = 0;
+    if (cudaMemcpyAsync(&gave_up, failed, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        cudaStreamSynchronize(st) != cudaSuccess)
+        return done(set_error(JDFT_ERR_CUDA, "status"));
+    if (gave_up) return done(product_timeout());
     *nrows = n;
     return done(JDFT_OK);
 }

@@ -13,6 +13,7 @@
 // of D (the same P^dag C, sparse Q rows, P X kernels and precisions); the
 // generalised Rayleigh-Ritz and orthonormalisation reuse the FP64 overlap
 // factorisation of jdft_orthonormalize_async with C^dag S C given as U.
+#include <cstring>
 #include <algorithm>
 #include <chrono>
 #include <cmath>
@@ -205,6 +206,15 @@ gteter_kernel(int npw, const double2* __restrict__ C, const double* __restrict__
     }
 }
 
+// Waits and reads the status words of a call: of its factorisations, and of its sliced products.
+jdft_status generalized_status(const int* status, const char* not_posdef, cudaStream_t st) {
+    int h[2] = {0, 0};
+    JDFT_CUDA_TRY(cudaMemcpyAsync(h, status, sizeof h, cudaMemcpyDeviceToHost, st));
+    JDFT_CUDA_TRY(cudaStreamSynchronize(st));
+    if (h[1]) return product_timeout();
+    return h[0] ? set_error(JDFT_ERR_NOT_POSDEF, not_posdef) : JDFT_OK;
+}
+
 struct GenMin {
     jdft_basis_s* b;
     int ik, npw, nb;
@@ -245,9 +255,13 @@ struct GenMin {
         return check_launch("gen_axpby");
     }
     jdft_status read(double* h, int n) {
-        JDFT_CUDA_TRY(cudaMemcpyAsync(h, scal, n * sizeof(double), cudaMemcpyDeviceToHost, st));
+        double all[16];  // the scalars, and the status words after them
+        JDFT_CUDA_TRY(cudaMemcpyAsync(all, scal, sizeof all, cudaMemcpyDeviceToHost, st));
         JDFT_CUDA_TRY(cudaStreamSynchronize(st));
-        return JDFT_OK;
+        std::memcpy(h, all, n * sizeof(double));
+        int words[2];
+        std::memcpy(words, all + 15, sizeof words);
+        return words[1] ? product_timeout() : JDFT_OK;
     }
     // X <- X - C (C^dag S X), with S X formed into T
     jdft_status project(double2* X) {
@@ -365,11 +379,13 @@ jdft_status jdft_subspace_generalized(jdft_basis_t b, int ik, const void* C, int
         return s_;
     };
     jdft_status s;
+    if (cudaMemsetAsync(status, 0, 2 * sizeof(int), st) != cudaSuccess)
+        return done(set_error(JDFT_ERR_CUDA, "jdft_subspace_generalized: memset"));
+    const ProductStatus watch(b->prodwork, status + 1);
     if ((s = run_op_S<double>(b, ik, C, ldc, SCb, npw, nb, JDFT_FP64, st))) return done(s);
     if (cudaMemsetAsync(CHC, 0, (size_t)nb * nb * sizeof(double2), st) != cudaSuccess ||
         cudaMemsetAsync(CSC, 0, (size_t)nb * nb * sizeof(double2), st) != cudaSuccess ||
-        cudaMemsetAsync(A, 0, (size_t)nb * nb * sizeof(double2), st) != cudaSuccess ||
-        cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess)
+        cudaMemsetAsync(A, 0, (size_t)nb * nb * sizeof(double2), st) != cudaSuccess)
         return done(set_error(JDFT_ERR_CUDA, "jdft_subspace_generalized: memset"));
     if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, (const double2*)C, ldc, (const double2*)HC, ldhc,
                              (double2*)CHC, nb, 1.0, st, &b->prodwork)))
@@ -388,13 +404,9 @@ jdft_status jdft_subspace_generalized(jdft_basis_t b, int ik, const void* C, int
         if ((s = jdft_orthonormalize_async(b, ik, Hc, npw, nb, CSC, JDFT_FP64, status, stream))) return done(s);
         if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, Cc, npw, Hc, npw, A, nb, 1.0, st, &b->prodwork)))
             return done(s);
-        int hs = 0;
-        if (cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess)
-            return done(set_error(JDFT_ERR_CUDA, "jdft_subspace_generalized: status"));
-        if (hs) return done(set_error(JDFT_ERR_NOT_POSDEF, "C^dag S C is not positive definite"));
-        if ((s = jdft_subspace_eigs(nb, A, eigs, stream))) return done(s);
     }
+    if ((s = generalized_status(status, "C^dag S C is not positive definite", st))) return done(s);
+    if (eigs && (s = jdft_subspace_eigs(nb, A, eigs, stream))) return done(s);
     return done(JDFT_OK);
 }
 
@@ -415,19 +427,15 @@ jdft_status jdft_orthonormalize_generalized(jdft_basis_t b, int ik, void* C, int
         return s_;
     };
     jdft_status s;
-    if ((s = run_op_S<double>(b, ik, C, ldc, SCb, npw, nb, JDFT_FP64, st))) return done(s);
     if (cudaMemsetAsync(U, 0, (size_t)nb * nb * sizeof(double2), st) != cudaSuccess ||
-        cudaMemsetAsync(status, 0, sizeof(int), st) != cudaSuccess)
+        cudaMemsetAsync(status, 0, 2 * sizeof(int), st) != cudaSuccess)
         return done(set_error(JDFT_ERR_CUDA, "jdft_orthonormalize_generalized: memset"));
+    const ProductStatus watch(b->prodwork, status + 1);
+    if ((s = run_op_S<double>(b, ik, C, ldc, SCb, npw, nb, JDFT_FP64, st))) return done(s);
     if ((s = gemm_cn<double>(JDFT_FP64, nb, nb, npw, (const double2*)C, ldc, SCb, npw, U, nb, 1.0, st, &b->prodwork)))
         return done(s);
     if ((s = jdft_orthonormalize_async(b, ik, C, ldc, nb, U, JDFT_FP64, status, stream))) return done(s);
-    int hs = 0;
-    if (cudaMemcpyAsync(&hs, status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-        return done(set_error(JDFT_ERR_CUDA, "jdft_orthonormalize_generalized: status"));
-    if (hs) return done(set_error(JDFT_ERR_NOT_POSDEF, "C^dag S C is not positive definite"));
-    return done(JDFT_OK);
+    return done(generalized_status(status, "C^dag S C is not positive definite", st));
 }
 
 jdft_status jdft_minimize_bands_generalized(jdft_basis_t b, int ik, void* C, int ldc, int nb,
@@ -467,10 +475,11 @@ jdft_status jdft_minimize_bands_generalized(jdft_basis_t b, int ik, void* C, int
     };
     const double noise_ulp = 64.0 * 2.220446049250313e-16;
     jdft_status s;
-    if (cudaMemsetAsync(M.status, 0, sizeof(int), st) != cudaSuccess ||
+    if (cudaMemsetAsync(M.status, 0, 2 * sizeof(int), st) != cudaSuccess ||
         cudaMemcpy2DAsync(M.C, npw * sizeof(double2), C, (size_t)ldc * sizeof(double2), npw * sizeof(double2), nb,
                           cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         return done(set_error(JDFT_ERR_CUDA, "jdft_minimize_bands_generalized: set-up copies"));
+    const ProductStatus watch(b->prodwork, M.status + 1);
     // S-orthonormal start
     if ((s = run_op_S<double>(b, ik, M.C, npw, M.SC, npw, nb, JDFT_FP64, st))) return done(s);
     if ((s = M.orthonormalize(M.C, M.SC))) return done(s);
@@ -553,11 +562,7 @@ jdft_status jdft_minimize_bands_generalized(jdft_basis_t b, int ik, void* C, int
         std::swap(M.Gp, M.G);
         have_prev = true;
     }
-    int hs = 0;
-    if (cudaMemcpyAsync(&hs, M.status, sizeof(int), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-        cudaStreamSynchronize(st) != cudaSuccess)
-        return done(set_error(JDFT_ERR_CUDA, "jdft_minimize_bands_generalized: status"));
-    if (hs) return done(set_error(JDFT_ERR_NOT_POSDEF, "Y^dag S Y is not positive definite"));
+    if ((s = generalized_status(M.status, "Y^dag S Y is not positive definite", st))) return done(s);
     if (cudaMemcpy2DAsync(C, (size_t)ldc * sizeof(double2), M.C, npw * sizeof(double2), npw * sizeof(double2), nb,
                           cudaMemcpyDeviceToDevice, st) != cudaSuccess)
         return done(set_error(JDFT_ERR_CUDA, "jdft_minimize_bands_generalized: output copy"));

@@ -305,7 +305,7 @@ __device__ __forceinline__ void sl_commit(uint32_t bar) {
 template <int NT, bool CONJ>
 __global__ void __launch_bounds__(SL_THREADS, 1)
     sl_mma_kernel(const char* __restrict__ As, const char* __restrict__ Bs, int nrbA, int nrbB, int nkc, int mtiles,
-                  SlPlan plan, int2* __restrict__ part) {
+                  SlPlan plan, int2* __restrict__ part, int* __restrict__ gave_up) {
     using L = SlLayout<NT>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -468,7 +468,11 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
     tc::tc_fence_before_sync();
     __syncthreads();
     if (warp == 2) tc::tmem_dealloc(tmem, L::NCOLS);
-    if (!ok && tid == 0) atomicExch(&g_tc_status, (int)JDFT_ERR_TIMEOUT);
+    if (!ok && tid == 0) {
+        // the block's part holds whatever was there before: the sums below must not use it
+        atomicExch(gave_up, 1);
+        atomicExch(&g_tc_status, (int)JDFT_ERR_TIMEOUT);
+    }
 }
 
 // ---- sums -------------------------------------------------------------------------
@@ -489,12 +493,14 @@ __device__ __forceinline__ double sl_to_double(__int128 t, int q) {
 
 // Block (columns j .. of a tile): thread (row r, q) sums units q, q + RZ, ... of
 // its output with 64-bit integers per group, the RZ sums meet in 128 bits.
-// out[m * sm + n * sn] (+)= scale * sum.
+// out[m * sm + n * sn] (+)= scale * sum, NaN where a block of the product gave up, which
+// *failed (or null) then says as well.
 template <int RZ>
 __global__ void __launch_bounds__(TCX_M* RZ)
     sl_reduce_kernel(const int2* __restrict__ part, SlPlan plan, int NT, int mtiles, int M, int N,
                      SlRows ra, SlRows rb, double2* __restrict__ out, size_t sm,
-                     size_t sn, double scale, int accumulate) {
+                     size_t sn, double scale, int accumulate, const int* __restrict__ gave_up,
+                     int* __restrict__ failed) {
     __shared__ longlong2 sum[RZ > 1 ? RZ : 1][2][RZ > 1 ? TCX_M : 1];
     const int r = threadIdx.x, q = threadIdx.y;
     const int col = blockIdx.x, tile = blockIdx.y;
@@ -535,7 +541,9 @@ __global__ void __launch_bounds__(TCX_M* RZ)
     const int eA = ra.pick(on)[m], eB = rb.pick(on)[n];
     const int w = (eA - SL_BIAS - 1083) + (eB - SL_BIAS - 1083) + 56;
     double2 v = make_double2(scale * sl_to_double(re, w), scale * sl_to_double(im, w));
-    if (eA == SL_BAD || eB == SL_BAD) v.x = v.y = __hiloint2double(0x7ff80000, 0);
+    const bool incomplete = *gave_up != 0;
+    if (eA == SL_BAD || eB == SL_BAD || incomplete) v.x = v.y = __hiloint2double(0x7ff80000, 0);
+    if (incomplete && failed && m + n == 0) *failed = (int)JDFT_ERR_TIMEOUT;
     double2* o = out + (size_t)m * sm + (size_t)n * sn;
     if (accumulate) {
         const double2 old = *o;
@@ -601,14 +609,14 @@ bool sl_eligible(int M, int N, int K) {
 
 template <int NT, bool CONJ>
 static jdft_status sl_launch_nt(const void* As, const void* Bs, int nrbA, int nrbB, int nkc, int mtiles, int tiles,
-                                const SlPlan& plan, int2* part, cudaStream_t st) {
+                                const SlPlan& plan, int2* part, int* gave_up, cudaStream_t st) {
     auto kern = sl_mma_kernel<NT, CONJ>;
     cudaError_t e = set_smem_attr((const void*)kern, SlLayout<NT>::SMEM);
     if (e != cudaSuccess) return set_error(JDFT_ERR_CUDA, std::string("sl_mma: ") + cudaGetErrorString(e));
     {
         Trace tr_("sl_mma", st);
         kern<<<dim3(plan.first[SL_GROUPS], tiles), SL_THREADS, SlLayout<NT>::SMEM, st>>>(
-            (const char*)As, (const char*)Bs, nrbA, nrbB, nkc, mtiles, plan, part);
+            (const char*)As, (const char*)Bs, nrbA, nrbB, nkc, mtiles, plan, part, gave_up);
     }
     return check_launch("sl_mma");
 }
@@ -616,24 +624,24 @@ static jdft_status sl_launch_nt(const void* As, const void* Bs, int nrbA, int nr
 template <bool CONJ>
 static jdft_status sl_product(const void* As, const void* Bs, int M, int N, int NT, int nkc, const SlRows& ra,
                               const SlRows& rb, void* partial, double2* out, size_t sm, size_t sn, double scale,
-                              bool accumulate, cudaStream_t st) {
+                              bool accumulate, int* gave_up, int* failed, cudaStream_t st) {
     const int mtiles = tcx_rows_pad(M) / TCX_M, ntiles = (N + NT - 1) / NT, tiles = mtiles * ntiles;
     const SlPlan plan = sl_plan(nkc, tiles);
     int2* part = (int2*)partial;
     jdft_status s;
-    if (NT == 32) s = sl_launch_nt<32, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, st);
-    else if (NT == 64) s = sl_launch_nt<64, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, st);
-    else s = sl_launch_nt<128, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, st);
+    if (NT == 32) s = sl_launch_nt<32, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, gave_up, st);
+    else if (NT == 64) s = sl_launch_nt<64, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, gave_up, st);
+    else s = sl_launch_nt<128, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, gave_up, st);
     if (s != JDFT_OK) return s;
     {
         Trace tr_("sl_reduce", st);
         const dim3 grid(std::min(NT, N), tiles);
         if (plan.first[SL_GROUPS] > 24)
             sl_reduce_kernel<8><<<grid, dim3(TCX_M, 8), 0, st>>>(part, plan, NT, mtiles, M, N, ra, rb, out, sm, sn,
-                                                                 scale, accumulate);
+                                                                 scale, accumulate, gave_up, failed);
         else
             sl_reduce_kernel<1><<<grid, dim3(TCX_M, 1), 0, st>>>(part, plan, NT, mtiles, M, N, ra, rb, out, sm, sn,
-                                                                 scale, accumulate);
+                                                                 scale, accumulate, gave_up, failed);
     }
     return check_launch("sl_reduce");
 }
@@ -684,8 +692,9 @@ jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const do
     const bool same = twin && NT == TCX_M;  // one set of slices
     const int rpA = tcx_rows_pad(M), rpB = (N + NT - 1) / NT * NT;
     const int tiles = rpA / TCX_M * ((N + NT - 1) / NT);
-    // places of the rows' largest values, exponents of the rows, of the scaled rows, the gain, the shifts
-    const int rows = M + N, words = 2 * rows + (twin ? 0 : 2 * rows + 1);
+    // places of the rows' largest values, exponents of the rows, of the scaled rows, whether a block gave up, the
+    // gain, the shifts
+    const int rows = M + N, words = 2 * rows + (twin ? 0 : 2 * rows + 1) + 1;
     const size_t head = sl_align(((size_t)words + (twin ? 0 : K)) * sizeof(int));
     auto bytes = [&](int k) {
         return head + sl_block_bytes(rpA, k) + (same ? 0 : sl_block_bytes(rpB, k)) +
@@ -699,7 +708,7 @@ jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const do
     jdft_status s;
     unsigned long long* at = twin ? nullptr : (unsigned long long*)ws;
     int* ex = (int*)ws + (twin ? 0 : 2 * rows);
-    int *scaled = ex + rows, *near = scaled + rows, *shift = near + 1;
+    int *scaled = ex + rows, *gave_up = scaled + rows, *near = gave_up + 1, *shift = near + 1;
     const SlScale none{nullptr, nullptr}, sc = twin ? none : SlScale{shift, near};
     const SlRows ra{ex, twin ? nullptr : scaled, sc, -1};
     const SlRows rb = twin ? ra : SlRows{ex + M, scaled + M, sc, +1};
@@ -721,7 +730,8 @@ jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const do
         }
         if ((s = sl_slice(A + k0, lda, M, TCX_M, k, false, ra, As, st))) return s;
         if (!same && (s = sl_slice(B + k0, ldb, N, NT, k, false, rb, Bs, st))) return s;
-        if ((s = sl_product<true>(As, Bs, M, N, NT, tcx_chunks(k), ra, rb, part, out, ldo, 1, scale, true, st)))
+        if ((s = sl_product<true>(As, Bs, M, N, NT, tcx_chunks(k), ra, rb, part, out, ldo, 1, scale, true, gave_up,
+                                   scratch.failed, st)))
             return s;
     }
     return JDFT_OK;
@@ -739,7 +749,7 @@ jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const do
     const int NT = sl_nt(N);
     const int rpB = (N + NT - 1) / NT * NT;
     const int nkc = tcx_chunks(K);
-    const size_t head = sl_align((size_t)(M + N + K) * sizeof(int));  // exponents
+    const size_t head = sl_align((size_t)(M + N + K + 1) * sizeof(int));  // exponents, and whether a block gave up
     auto bytes = [&](int m) {
         const int rpA = tcx_rows_pad(m), tiles = rpA / TCX_M * (rpB / NT);
         return head + sl_block_bytes(rpA, K) + sl_block_bytes(rpB, K) +
@@ -753,7 +763,8 @@ jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const do
     if (!ws) return JDFT_ERR_UNSUPPORTED;
     const ScratchUse use{scratch, st};
     jdft_status s;
-    int* shift = (int*)ws;
+    int* gave_up = (int*)ws;
+    int* shift = gave_up + 1;
     int* exB = shift + K;
     int* exA = exB + N;
     char* Bs = (char*)ws + head;
@@ -770,7 +781,8 @@ jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const do
         if (m0) JDFT_CUDA_TRY(cudaMemsetAsync(exA, 0, (size_t)m * sizeof(int), st));
         if ((s = sl_exponents_t(A + m0, lda, m, K, shift, -1, exA, st))) return s;
         if ((s = sl_slice(A + m0, lda, m, TCX_M, K, true, ra, As, st))) return s;
-        if ((s = sl_product<false>(As, Bs, m, N, NT, nkc, ra, rb, part, out + m0, 1, ldo, 1.0, accumulate, st)))
+        if ((s = sl_product<false>(As, Bs, m, N, NT, nkc, ra, rb, part, out + m0, 1, ldo, 1.0, accumulate, gave_up,
+                                    scratch.failed, st)))
             return s;
     }
     return JDFT_OK;
