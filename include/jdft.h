@@ -35,7 +35,10 @@
  *   - A basis handle owns device copies of its maps, potential and
  *     projectors, and a workspace that grows on demand (growth calls
  *     cudaMalloc, which synchronises the device).  Large FP64 products (on the
- *     tensor cores, see jdft_subspace) have scratch of their own that grows so.  One basis must not be used
+ *     tensor cores, see jdft_subspace) have scratch of their own that grows so,
+ *     to 1 GB at most for jdft_subspace and 1 GB for the other calls, and is kept
+ *     until the basis is destroyed (with it the block it last outgrew, and those
+ *     that a captured graph may use).  One basis must not be used
  *     from two host threads at once.
  *   - On any status other than JDFT_OK, jdft_last_error() returns a message
  *     (thread-local, valid until the next call on that thread).

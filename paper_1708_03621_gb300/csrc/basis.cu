@@ -65,7 +65,11 @@ void* ProductScratch::get(size_t need, cudaStream_t st) {
         cudaGetLastError();
         return nullptr;
     }
-    if (cap != cudaStreamCaptureStatusNone) return !ordered && bytes >= need ? ptr : nullptr;
+    if (cap != cudaStreamCaptureStatusNone) {
+        if (ordered || bytes < need) return nullptr;
+        in_graph = true;
+        return ptr;
+    }
     if (ordered) {
         if (!done && cudaEventCreateWithFlags(&done, cudaEventDisableTiming) != cudaSuccess) {
             cudaGetLastError();
@@ -75,16 +79,24 @@ void* ProductScratch::get(size_t need, cudaStream_t st) {
         if (bytes >= need) return cudaStreamWaitEvent(st, done, 0) == cudaSuccess ? ptr : nullptr;
     }
     if (bytes >= need) return ptr;
+    if (need > kMost) return nullptr;
+    // the block outgrown now goes with the next growth: freeing it here would wait for the work on it
+    cudaFree(spare);
+    spare = nullptr;
+    if (ptr && in_graph) retired.push_back(ptr);
+    else spare = ptr;
+    const size_t more = std::min(kMost, std::max(need, bytes + bytes / 2));
+    ptr = nullptr;
+    bytes = 0;
+    in_graph = false;
     // half again, so that the blocks outgrown stay few; the plain size where that much is not left
-    for (const size_t want : {std::max(need, bytes + bytes / 2), need}) {
-        void* p = nullptr;
-        if (cudaMalloc(&p, want) == cudaSuccess) {
-            if (ptr) retired.push_back(ptr);
-            ptr = p;
+    for (const size_t want : {more, need}) {
+        if (cudaMalloc(&ptr, want) == cudaSuccess) {
             bytes = want;
             return ptr;
         }
         cudaGetLastError();
+        ptr = nullptr;
     }
     return nullptr;
 }
@@ -95,10 +107,11 @@ void ProductScratch::finish(cudaStream_t st) {
 
 void ProductScratch::release() {
     cudaFree(ptr);
+    cudaFree(spare);
     for (void* p : retired) cudaFree(p);
     if (done) cudaEventDestroy(done);
     retired.clear();
-    ptr = nullptr;
+    ptr = spare = nullptr;
     done = nullptr;
     bytes = 0;
 }

@@ -129,16 +129,18 @@ struct Workspace {
     size_t bytes = 0;
 };
 
-// Scratch of the sliced FP64 products.  It grows by at least half again and keeps the
-// blocks it has outgrown until the basis goes (their sizes add up to less than
-// twice the last one), so that a captured graph that holds a pointer to one
-// stays valid.
+// Scratch of the sliced FP64 products, kMost bytes at most.  It grows by at least half
+// again, and keeps the block it last outgrew, and until the basis goes those that a captured
+// graph may hold a pointer to (their sizes add up to less than twice the last one).
 // ordered: for calls that nothing else keeps apart.  A product then waits on the device
 // for the one before it, on whatever stream that ran, and no graph takes a pointer.
 struct ProductScratch {
+    static constexpr size_t kMost = size_t(1) << 30;
     bool ordered = false;
+    bool in_graph = false;  // a graph was captured with ptr
     void* ptr = nullptr;
     size_t bytes = 0;
+    void* spare = nullptr;
     std::vector<void*> retired;
     cudaEvent_t done = nullptr;
     int* failed = nullptr;  // device word (or null) that a product whose waits ran out sets to JDFT_ERR_TIMEOUT

@@ -301,11 +301,11 @@ __device__ __forceinline__ void sl_commit(uint32_t bar) {
 }
 
 // CONJ: Re = Ar.Br + Ai.Bi, Im = Ar.Bi - Ai.Br (conj(A) B); else Re = Ar.Br - Ai.Bi, Im = Ar.Bi + Ai.Br.
-// part: [tile][unit][column][row] of (Re, Im) integers, S_D + 2^7 S_(D-1).
+// part: [tile - tile0][unit][column][row] of (Re, Im) integers, S_D + 2^7 S_(D-1).
 template <int NT, bool CONJ>
 __global__ void __launch_bounds__(SL_THREADS, 1)
     sl_mma_kernel(const char* __restrict__ As, const char* __restrict__ Bs, int nrbA, int nrbB, int nkc, int mtiles,
-                  SlPlan plan, int2* __restrict__ part, int* __restrict__ gave_up) {
+                  int tile0, SlPlan plan, int2* __restrict__ part, int* __restrict__ gave_up) {
     using L = SlLayout<NT>;
     extern __shared__ unsigned char smem_raw[];
     unsigned char* smem = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
@@ -321,7 +321,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1)
     while (g + 1 < SL_GROUPS && unit >= plan.first[g + 1]) ++g;
     const int D = sl_top(g), steps = D - 1;
     const int c0 = (unit - plan.first[g]) * plan.per[g], c1 = min(nkc, c0 + plan.per[g]);
-    const int mt = tile % mtiles, nt = tile / mtiles;
+    const int mt = (tile0 + tile) % mtiles, nt = (tile0 + tile) / mtiles;
     const int runs = (steps + SL_RUN - 1) / SL_RUN;  // stages per chunk
     const int total = (c1 - c0) * runs;              // at least one: the plan has no empty units
     if (tid == 0) {
@@ -497,14 +497,14 @@ __device__ __forceinline__ double sl_to_double(__int128 t, int q) {
 // *failed (or null) then says as well.
 template <int RZ>
 __global__ void __launch_bounds__(TCX_M* RZ)
-    sl_reduce_kernel(const int2* __restrict__ part, SlPlan plan, int NT, int mtiles, int M, int N,
+    sl_reduce_kernel(const int2* __restrict__ part, SlPlan plan, int NT, int mtiles, int tile0, int M, int N,
                      SlRows ra, SlRows rb, double2* __restrict__ out, size_t sm,
                      size_t sn, double scale, int accumulate, const int* __restrict__ gave_up,
                      int* __restrict__ failed) {
     __shared__ longlong2 sum[RZ > 1 ? RZ : 1][2][RZ > 1 ? TCX_M : 1];
     const int r = threadIdx.x, q = threadIdx.y;
     const int col = blockIdx.x, tile = blockIdx.y;
-    const int m = (tile % mtiles) * TCX_M + r, n = (tile / mtiles) * NT + col;
+    const int m = ((tile0 + tile) % mtiles) * TCX_M + r, n = ((tile0 + tile) / mtiles) * NT + col;
     if (n >= N) return;  // the whole block
     const int units = plan.first[SL_GROUPS];
     const size_t ustride = (size_t)NT * TCX_M;
@@ -587,9 +587,20 @@ static size_t sl_block_bytes(int rows_pad, int K) {
     return sl_align((size_t)rows_pad * tcx_chunks(K) * TCX_KC * SL_PLANES * 2);
 }
 
-// Scratch budget of a product: larger ones run in panels (of K for conj(A) B, of
-// output rows for A B).
-constexpr size_t SL_BUDGET = size_t(1) << 30;
+// Scratch of a product is at most SL_BUDGET (the largest that ProductScratch grows to of
+// itself): larger ones run in panels, of K for conj(A) B and of output rows and columns for
+// A B, and in groups of output tiles.
+constexpr size_t SL_BUDGET = ProductScratch::kMost;
+// Partial sums of `group` tiles.
+static size_t sl_partial_bytes(int nkc, int group, int NT) {
+    return sl_align((size_t)group * sl_units_max(nkc, group) * NT * TCX_M * sizeof(int2));
+}
+// The largest group of `tiles` whose partial sums fit, by halving (0: none).
+static int sl_group(int nkc, int tiles, int NT, size_t room) {
+    int g = tiles;
+    while (g > 1 && sl_partial_bytes(nkc, g, NT) > room) g = (g + 1) / 2;
+    return sl_partial_bytes(nkc, g, NT) <= room ? g : 0;
+}
 
 // Whether the slices are the faster way: estimated times of both (microseconds).
 // Slices: 54 for the launches, reading both operands twice and writing their padded
@@ -608,42 +619,50 @@ bool sl_eligible(int M, int N, int K) {
 }
 
 template <int NT, bool CONJ>
-static jdft_status sl_launch_nt(const void* As, const void* Bs, int nrbA, int nrbB, int nkc, int mtiles, int tiles,
-                                const SlPlan& plan, int2* part, int* gave_up, cudaStream_t st) {
+static jdft_status sl_launch_nt(const void* As, const void* Bs, int nrbA, int nrbB, int nkc, int mtiles, int tile0,
+                                int tiles, const SlPlan& plan, int2* part, int* gave_up, cudaStream_t st) {
     auto kern = sl_mma_kernel<NT, CONJ>;
     cudaError_t e = set_smem_attr((const void*)kern, SlLayout<NT>::SMEM);
     if (e != cudaSuccess) return set_error(JDFT_ERR_CUDA, std::string("sl_mma: ") + cudaGetErrorString(e));
     {
         Trace tr_("sl_mma", st);
         kern<<<dim3(plan.first[SL_GROUPS], tiles), SL_THREADS, SlLayout<NT>::SMEM, st>>>(
-            (const char*)As, (const char*)Bs, nrbA, nrbB, nkc, mtiles, plan, part, gave_up);
+            (const char*)As, (const char*)Bs, nrbA, nrbB, nkc, mtiles, tile0, plan, part, gave_up);
     }
     return check_launch("sl_mma");
 }
 
+// `group` output tiles at a time, as many as the partial sums have room for.
 template <bool CONJ>
-static jdft_status sl_product(const void* As, const void* Bs, int M, int N, int NT, int nkc, const SlRows& ra,
+static jdft_status sl_product(const void* As, const void* Bs, int M, int N, int NT, int nkc, int group, const SlRows& ra,
                               const SlRows& rb, void* partial, double2* out, size_t sm, size_t sn, double scale,
                               bool accumulate, int* gave_up, int* failed, cudaStream_t st) {
-    const int mtiles = tcx_rows_pad(M) / TCX_M, ntiles = (N + NT - 1) / NT, tiles = mtiles * ntiles;
-    const SlPlan plan = sl_plan(nkc, tiles);
+    const int mtiles = tcx_rows_pad(M) / TCX_M, ntiles = (N + NT - 1) / NT, all = mtiles * ntiles;
     int2* part = (int2*)partial;
-    jdft_status s;
-    if (NT == 32) s = sl_launch_nt<32, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, gave_up, st);
-    else if (NT == 64) s = sl_launch_nt<64, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, gave_up, st);
-    else s = sl_launch_nt<128, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, tiles, plan, part, gave_up, st);
-    if (s != JDFT_OK) return s;
-    {
-        Trace tr_("sl_reduce", st);
-        const dim3 grid(std::min(NT, N), tiles);
-        if (plan.first[SL_GROUPS] > 24)
-            sl_reduce_kernel<8><<<grid, dim3(TCX_M, 8), 0, st>>>(part, plan, NT, mtiles, M, N, ra, rb, out, sm, sn,
-                                                                 scale, accumulate, gave_up, failed);
+    for (int t0 = 0; t0 < all; t0 += group) {
+        const int tiles = std::min(group, all - t0);
+        const SlPlan plan = sl_plan(nkc, group);
+        jdft_status s;
+        if (NT == 32)
+            s = sl_launch_nt<32, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, t0, tiles, plan, part, gave_up, st);
+        else if (NT == 64)
+            s = sl_launch_nt<64, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, t0, tiles, plan, part, gave_up, st);
         else
-            sl_reduce_kernel<1><<<grid, dim3(TCX_M, 1), 0, st>>>(part, plan, NT, mtiles, M, N, ra, rb, out, sm, sn,
-                                                                 scale, accumulate, gave_up, failed);
+            s = sl_launch_nt<128, CONJ>(As, Bs, mtiles, ntiles, nkc, mtiles, t0, tiles, plan, part, gave_up, st);
+        if (s != JDFT_OK) return s;
+        {
+            Trace tr_("sl_reduce", st);
+            const dim3 grid(std::min(NT, N), tiles);
+            if (plan.first[SL_GROUPS] > 24)
+                sl_reduce_kernel<8><<<grid, dim3(TCX_M, 8), 0, st>>>(part, plan, NT, mtiles, t0, M, N, ra, rb, out, sm,
+                                                                     sn, scale, accumulate, gave_up, failed);
+            else
+                sl_reduce_kernel<1><<<grid, dim3(TCX_M, 1), 0, st>>>(part, plan, NT, mtiles, t0, M, N, ra, rb, out, sm,
+                                                                     sn, scale, accumulate, gave_up, failed);
+        }
+        if ((s = check_launch("sl_reduce"))) return s;
     }
-    return check_launch("sl_reduce");
+    return JDFT_OK;
 }
 
 // Exponents of an operand's rows (K values a row) into ex, zeroed before; `finite` and sc as in the kernel.
@@ -696,13 +715,18 @@ jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const do
     // gain, the shifts
     const int rows = M + N, words = 2 * rows + (twin ? 0 : 2 * rows + 1) + 1;
     const size_t head = sl_align(((size_t)words + (twin ? 0 : K)) * sizeof(int));
-    auto bytes = [&](int k) {
-        return head + sl_block_bytes(rpA, k) + (same ? 0 : sl_block_bytes(rpB, k)) +
-               sl_align((size_t)tiles * sl_units_max(tcx_chunks(k), tiles) * NT * TCX_M * sizeof(int2));
-    };
-    int kp = K;
-    while (kp > 2048 && bytes(kp) > SL_BUDGET) kp = (kp / 2 + TCX_KC - 1) / TCX_KC * TCX_KC;
-    void* ws = scratch.get(std::max(bytes(kp), K % kp ? bytes(K % kp) : 0), st);
+    auto slices = [&](int k) { return head + sl_block_bytes(rpA, k) + (same ? 0 : sl_block_bytes(rpB, k)); };
+    // K panels of which the slices take at most three quarters of the budget, tiles for the rest
+    int kp = K, group = 0;
+    for (;; kp = (kp / 2 + TCX_KC - 1) / TCX_KC * TCX_KC) {
+        const size_t b = slices(kp);
+        group = b < SL_BUDGET ? sl_group(tcx_chunks(kp), tiles, NT, SL_BUDGET - b) : 0;
+        if (group == tiles || (group && b <= SL_BUDGET / 4 * 3) || kp <= 256) break;
+    }
+    // (a last panel of fewer chunks may cut them finer)
+    auto bytes = [&](int k) { return k ? slices(k) + sl_partial_bytes(tcx_chunks(k), group, NT) : 0; };
+    while (group > 1 && bytes(K % kp) > SL_BUDGET) group = (group + 1) / 2;
+    void* ws = group ? scratch.get(std::max(bytes(kp), bytes(K % kp)), st) : nullptr;
     if (!ws) return JDFT_ERR_UNSUPPORTED;
     const ScratchUse use{scratch, st};
     jdft_status s;
@@ -730,8 +754,8 @@ jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const do
         }
         if ((s = sl_slice(A + k0, lda, M, TCX_M, k, false, ra, As, st))) return s;
         if (!same && (s = sl_slice(B + k0, ldb, N, NT, k, false, rb, Bs, st))) return s;
-        if ((s = sl_product<true>(As, Bs, M, N, NT, tcx_chunks(k), ra, rb, part, out, ldo, 1, scale, true, gave_up,
-                                   scratch.failed, st)))
+        if ((s = sl_product<true>(As, Bs, M, N, NT, tcx_chunks(k), group, ra, rb, part, out, ldo, 1, scale, true,
+                                   gave_up, scratch.failed, st)))
             return s;
     }
     return JDFT_OK;
@@ -747,19 +771,27 @@ jdft_status sl_zgemm_cn(int M, int N, int K, const double2* A, int lda, const do
 jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const double2* Bm, int ldb, double2* out,
                         int ldo, bool accumulate, ProductScratch& scratch, cudaStream_t st) {
     const int NT = sl_nt(N);
-    const int rpB = (N + NT - 1) / NT * NT;
     const int nkc = tcx_chunks(K);
     const size_t head = sl_align((size_t)(M + N + K + 1) * sizeof(int));  // exponents, and whether a block gave up
-    auto bytes = [&](int m) {
-        const int rpA = tcx_rows_pad(m), tiles = rpA / TCX_M * (rpB / NT);
-        return head + sl_block_bytes(rpA, K) + sl_block_bytes(rpB, K) +
-               sl_align((size_t)tiles * sl_units_max(nkc, tiles) * NT * TCX_M * sizeof(int2));
+    auto slices = [&](int m, int n) {
+        return head + sl_block_bytes(tcx_rows_pad(m), K) + sl_block_bytes((n + NT - 1) / NT * NT, K);
     };
-    int mp = M;
-    while (mp > 4096 && bytes(mp) > SL_BUDGET) mp = (mp / 2 + TCX_M - 1) / TCX_M * TCX_M;
-    // smaller panels cut K finer: the last panel may need as much as a full one
-    const int last = M % mp;
-    void* ws = scratch.get(std::max(bytes(mp), last ? bytes(last) : 0), st);
+    auto tiles_of = [&](int m, int n) { return tcx_rows_pad(m) / TCX_M * ((n + NT - 1) / NT); };
+    // panels of rows (and, where one row block beside B's slices is too much, of columns) of which the slices take
+    // at most three quarters of the budget, tiles for the rest
+    int mp = M, np = N, group = 0;
+    for (;;) {
+        const size_t b = slices(mp, np);
+        const int tiles = tiles_of(mp, np);
+        group = b < SL_BUDGET ? sl_group(nkc, tiles, NT, SL_BUDGET - b) : 0;
+        if (group == tiles || (group && b <= SL_BUDGET / 4 * 3)) break;
+        if (mp > 4096 || (mp > TCX_M && np <= NT)) mp = (mp / 2 + TCX_M - 1) / TCX_M * TCX_M;
+        else if (np > NT) np = (np / 2 + NT - 1) / NT * NT;
+        else break;
+    }
+    if (!group) return JDFT_ERR_UNSUPPORTED;
+    // (a smaller last panel has no more tiles, and its partial sums are laid out by the same plan)
+    void* ws = scratch.get(slices(mp, np) + sl_partial_bytes(nkc, group, NT), st);
     if (!ws) return JDFT_ERR_UNSUPPORTED;
     const ScratchUse use{scratch, st};
     jdft_status s;
@@ -767,23 +799,26 @@ jdft_status sl_zgemm_nn(int M, int N, int K, const double2* A, int lda, const do
     int* shift = gave_up + 1;
     int* exB = shift + K;
     int* exA = exB + N;
-    char* Bs = (char*)ws + head;
-    char* As = Bs + sl_block_bytes(rpB, K);
+    char* As = (char*)ws + head;
+    char* Bs = As + sl_block_bytes(tcx_rows_pad(mp), K);
+    char* part = Bs + sl_block_bytes((np + NT - 1) / NT * NT, K);
     JDFT_CUDA_TRY(cudaMemsetAsync(ws, 0, head, st));
     const SlScale none{nullptr, nullptr}, sc{shift, nullptr};
-    const SlRows ra{exA, nullptr, sc, -1}, rb{exB, nullptr, sc, +1};
     if ((s = sl_exponents(A, lda, K, nullptr, 0, 0, M, none, shift, st, true))) return s;
     if ((s = sl_exponents_t(Bm, ldb, N, K, shift, +1, exB, st))) return s;
-    if ((s = sl_slice(Bm, ldb, N, NT, K, true, rb, Bs, st))) return s;
-    for (int m0 = 0; m0 < M; m0 += mp) {
-        const int m = std::min(mp, M - m0);
-        char* part = As + sl_block_bytes(tcx_rows_pad(m), K);
-        if (m0) JDFT_CUDA_TRY(cudaMemsetAsync(exA, 0, (size_t)m * sizeof(int), st));
-        if ((s = sl_exponents_t(A + m0, lda, m, K, shift, -1, exA, st))) return s;
-        if ((s = sl_slice(A + m0, lda, m, TCX_M, K, true, ra, As, st))) return s;
-        if ((s = sl_product<false>(As, Bs, m, N, NT, nkc, ra, rb, part, out + m0, 1, ldo, 1.0, accumulate, gave_up,
-                                    scratch.failed, st)))
-            return s;
+    if ((s = sl_exponents_t(A, lda, M, K, shift, -1, exA, st))) return s;
+    for (int n0 = 0; n0 < N; n0 += np) {
+        const int n = std::min(np, N - n0);
+        const SlRows rb{exB + n0, nullptr, sc, +1};
+        if ((s = sl_slice(Bm + n0, ldb, n, NT, K, true, rb, Bs, st))) return s;
+        for (int m0 = 0; m0 < M; m0 += mp) {
+            const int m = std::min(mp, M - m0);
+            const SlRows ra{exA + m0, nullptr, sc, -1};
+            if ((mp < M || n0 == 0) && (s = sl_slice(A + m0, lda, m, TCX_M, K, true, ra, As, st))) return s;
+            if ((s = sl_product<false>(As, Bs, m, n, NT, nkc, group, ra, rb, part, out + (size_t)n0 * ldo + m0, 1, ldo,
+                                       1.0, accumulate, gave_up, scratch.failed, st)))
+                return s;
+        }
     }
     return JDFT_OK;
 }
