@@ -9,6 +9,7 @@
 #include <map>
 #include <mutex>
 
+#include "alloc_pair.h"
 #include "chain.cuh"
 #include "common.cuh"
 #include "gemm.cuh"
@@ -485,14 +486,14 @@ jdft_status jdft_basis_info(jdft_basis_t b, int ik, double* omega, int64_t* nbox
 jdft_status jdft_set_potential(jdft_basis_t b, const double* V, void* stream) {
     clear_error();
     JDFT_CHECK_ARG(b && V, "null argument");
-    if (!b->V) {
-        JDFT_CUDA_TRY(cudaMalloc(&b->V, b->N * sizeof(double)));
-        JDFT_CUDA_TRY(cudaMalloc(&b->V32, b->N * sizeof(float)));
-    }
-    if (!b->Vn && lines_serve(b)) {
-        JDFT_CUDA_TRY(cudaMalloc(&b->Vn, b->N * sizeof(double)));
-        JDFT_CUDA_TRY(cudaMalloc(&b->Vn32, b->N * sizeof(float)));
-    }
+    const size_t n64 = b->N * sizeof(double), n32 = b->N * sizeof(float);
+    cudaError_t e = cudaSuccess;
+    auto alloc = [&](void** p, size_t n) { return (e = cudaMalloc(p, n)) == cudaSuccess; };
+    if (!alloc_pair((void**)&b->V, n64, (void**)&b->V32, n32, alloc, cudaFree))
+        return set_error(e == cudaErrorMemoryAllocation ? JDFT_ERR_OOM : JDFT_ERR_CUDA,
+                         std::string("potential: ") + cudaGetErrorString(e));
+    // where these do not fit, H C takes the kernels that do without them (use_lines)
+    if (lines_serve(b) && !alloc_pair((void**)&b->Vn, n64, (void**)&b->Vn32, n32, alloc, cudaFree)) cudaGetLastError();
     {
         Trace tr_("permute_potential", (cudaStream_t)stream);
         permute_potential<<<grid_for(b->N, 256), 256, 0, (cudaStream_t)stream>>>(V, b->V, b->V32, b->Vn, b->Vn32, b->S[0],
