@@ -308,18 +308,13 @@ __global__ void jacobi_eig_kernel(int n, int m, double2* Ag, int sweeps, double*
     int* pp = idx + m;                                   // m/2 pair indices
     int* qq = pp + m / 2;
     for (int i = threadIdx.x; i < m; i += blockDim.x) idx[i] = i;
-    __shared__ double limit;
     __shared__ int turned;
     __syncthreads();
     for (int sw = 0; sw < sweeps; ++sw) {
-        // a sweep whose rotations were all below 2^-60 of the largest diagonal entry ends the iteration:
-        // what is left changes no eigenvalue by more than that
-        if (threadIdx.x == 0) {
-            double big = 0.0;
-            for (int i = 0; i < n; ++i) big = fmax(big, fabs(A[i * m + i].x));
-            limit = big * 8.673617379884035e-19;
-            turned = 0;
-        }
+        // a sweep in which every entry was below 2^-60 of both its diagonal entries ends the iteration: what is
+        // left changes no eigenvalue by more than that of itself (of the largest entry would do for the
+        // largest: small blocks beside it came out after a single sweep)
+        if (threadIdx.x == 0) turned = 0;
         __syncthreads();
         for (int step = 0; step < m - 1; ++step) {
             for (int k = threadIdx.x; k < m / 2; k += blockDim.x) {
@@ -337,7 +332,7 @@ __global__ void jacobi_eig_kernel(int n, int m, double2* Ag, int sweeps, double*
                         const double t = (th >= 0.0 ? 1.0 : -1.0) / (fabs(th) + sqrt(th * th + 1.0));
                         c = 1.0 / sqrt(t * t + 1.0);
                         s = t * c;
-                        if (!(ac <= limit)) turned = 1;
+                        if (!(ac <= 8.673617379884035e-19 * fmin(fabs(A[p * m + p].x), fabs(A[q * m + q].x)))) turned = 1;
                     }
                 }
                 cs[k] = c; sn[k] = s; ph[k] = e;
