@@ -2,6 +2,7 @@
 #pragma once
 
 #include "field_fast.cuh"
+#include "running_sum.h"
 
 namespace jdft {
 
@@ -23,12 +24,12 @@ __device__ __forceinline__ double block_total(double x) {
 // partial[NOUT * block + k]; the last block to arrive adds them, each thread its
 // share of the blocks in order, then the threads in order (deterministic), and
 // resets the counter for the next launch.
-template <int NOUT, int THREADS, typename T>
-__device__ __forceinline__ void finish_sum(const T* x, const BlockSum& b, double scale) {
+template <int NOUT, int THREADS>
+__device__ __forceinline__ void finish_sum(const double* x, const BlockSum& b, double scale) {
     __shared__ bool last;
 #pragma unroll
     for (int k = 0; k < NOUT; ++k) {
-        const double s = block_total<THREADS>((double)x[k]);
+        const double s = block_total<THREADS>(x[k]);
         if (threadIdx.x == 0) b.partial[NOUT * blockIdx.x + k] = s;
     }
     if (threadIdx.x == 0) {

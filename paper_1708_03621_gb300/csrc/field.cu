@@ -867,7 +867,8 @@ pcm_init_kernel(const double2* __restrict__ rho, c_t<T>* __restrict__ x, c_t<T>*
 // division that finds (m0, m1) is per row, and the grid is small (update_grid): a
 // block's sums cost 3000 FP64 additions, which were half of the kernel's time with
 // a thousand blocks.  Four boxes are read and two written, which bounds the rest
-// (128^3, FP32: 37 -> 31 us).
+// (128^3, FP32: 37 -> 31 us).  A thread then sums some twenty values, in FP32 with their
+// rounding errors (the time is the same).
 template <typename T>
 __global__ void __launch_bounds__(kFieldThreads)
 pcm_update_kernel(c_t<T>* __restrict__ x, c_t<T>* __restrict__ r, const c_t<T>* __restrict__ d,
@@ -876,7 +877,7 @@ pcm_update_kernel(c_t<T>* __restrict__ x, c_t<T>* __restrict__ r, const c_t<T>* 
     const T alpha = (T)(*rz / *dHd);
     const int rows = q.S[0] * q.S[1], S2 = q.S[2];
     const int lane = threadIdx.x & 31, warps = gridDim.x * (kFieldThreads / 32);
-    T s[2] = {0, 0};
+    RunningSum<T> rr, rz_new;
     for (int row = blockIdx.x * (kFieldThreads / 32) + (threadIdx.x >> 5); row < rows; row += warps) {
         const int m0 = row / q.S[1], m1 = row - m0 * q.S[1];
         const T f0 = (T)fold(m0, q.S[0]), f1 = (T)fold(m1, q.S[1]);
@@ -897,10 +898,11 @@ pcm_update_kernel(c_t<T>* __restrict__ x, c_t<T>* __restrict__ r, const c_t<T>* 
             const T g2 = ax * ax + ay * ay + az * az;
             const T K = g2 > (T)0 ? (T)kFourPi / g2 : (T)0;
             const T a = rv.x * rv.x + rv.y * rv.y;
-            s[0] += a;
-            s[1] += K * a;
+            rr.add(a);
+            rz_new.add(K * a);
         }
     }
+    const double s[2] = {rr.total(), rz_new.total()};
     finish_sum<2, kFieldThreads>(s, sum, 1.0);
 }
 

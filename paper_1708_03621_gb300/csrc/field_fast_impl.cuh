@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(Line<T, N>::THREADS)
         }
         __syncwarp();
     }
-    T part = 0;
+    RunningSum<T> part;
     const T sc = (T)scale;
     if (act) {
 #pragma unroll
@@ -228,11 +228,12 @@ __global__ void __launch_bounds__(Line<T, N>::THREADS)
             out[a] = r;
             if (din) {
                 const c_t<T> d = din[a];
-                part += d.x * r.x + d.y * r.y;
+                part.add(d.x * r.x + d.y * r.y);
             }
         }
     }
-    if (din) finish_sum<1, L::THREADS>(&part, sum, 1.0);
+    const double total = part.total();
+    if (din) finish_sum<1, L::THREADS>(&total, sum, 1.0);
 }
 
 // ---- the Hartree chain on the half box -----------------------------------------
