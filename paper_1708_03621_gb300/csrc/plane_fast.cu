@@ -592,7 +592,9 @@ static size_t fast_smem(const ChainGeom& g, int nw = kFastWarps) {
 // some 50 spilled words); 128^3, 64 bands, 16 warps of 8-value lanes against 8 of
 // 16-value ones 5.34 -> 4.05 ms.  FP32 blocks alike: H C of 32 bands on 80^3 232 -> 180 us,
 // the 256 x 128 planes of the slab's 1024 bands 19.5 -> 16.7 ms with 16 warps on the one
-// block an SM holds.
+// block an SM holds.  FP64 blocks on 40, 48 and 80 planes have become faster still by line
+// transforms where the z edge is a compiled line length too (use_lines: 48^3 170 -> 133 us
+// a call); these kernels serve the other z edges and jdft_apply_H_noalloc.
 template <typename T, int N0, int N1>
 struct PlaneBlock {
     static constexpr int warps = kFastWarps, per_sm = 1;

@@ -13,13 +13,21 @@
 // Mukunoki et al., ISC 2020 (with FP16 tensor cores).  A product of digits is at
 // most 2^12 and FP32 sums of integers are exact up to 2^24, so a block sums
 // 2 (D - 1) K <= 4096 products (D = i + j) in tensor memory before the sum is
-// taken out as an integer.  What is dropped (digits below 2^-62 of a row's
-// largest value, pairs beyond 10) is below 2^-62 of the rows' largest products: over
-// the block shapes here the results are nearer to extended precision than the
-// FP64 sums they replace.
+// taken out as an integer.
 //
-// Launches: row maxima, slices (36 bytes a complex value) of both operands, the
-// products, and the sum of the blocks' integers (128 bits) into the FP64 output.
+// What is dropped: a row's largest component becomes an integer of 2^60 to 2^61 and all of
+// them are cut toward zero to integers, 2^-58 of the product of the two rows' largest at
+// worst for each real product; the digit pairs beyond 10 are up to 8 2^12 2^49 = 2^64 of
+// its 2^120 or more, 2^-56.  Both have either sign, and over the block shapes here the
+// results are nearer to extended precision than the FP64 sums they replace.  But the bound
+// is relative to the rows' maxima, not to the sum of the terms' absolute values as in FP64:
+// sl_zgemm_cn and sl_zgemm_nn scale the summed index where that would show.
+//
+// Launches: row exponents, slices (36 bytes a complex value) of both operands, the
+// products, and the sum of the blocks' integers (128 bits) into the FP64 output; for A B
+// the exponents of A's columns first, for conj(A) B of two operands a look at the columns
+// of the largest values (and a reading of both operands and two more launches, which return
+// at once in ordinary products).
 // A unit of work (block) is a 128 x NT output tile, a pair of digit sums (D, D - 1)
 // and a range of K: at step j it adds A_j B_(D-j) to the first and
 // A_(j-1) B_(D-j) to the second accumulator, so each slice is staged once for
@@ -27,7 +35,7 @@
 // Tensor memory holds 2 x 2 x NT columns.
 //
 // Measured (event times, against the CUDA-core products): overlap, subspace matrix
-// and rotation of 120 bands of 27 000 plane waves 19.86 -> 1.32 ms, error against
+// and rotation of 120 bands of 27 000 plane waves 19.86 -> 1.33 ms, error against
 // 64-bit references 6.7e-16 -> 5.9e-16 (the Cholesky factorisation between them
 // takes 0.35 ms); H C of 64 bands on a 128^3 box with 256 projectors 28.06 -> 7.64 ms
 // when they came in, their two launches of products 0.65 ms each then and 0.58 now.
@@ -603,12 +611,13 @@ static int sl_group(int nkc, int tiles, int NT, size_t room) {
 }
 
 // Whether the slices are the faster way: estimated times of both (microseconds).
-// Slices: 54 for the launches, reading both operands twice and writing their padded
-// slices at 3.5 TB/s, and per tile of 128 rows 3.6 ns a K and, for five blocks' start
+// Slices: 54 for the launches, reading both operands twice (three times for A of A B) and
+// writing their padded slices at 3.5 TB/s, and per tile of 128 rows 3.6 ns a K and, for five blocks' start
 // and end, 4 us on each of 152 SMs.  CUDA cores: 10 for the launch and 8 flops a padded
 // output and K at 1 TFLOP/s.  Measured (conj(A) B of 4 259 plane waves, CUDA cores /
-// slices): 32 x 32 50 / 67, 40 x 40 108 / 67; of 19 778: 16 x 16 53 / 154, 32 x 32
-// 165 / 160; H C with 128 projectors on 4 259: 16 bands 193 / 225, 32 bands 364 / 274.
+// slices, the mean of one and of two operands): 32 x 32 51 / 69, 40 x 40 109 / 69; of
+// 19 778: 16 x 16 52 / 152, 32 x 32 166 / 161; H C with 128 projectors on 4 259: 16 bands
+// 193 / 240, 32 bands 364 / 288.
 bool sl_eligible(int M, int N, int K) {
     const int NT = sl_nt(N), ntiles = (N + NT - 1) / NT;
     const double m = tcx_rows_pad(M), n = (double)ntiles * NT, k = K, tiles = m / TCX_M * ntiles;

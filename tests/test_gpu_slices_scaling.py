@@ -90,8 +90,9 @@ def test_subspace_of_oppositely_graded_blocks(nb, spread, norms):
     """C^dag H C where C falls by 10^spread over the plane waves (in random order) and H C rises by as much, bands of
     different norms among them: every term is of one size, far below the product of the rows' maxima.  With r the rows'
     largest components and a_k, b_k the columns' largest relative to them, the scaled rows stay below 2 sqrt(a_k b_k)
-    r each (halves and exponents rounded down); a component's two products lose 2^-60 of the scaled maxima for either
-    operand and 2^-58 in the digits left out: npw 2^-54 max(a_k b_k) r r', and the entry is rounded three times."""
+    r each (halves and exponents rounded down), and each real product loses 2^-58 of their maxima to the cut and 2^-56
+    in the digit pairs left out: npw 2^-53 max(a_k b_k) r r' for a component's two, of either sign.  Half of that is
+    asked for, and the entry is rounded three times."""
     jdft, b, npw = _basis()
     rng = np.random.default_rng(nb + spread + norms)
     x = _power(rng, spread, npw)[None, :]
