@@ -291,6 +291,27 @@ def kernel_work(p: Problem, name: str, launches: int, nb: int) -> tuple[float, f
         fl = 5 * ncols * S2 * l2(S2)
         by = (p.npw + S2 * ncols) * e + (p.npw * e if name == "zpass_forward" else 0)
         return fl * per_launch_bands, by * per_launch_bands
+    if name in ("line_z_inverse", "line_z_forward"):
+        return kernel_work(p, "zpass_" + name[7:], launches, nb)
+    if name in ("line_rows_inverse", "line_rows_forward"):
+        # sphere columns and rows, one read and the other written
+        fl = 5 * nrows * S2 * S1 * l2(S1)
+        return fl * per_launch_bands, (S2 * ncols + nrows * S1 * S2) * e * per_launch_bands
+    if name == "line_columns":
+        fl = 2 * 5 * S1 * S2 * S0 * l2(S0)
+        return fl * per_launch_bands, 2 * nrows * S1 * S2 * e * per_launch_bands + p.N * (8 if e == 16 else 4)
+    if name == "line_density":
+        fl = 5 * S1 * S2 * S0 * l2(S0)
+        return fl * per_launch_bands, nrows * S1 * S2 * e * per_launch_bands + p.N * 16
+    if name in ("sl_mma", "sl_slice"):
+        # the FP64 step's five products (those of zgemm_cn and zgemm_nn above) on slices of 36 bytes a complex
+        # value; C^dag C needs one operand's.  Averages over the launches, each of both operands for sl_slice.
+        cn, nn = [(p.nproj, p.nb), (p.nb, p.nb), (p.nb, 0)], [p.nproj, p.nb]
+        vals = sum((M + N) * p.npw for M, N in cn) + sum((p.npw + p.nb) * K for K in nn)
+        if name == "sl_slice":
+            return 0.0, (16.0 + 36.0) * vals / max(1, launches)
+        fl = 3 * kernel_work(p, "zgemm_cn", 3, nb)[0] + 2 * kernel_work(p, "zgemm_nn", 2, nb)[0]
+        return fl / max(1, launches), 36.0 * vals / max(1, launches)
     if name == "zgemm_cn":
         # per step: P^dag C (nproj x nb), C^dag HC and C^dag C (nb x nb), over npw (the orthonormaliser
         # reuses the subspace step's C^dag O C)
@@ -314,8 +335,9 @@ def roofline_of(k: dict, prec: str, peaks: dict, fp32: dict) -> dict:
     chains), or the nominal FP64 rate for FP64 blocks; tensor-core GEMMs: the
     measured BF16 burst (BF16x3 pieces), or TF32 = that x (1.1 / 2.25), the
     nominal TF32/BF16 ratio, against algorithmic 8MNK flops (the 3-term split
-    issues 3x that, so 1/3 is that kernel's ceiling); everything else: HBM
-    copy bandwidth.
+    issues 3x that, so 1/3 is that kernel's ceiling; the FP64 products from
+    slices 45x); everything else: HBM copy bandwidth.  FP64 transforms run in
+    64-bit integers, so their nominal flops can pass the FP64 pipe's rate.
     """
     name = k["name"]
     hbm = peaks.get("hbm_gbs", 6800.0)
@@ -329,7 +351,12 @@ def roofline_of(k: dict, prec: str, peaks: dict, fp32: dict) -> dict:
             peak, how = bf16 * 1.1 / 2.25, f"measured bf16 burst x nominal tf32/bf16 ratio 1.1/2.25 ({src})"
         return {"bound": "tensor", "achieved": k["achieved_tflops"], "peak": round(peak, 1), "unit": "TFLOP/s",
                 "frac": round((k["achieved_tflops"] or 0) / peak, 4), "split_passes": 3, "peak_source": how}
-    if name.startswith("plane_") or name.startswith("zgemm") or name.startswith("zpass"):
+    if name == "sl_mma":
+        bf16 = peaks.get("bf16_tflops", 1900.0)
+        return {"bound": "tensor", "achieved": k["achieved_tflops"], "peak": round(bf16, 1), "unit": "TFLOP/s",
+                "frac": round((k["achieved_tflops"] or 0) / bf16, 4), "split_passes": 45,
+                "peak_source": "measured bf16 burst (%s)" % ("of measured" if "bf16_tflops" in peaks else "of fallback")}
+    if name.startswith(("plane_", "zgemm", "zpass", "line_")):
         if prec == "fp64":
             alu, how = FP64_NOMINAL_TFLOPS, "FP64 nominal 1.25 TFLOP/s"
         else:
