@@ -163,7 +163,8 @@ __global__ void __launch_bounds__(256) sl_balance_kernel(const double2* __restri
                                                          int* __restrict__ near) {
     __shared__ int top[2][8][32];
     constexpr int kNone = -(1 << 24);
-    if (*(volatile const int*)near >= SL_NEAR) return;  // only rises: the same to whoever reads it later
+    // the word rises while blocks run: the block decides as one
+    if (__syncthreads_or(*(volatile const int*)near >= SL_NEAR)) return;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, k = blockIdx.x * 32 + lane;
     int m[2] = {kNone, kNone};
 #pragma unroll
