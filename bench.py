@@ -382,8 +382,8 @@ def roofline_of(k: dict, prec: str, peaks: dict, fp32: dict) -> dict:
 TRAFFIC_SOURCES = {"plane_apply_density_pair": ["csrc/plane_pair.cu", "csrc/fft_pair.cuh", "csrc/fft_reg.cuh",
                                                 "csrc/chain.cuh", "csrc/common.cuh", "csrc/tc_ptx.cuh"]}
 TRAFFIC_PER_BAND = {
-    # 150 439 680 + 86 020 608 bytes over 64 bands (ncu capture of one 64-band launch)
-    "plane_apply_density_pair": (3.6947e6, "8cb9836a2c6096cd"),
+    # 150 366 464 + 85 970 944 bytes over 64 bands (ncu capture of one 64-band launch)
+    "plane_apply_density_pair": (3.6928e6, "889ba492c2968694"),
 }
 
 
